@@ -132,7 +132,7 @@ METRIC = "MLUPS of the fused f+g step (FP32 plain)"
 # kernel sources it was taken on: any change to them makes it null.
 STEP_TRAFFIC = {"bytes_per_launch": (309391616 + 255389184 + 308886528 + 253282560) // 2,
                 "sources_sha256": "22adc04600794184e7f2dc0308ed44331d9bf8cfaa462689084fc037aff67e11"}
-STEP_SOURCES = ["lbm_step.cu", "lbm_device.cuh", "lbm_internal.h", "lbm_ptx.cuh"]
+STEP_SOURCES = ["lbm_march.cu", "lbm_march.cuh", "lbm_store.cuh", "lbm_device.cuh", "lbm_internal.h"]
 
 
 def step_traffic():
@@ -346,7 +346,7 @@ def batch_variant(lbm, torch, steps, ncases=256, seed=4):
     nodes = b.nodes
     out = {"cases": ncases, "nodes": nodes, "mlups": nodes / (ms_step * 1e-3) / 1e6, "ms_per_step": ms_step,
            "bytes_per_lu": b.bytes_per_step() / nodes,
-           "autotune": {"tile_shape": ["64x32", "32x16"][choice[0]], "order": lbm.Batch.ORDERS[choice[1]],
+           "autotune": {"work_split": ["even", "32 rows"][choice[0]], "order": lbm.Batch.ORDERS[choice[1]],
                         "ms_per_step_candidates": [round(float(x), 4) for x in ms]}}
     b.close()
     # the same cases, each on its own plain FP32 handle, stepped one after another

@@ -252,20 +252,17 @@ int lbm_synchronize(lbm_handle* h);
 /* Steps taken since init (or restored by lbm_load). */
 int64_t lbm_step_count(const lbm_handle* h);
 
-/* Default bound on each wait of the step kernel for a tile's copies: 2 s. */
+/* Default bound on a warp's wait for its first rows in the step kernel: 2 s. */
 #define LBM_TILE_WAIT_DEFAULT_NS 2000000000LL
 
-/* Bound, in nanoseconds, on each wait of the step kernel for the copies of
- * a tile into shared memory (failure detection; not a parameter of the
- * paper's method). A wait that runs out ends the launch early in every
- * block that met it, sets the handle's status, and the next synchronising
- * call returns LBM_ERR_TIMEOUT; the state is then undefined until the next
- * lbm_set_fields, lbm_set_populations or lbm_load. 0 means no waiting: a
- * tile whose copies have not landed when its turn comes times out, which a
- * step from a fresh state always meets (its first copies were issued just
- * before). The kernel never exits with a copy in flight: after a timeout it
- * still waits, within the default bound, for the copies it has issued.
- * ns < 0: LBM_ERR_ARG. Takes effect from the next lbm_step. */
+/* Bound, in nanoseconds, on the time a warp of the step kernel waits for the
+ * loads of its first rows (later rows load while earlier ones are computed;
+ * failure detection, not a parameter of the paper's method). A warp whose
+ * wait was longer stores nothing and sets the handle's status, and the next
+ * synchronising call returns LBM_ERR_TIMEOUT; the state is then undefined
+ * until the next lbm_set_fields, lbm_set_populations or lbm_load. 0 means no
+ * waiting, which every warp runs out of. ns < 0: LBM_ERR_ARG. Takes effect
+ * from the next lbm_step. */
 int lbm_set_tile_wait(lbm_handle* h, int64_t ns);
 
 /* Bytes of population traffic one time step moves at the algorithmic
@@ -276,9 +273,9 @@ int lbm_destroy(lbm_handle* h);
 
 /* ---- Batched cases -------------------------------------------------------
  * Many independent cases (each its own lattice size, temperature and
- * droplet) advanced together: one persistent launch per time step walks a
- * work list of (case, tile) items, with the cases' tensor maps and constants
- * in device tables. The rows are the same model as lbm_step; a case in a
+ * droplet) advanced together: one launch per time step walks work lists of
+ * (case, strip, rows) items, with the cases' layouts and constants in device
+ * tables. The rows are the same model as lbm_step; a case in a
  * batch gives the same populations as that case on its own handle with the
  * same precision, up to floating-point rounding (the two kernels are
  * compiled separately). With 16-bit storage the batch rounds its stores
@@ -302,7 +299,7 @@ int lbm_batch_moments(lbm_batch* b, int32_t i, double* rho, double* ux, double* 
 int lbm_batch_conservation(lbm_batch* b, int32_t i, double out[6]);
 int lbm_batch_get_populations(lbm_batch* b, int32_t i, double* f, double* g);
 /* Case i's conservation record as reduced inside the most recent step
- * (per-tile FP32 partial sums, summed per case in FP64): layout of
+ * (FP32 partial sums per work item, summed per case in FP64): layout of
  * lbm_step_stats out[0..6]; out[7] = the steps the batch has executed, as
  * counted on the device (the count that keys stochastic rounding).
  * Synchronous. */
@@ -310,18 +307,18 @@ int lbm_batch_step_stats(lbm_batch* b, int32_t i, double out[8]);
 /* Steps the batch has executed (host count; includes autotuner trials). */
 int64_t lbm_batch_step_count(const lbm_batch* b);
 /* As lbm_set_tile_wait, for the batch's step kernel: the bound on each wait
- * for an item's copies (0: no waiting); a wait that runs out is reported as
- * LBM_ERR_TIMEOUT by the next synchronising call, and the cases' states are
- * undefined until set again. ns < 0: LBM_ERR_ARG. */
+ * for the first rows of an item (0: no waiting); a wait that runs out is
+ * reported as LBM_ERR_TIMEOUT by the next synchronising call, and the cases'
+ * states are undefined until set again. ns < 0: LBM_ERR_ARG. */
 int lbm_batch_set_tile_wait(lbm_batch* b, int64_t ns);
-/* Autotuner: times every candidate (tile shape x work-list order) for
+/* Autotuner: times every candidate (work split x work-list order) for
  * trial_steps steps on the current state and keeps the fastest; the trial
  * steps are real steps of every case (the state advances). choice[0] =
- * tile shape index, choice[1] = order index (0 case-major, 1 largest case
+ * work split index (0 an equal run of rows per warp, 1 items of 32 rows), choice[1] = order index (0 case-major, 1 largest case
  * first, 2 round-robin over cases); ms[k] (may be NULL, >= 6 entries) =
  * the time per step of candidate k = 3 * shape + order. Synchronous. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, int32_t choice[2], double* ms);
-/* Select a candidate directly (tile shape, order). */
+/* Select a candidate directly (work split, order). */
 int lbm_batch_select(lbm_batch* b, int32_t shape, int32_t order);
 int lbm_batch_get_params(const lbm_batch* b, int32_t i, lbm_params* out);
 int lbm_batch_synchronize(lbm_batch* b);

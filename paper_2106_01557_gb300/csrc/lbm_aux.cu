@@ -24,7 +24,7 @@ constexpr int AUX_NT = 256;
 
 template <class S>
 __device__ __forceinline__ double load_d(const S* buf, const Geometry& G, int p, int x, int y, double rest) {
-    const S v = buf[(long long)p * G.plane + (long long)(y + 2) * G.pitch + G.PX + x];
+    const S v = buf[G.at(p, x, y)];
     if constexpr (sizeof(S) == 2) return rest + (double)Store<S, float>::ld(v, 0.0f);
     else return (double)v;
 }
@@ -38,7 +38,7 @@ __device__ __forceinline__ S to_store(double v, double rest) {
 // load_d / to_store in the compute type C (identical to them for C = double)
 template <class S, class C>
 __device__ __forceinline__ C load_c(const S* buf, const Geometry& G, int p, int x, int y, C rest) {
-    const S v = buf[(long long)p * G.plane + (long long)(y + 2) * G.pitch + G.PX + x];
+    const S v = buf[G.at(p, x, y)];
     if constexpr (sizeof(S) == 2) return rest + (C)Store<S, float>::ld(v, 0.0f);
     else return (C)v;
 }

@@ -116,22 +116,26 @@ __device__ __forceinline__ const KC<float>& kc<float>(const Launch& L) { return 
 template <>
 __device__ __forceinline__ const KC<double>& kc<double>(const Launch& L) { return L.kd; }
 
-// m = M l (SM Eq. S2)
+// m = M l (SM Eq. S2), 24 operations. The density m[0] = (((l1 + l3) +
+// (l2 + l4)) + ((l5 + l7) + (l6 + l8))) + l0 is a pairwise tree, so a
+// butterfly over lanes holding the nine populations gives it too, bit for
+// bit (the row-marching step forms the densities beside a warp's strip so).
 template <class C>
 __device__ __forceinline__ void moments9(const C l[9], C m[9]) {
-    const C ax = l[1] + l[2] + l[3] + l[4];
-    const C dg = l[5] + l[6] + l[7] + l[8];
-    m[0] = l[0] + ax + dg;
+    const C s13 = l[1] + l[3], s24 = l[2] + l[4], s57 = l[5] + l[7], s68 = l[6] + l[8];
+    const C ax = s13 + s24, dg = s57 + s68;
+    m[0] = (ax + dg) + l[0];
     m[1] = C(-4) * l[0] - ax + C(2) * dg;
     m[2] = C(4) * l[0] - C(2) * ax + dg;
-    const C dx = l[5] - l[6] - l[7] + l[8];
-    const C dy = l[5] + l[6] - l[7] - l[8];
-    m[3] = l[1] - l[3] + dx;
-    m[4] = C(-2) * (l[1] - l[3]) + dx;
-    m[5] = l[2] - l[4] + dy;
-    m[6] = C(-2) * (l[2] - l[4]) + dy;
-    m[7] = l[1] - l[2] + l[3] - l[4];
-    m[8] = l[5] - l[6] + l[7] - l[8];
+    const C d57 = l[5] - l[7], d68 = l[6] - l[8];
+    const C dx = d57 - d68, dy = d57 + d68;
+    const C d13 = l[1] - l[3], d24 = l[2] - l[4];
+    m[3] = d13 + dx;
+    m[4] = C(-2) * d13 + dx;
+    m[5] = d24 + dy;
+    m[6] = C(-2) * d24 + dy;
+    m[7] = s13 - s24;
+    m[8] = s57 - s68;
 }
 
 // m0 / 9, the weight of moment 0 in every population. Each column of M^-1
@@ -164,26 +168,28 @@ __device__ __forceinline__ void rest_as_complement(C m0, C l[9]) {
     if constexpr (sizeof(C) == 4) l[0] = m0 - (((l[1] + l[2]) + (l[3] + l[4])) + ((l[5] + l[6]) + (l[7] + l[8])));
 }
 
-// l = M^-1 m = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4) m
+// l = M^-1 m = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4) m,
+// the weights folded into fused multiply-adds (28 operations)
 template <class C>
 __device__ __forceinline__ void populations9(const C m[9], C l[9]) {
-    const C a0 = ninth(m[0]), a1 = m[1] * C(1.0 / 36.0), a2 = m[2] * C(1.0 / 36.0);
-    const C a3 = m[3] * C(1.0 / 6.0), a4 = m[4] * C(1.0 / 12.0);
-    const C a5 = m[5] * C(1.0 / 6.0), a6 = m[6] * C(1.0 / 12.0);
-    const C a7 = m[7] * C(0.25), a8 = m[8] * C(0.25);
-    l[0] = a0 - C(4) * a1 + C(4) * a2;
-    const C axis = a0 - a1 - C(2) * a2;
-    const C px = a3 - C(2) * a4, py = a5 - C(2) * a6;
-    l[1] = axis + px + a7;
-    l[2] = axis + py - a7;
-    l[3] = axis - px + a7;
-    l[4] = axis - py - a7;
-    const C diag = a0 + C(2) * a1 + a2;
-    const C qx = a3 + a4, qy = a5 + a6;
-    l[5] = diag + qx + qy + a8;
-    l[6] = diag - qx + qy - a8;
-    l[7] = diag - qx - qy + a8;
-    l[8] = diag + qx - qy - a8;
+    const C a0 = ninth(m[0]);
+    const C axis = a0 - m[1] * C(1.0 / 36.0) - m[2] * C(1.0 / 18.0);
+    const C diag = a0 + m[1] * C(1.0 / 18.0) + m[2] * C(1.0 / 36.0);
+    l[0] = a0 - m[1] * C(1.0 / 9.0) + m[2] * C(1.0 / 9.0);
+    const C bx = m[3] * C(1.0 / 6.0), by = m[5] * C(1.0 / 6.0);
+    const C px = bx - m[4] * C(1.0 / 6.0), py = by - m[6] * C(1.0 / 6.0);
+    const C qx = bx + m[4] * C(1.0 / 12.0), qy = by + m[6] * C(1.0 / 12.0);
+    const C ap = axis + m[7] * C(0.25), am = axis - m[7] * C(0.25);
+    l[1] = ap + px;
+    l[3] = ap - px;
+    l[2] = am + py;
+    l[4] = am - py;
+    const C dp = diag + m[8] * C(0.25), dm = diag - m[8] * C(0.25);
+    const C qs = qx + qy, qd = qx - qy;
+    l[5] = dp + qs;
+    l[7] = dp - qs;
+    l[8] = dm + qd;
+    l[6] = dm - qd;
 }
 
 // Per-node macroscopic state (Eq. 13, 14) from the pulled populations and
@@ -200,20 +206,21 @@ struct NodeMacro {
     C m[9], n[9];
 };
 
-// SH: f and g hold deviations from the rest populations; their moments get
-// the rest moments added back (moments 0-2, the others vanish).
-template <bool SH = false, class C, class K>
-__device__ __forceinline__ void node_macro(const K& k, const C f[9], const C g[9], const C rn[9],
-                                           NodeMacro<C>& s) {
-    moments9(f, s.m);
-    moments9(g, s.n);
+// Moments of pulled populations; SH: they hold deviations from the rest
+// populations, whose moments 0-2 (the others vanish) are added back.
+template <bool SH, class C, class R>
+__device__ __forceinline__ void moments_of(const C l[9], const R* rest, C m[9]) {
+    moments9(l, m);
     if constexpr (SH) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            s.m[q] += k.mrest[q];
-            s.n[q] += k.nrest[q];
-        }
+        for (int q = 0; q < 3; ++q) m[q] += rest[q];
     }
+}
+
+// The macroscopic state from the moments s.m and s.n and the density around
+// the node.
+template <class C, class K>
+__device__ __forceinline__ void macro_of(const K& k, const C rn[9], NodeMacro<C>& s) {
     const C rho = rn[0];
     // Eq. 13 weights: 1/3 on the axes, 1/12 on the diagonals
     const C third = C(1.0 / 3.0), twelfth = C(1.0 / 12.0);
@@ -231,6 +238,15 @@ __device__ __forceinline__ void node_macro(const K& k, const C f[9], const C g[9
     s.rek = s.n[0] + k.half_dt * s.q;
     const C ke = C(0.5) * k.c2 * (s.uhx * s.uhx + s.uhy * s.uhy);
     s.T = (s.rek * s.inv_rho - ke) * k.inv_cv;
+}
+
+// SH: f and g hold deviations from the rest populations.
+template <bool SH = false, class C, class K>
+__device__ __forceinline__ void node_macro(const K& k, const C f[9], const C g[9], const C rn[9],
+                                           NodeMacro<C>& s) {
+    moments_of<SH>(f, k.mrest, s.m);
+    moments_of<SH>(g, k.nrest, s.n);
+    macro_of(k, rn, s);
 }
 
 // p_BE = p_EOS + a rho^2 with Eq. 17
@@ -415,13 +431,12 @@ __device__ __forceinline__ void g_rest_wall(const KC<C>& k, C rho_w, C T_w, C& g
     g_diag = a0 + C(2) * a1 + a2;
 }
 
-// Store one post-collision value at physical (x, y) of plane p, with the
+// Store one post-collision value at physical (x, y) of population p, with the
 // copies the periodic ghost cells need. y may be -1 or ny for a wall ghost,
 // and, with open left and right sides, x may be -1 or nx. XOPEN = false:
 // the caller knows that x is periodic.
 template <class S, bool XOPEN = true>
 __device__ __forceinline__ void put(S* __restrict__ out, const Geometry& G, int p, int x, int y, S v) {
-    S* base = out + (long long)p * G.plane;
     int rows[2];
     int nr = 1;
     rows[0] = y;
@@ -432,11 +447,10 @@ __device__ __forceinline__ void put(S* __restrict__ out, const Geometry& G, int 
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         if (r >= nr) break;
-        S* row = base + (long long)(rows[r] + 2) * G.pitch + G.PX;
-        row[x] = v;
+        out[G.at(p, x, rows[r])] = v;
         if (!(XOPEN && (G.open & 12))) {
-            if (x < GHOST_COLS) row[x + G.nx] = v;
-            if (x >= G.nx - GHOST_COLS) row[x - G.nx] = v;
+            if (x < GHOST_COLS) out[G.at(p, x + G.nx, rows[r])] = v;
+            if (x >= G.nx - GHOST_COLS) out[G.at(p, x - G.nx, rows[r])] = v;
         }
     }
 }

@@ -1,8 +1,7 @@
 // Host runtime of liblbm: configuration checks, parameter derivation
-// (Eq. 16-19 and the Maxwell coexistence of Eq. 17), device buffers and
-// TMA descriptors, the step loop (CUDA graphs of step pairs), and the C ABI
+// (Eq. 16-19 and the Maxwell coexistence of Eq. 17), device buffers, the
+// batch's work lists, the step loop (CUDA graphs of 20 steps), and the C ABI
 // declared in include/lbm.h.
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -158,24 +157,6 @@ int storage_of(int precision) {
 
 size_t elem_size(int storage) { return storage == S_F64 ? 8 : (storage == S_F32 ? 4 : 2); }
 
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiled get_encoder() {
-    static EncodeTiled fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiled>(p);
-    });
-    return fn;
-}
-
 }  // namespace
 
 struct lbm_handle {
@@ -186,9 +167,9 @@ struct lbm_handle {
     size_t esize;
     void* buf[2] = {nullptr, nullptr};
     int cur = 0;  // index of the buffer holding the current state
-    CUtensorMap tmf[2], tmg[2];
-    double* partials = nullptr;  // step_blocks x NQ
-    double* stats = nullptr;     // NQ (step) + NQ (moments)
+    double* partials = nullptr;  // 2 (by the buffer a step reads) x blocks x NQ
+    size_t part_stride = 0;      // doubles between the two
+    double* stats = nullptr;     // NQ (step) + NQ (moments) + the step count as of buffer 0 and of buffer 1
     unsigned* counter = nullptr; // 2 counters
     int* status = nullptr;
     double* scratch = nullptr;   // 9 * 2 * n doubles (populations / fields)
@@ -197,7 +178,10 @@ struct lbm_handle {
     bool own_stream = false;
     cudaGraphExec_t graph = nullptr;  // GRAPH_STEPS steps starting from buffer 0
     int64_t steps = 0;
+    MarchGrid grid;        // of the row-marching step
+    bool pending = false;  // the last step's record is not combined yet
     static constexpr int GRAPH_STEPS = 20;  // even: the graph returns to buffer 0
+    double* count(int b) const { return stats + 2 * NQ + b; }
 };
 
 extern "C" {
@@ -233,6 +217,16 @@ void lbm_default_config(lbm_config* c, int32_t nx, int32_t ny) {
     c->stream = nullptr;
     c->device = 0;
     c->rounding = 1;
+}
+
+// every constant in both lanes of a pair (the structures hold nothing else)
+static KC<float2> pair_constants(const KC<float>& k) {
+    static_assert(sizeof(KC<float2>) == 2 * sizeof(KC<float>), "plain arrays of constants");
+    KC<float2> p;
+    const float* a = reinterpret_cast<const float*>(&k);
+    float2* b = reinterpret_cast<float2*>(&p);
+    for (size_t i = 0; i < sizeof k / sizeof(float); ++i) b[i] = make_float2(a[i], a[i]);
+    return p;
 }
 
 static int derive(const lbm_config& c, lbm_params& p, Launch& L) {
@@ -317,19 +311,13 @@ static int derive(const lbm_config& c, lbm_params& p, Launch& L) {
 
     Geometry& G = L.geo;
     const int storage = storage_of(c.precision);
-    int bx, by, hx;
-    step_tile(storage, &bx, &by, &hx);
     G.nx = c.nx;
     G.ny = c.ny;
     G.walls = c.walls;
-    G.HX = hx;
-    const int line = 128 / (int)elem_size(storage);  // elements per 128 bytes
-    G.PX = line;
-    int pitch = G.PX + (c.nx > bx ? c.nx : bx) + hx;
-    pitch = ((pitch + line - 1) / line) * line;
-    G.pitch = pitch;
-    G.nyp = c.ny + 4 > by + 4 ? c.ny + 4 : by + 4;
-    G.plane = (long long)G.pitch * G.nyp;
+    const int sw = march_strip(storage);
+    G.lsw = sw == 64 ? 6 : 5;
+    G.nyp = c.ny + 4;
+    G.strips = (c.nx + sw - 1) / sw + 2;
     G.hot_x0 = ((c.hot_x0 % c.nx) + c.nx) % c.nx;
     G.hot_len = c.hot_len;
     G.open = c.open_sides;
@@ -380,6 +368,9 @@ static int derive(const lbm_config& c, lbm_params& p, Launch& L) {
         k.c4g1_Cref = cast((4.0 + c.gamma1) * p.Cref);
         k.c4g2_Cref = cast((4.0 - c.gamma2) * p.Cref);
         k.c2_third = cast(p.c * p.c / 3.0);
+        k.rec_rho = cast(p.a - 5.0 * p.kappa / 3.0);
+        k.rec_ax = cast(p.kappa / 3.0);
+        k.rec_dg = cast(p.kappa / 12.0);
         k.T_bottom = cast(c.Tr_bottom > 0 ? c.Tr_bottom * p.Tc : 0.0);
         k.T_top = cast(c.Tr_top > 0 ? c.Tr_top * p.Tc : 0.0);
         k.T_hot = cast(c.Tr_hot > 0 ? c.Tr_hot * p.Tc : 0.0);
@@ -441,40 +432,7 @@ static int derive(const lbm_config& c, lbm_params& p, Launch& L) {
             L.kd.nrest[q] = mg[q];
         }
     }
-    return LBM_OK;
-}
-
-static int make_maps(lbm_handle* h) {
-    EncodeTiled enc = get_encoder();
-    if (!enc) return fail(LBM_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-    const Geometry& G = h->L.geo;
-    int bx, by, hx;
-    step_tile(h->storage, &bx, &by, &hx);
-    CUtensorMapDataType dt = h->storage == S_F64   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
-                             : h->storage == S_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                             : h->storage == S_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                   : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    // map x = 0 is the first ghost column (row element PX - HX, 16-byte aligned);
-    // the map ends after the right ghost block, so that a box reaching into
-    // the row padding reads the out-of-bounds fill instead of memory
-    const int x0 = G.PX - G.HX;
-    cuuint64_t dims[3] = {(cuuint64_t)((G.nx > bx ? G.nx : bx) + 2 * G.HX), (cuuint64_t)G.nyp, 18};
-    cuuint64_t strides[2] = {(cuuint64_t)G.pitch * h->esize, (cuuint64_t)G.plane * h->esize};
-    cuuint32_t estr[3] = {1, 1, 1};
-    cuuint32_t boxf[3] = {(cuuint32_t)(bx + 2 * hx), (cuuint32_t)(by + 4), 9};
-    cuuint32_t boxg[3] = {(cuuint32_t)(bx + 2 * hx), (cuuint32_t)(by + 2), 9};
-    for (int b = 0; b < 2; ++b) {
-        void* base = static_cast<unsigned char*>(h->buf[b]) + (size_t)x0 * h->esize;
-        CUresult r1 = enc(&h->tmf[b], dt, 3, base, dims, strides, boxf, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        CUresult r2 = enc(&h->tmg[b], dt, 3, base, dims, strides, boxg, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS)
-            return fail(LBM_ERR_CUDA, "cuTensorMapEncodeTiled failed (code " + std::to_string((int)r1) + "/" +
-                                          std::to_string((int)r2) + ")");
-    }
+    L.kp = pair_constants(L.kf);
     return LBM_OK;
 }
 
@@ -514,13 +472,15 @@ int lbm_init(const lbm_config* cfg, lbm_handle** out) {
         h->own_stream = true;
     }
     const Geometry& G = h->L.geo;
-    const size_t bytes = (size_t)18 * G.plane * h->esize;
+    const size_t bytes = (size_t)G.elems() * h->esize;
     const size_t n = (size_t)G.nx * G.ny;
-    const int nb = std::max(step_blocks(h->storage, G), moments_blocks(G));
+    h->grid = march_grid(h->storage, G);
+    const int nb = std::max(moments_blocks(G), h->grid.groups * h->grid.chunks);
+    h->part_stride = (size_t)nb * NQ;
     h->scratch_elems = 18 * n;
     bool ok = cudaMalloc(&h->buf[0], bytes) == cudaSuccess && cudaMalloc(&h->buf[1], bytes) == cudaSuccess &&
-              cudaMalloc(&h->partials, (size_t)nb * NQ * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&h->stats, 2 * NQ * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&h->partials, 2 * h->part_stride * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&h->stats, (2 * NQ + 2) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&h->counter, 2 * sizeof(unsigned)) == cudaSuccess &&
               cudaMalloc(&h->status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&h->scratch, h->scratch_elems * sizeof(double)) == cudaSuccess;
@@ -532,15 +492,12 @@ int lbm_init(const lbm_config* cfg, lbm_handle** out) {
     }
     ok = cudaMemsetAsync(h->buf[0], 0, bytes, h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->buf[1], 0, bytes, h->stream) == cudaSuccess &&
-         cudaMemsetAsync(h->stats, 0, 2 * NQ * sizeof(double), h->stream) == cudaSuccess &&
+         cudaMemsetAsync(h->stats, 0, (2 * NQ + 2) * sizeof(double), h->stream) == cudaSuccess &&
+         cudaMemsetAsync(h->partials, 0, 2 * h->part_stride * sizeof(double), h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->counter, 0, 2 * sizeof(unsigned), h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) == cudaSuccess &&
          cudaStreamSynchronize(h->stream) == cudaSuccess;
     if (!ok) { release(h); delete h; return fail(LBM_ERR_CUDA, "device initialisation failed"); }
-    rc = make_maps(h);
-    if (rc) { release(h); delete h; return rc; }
-    e = prepare_step(h->storage);
-    if (e != cudaSuccess) { release(h); delete h; return cuda_fail(e, "cudaFuncSetAttribute"); }
     *out = h;
     return LBM_OK;
 }
@@ -639,6 +596,15 @@ int lbm_synchronize(lbm_handle* h) {
     return check_status(h);
 }
 
+// A new state goes into buffer 0: the step count follows it.
+static cudaError_t restart(lbm_handle* h) {
+    cudaError_t e = cudaSuccess;
+    if (h->cur == 1)
+        e = cudaMemcpyAsync(h->count(0), h->count(1), sizeof(double), cudaMemcpyDeviceToDevice, h->stream);
+    h->cur = 0;
+    return e;
+}
+
 // Copy n doubles of a caller field into the scratch area (device), or
 // use the caller's device pointer directly.
 static const double* stage_in(lbm_handle* h, const double* src, size_t off, size_t n, int on_device,
@@ -662,12 +628,12 @@ int lbm_set_fields(lbm_handle* h, const double* rho, const double* ux, const dou
     }
     // The scatter writes every stored entry that a pull reads (including
     // ghost copies); clear first so the unread corners are defined too.
-    const size_t bytes = (size_t)18 * h->L.geo.plane * h->esize;
+    const size_t bytes = (size_t)h->L.geo.elems() * h->esize;
     CK(cudaMemsetAsync(h->buf[0], 0, bytes, h->stream));
     // per-node arithmetic in the storage's compute type: FP64 for FP64
     // storage, FP32 otherwise (the stored values are FP32 or narrower)
     CK(launch_init(h->storage, h->L, d[0], d[1], d[2], d[3], h->buf[0], h->stream, h->storage != S_F64));
-    h->cur = 0;
+    CK(restart(h));
     return check_status(h);
 }
 
@@ -676,10 +642,10 @@ int lbm_set_populations(lbm_handle* h, const double* f, const double* g) {
     const size_t n = (size_t)h->cfg.nx * h->cfg.ny;
     CK(cudaMemcpyAsync(h->scratch, f, 9 * n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->scratch + 9 * n, g, 9 * n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    const size_t bytes = (size_t)18 * h->L.geo.plane * h->esize;
+    const size_t bytes = (size_t)h->L.geo.elems() * h->esize;
     CK(cudaMemsetAsync(h->buf[0], 0, bytes, h->stream));
     CK(launch_set_pops(h->storage, h->L, h->scratch, h->scratch + 9 * n, h->buf[0], h->stream));
-    h->cur = 0;
+    CK(restart(h));
     return check_status(h);
 }
 
@@ -692,7 +658,10 @@ int lbm_get_populations(lbm_handle* h, double* f, double* g) {
     return check_status(h);
 }
 
-static cudaError_t step_once(lbm_handle* h, int from) {
+// One step from buffer `from`. last: no step follows it in this call, so the
+// step combines its own record; otherwise the next step does. first: the
+// record of the step before is combined already.
+static cudaError_t step_once(lbm_handle* h, int from, bool first, bool last) {
     const double* phi = nullptr;
     if (h->L.cubic) {
         // rho u^3 of the entering state, for the cubic-term source
@@ -701,15 +670,18 @@ static cudaError_t step_once(lbm_handle* h, int from) {
         if (e != cudaSuccess) return e;
         phi = h->scratch + n;
     }
-    return launch_step(h->storage, h->L, &h->tmf[from], &h->tmg[from], h->buf[1 - from], h->partials, h->stats,
-                       h->counter, h->status, h->stream, phi);
+    MarchGrid mg = h->grid;
+    mg.combine_prev = first ? 0 : 1;
+    mg.combine_here = last ? 1 : 0;
+    return launch_march(h->storage, h->L, h->buf[from], h->buf[1 - from], mg, h->partials + from * h->part_stride, h->partials + (1 - from) * h->part_stride, h->stats,
+                        h->count(from), h->count(1 - from), h->counter, h->status, h->stream, phi);
 }
 
 static int build_graph(lbm_handle* h) {
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < lbm_handle::GRAPH_STEPS && e == cudaSuccess; ++k) e = step_once(h, k & 1);
+    for (int k = 0; k < lbm_handle::GRAPH_STEPS && e == cudaSuccess; ++k) e = step_once(h, k & 1, false, false);
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) return cuda_fail(e, "step launch during capture");
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
@@ -730,13 +702,20 @@ int lbm_step(lbm_handle* h, int n) {
             }
             CK(cudaGraphLaunch(h->graph, h->stream));
             h->steps += lbm_handle::GRAPH_STEPS;
+            h->pending = true;
             n -= lbm_handle::GRAPH_STEPS;
             continue;
         }
-        CK(step_once(h, h->cur));
+        CK(step_once(h, h->cur, !h->pending, n == 1));
+        h->pending = n > 1;
         h->cur = 1 - h->cur;
         h->steps += 1;
         n -= 1;
+    }
+    if (h->pending) {
+        // the call ended with a graph: the record of its last step (from buffer 1)
+        CK(launch_record_finish(h->partials + h->part_stride, h->grid.groups * h->grid.chunks, h->stats, h->stream));
+        h->pending = false;
     }
     return LBM_OK;
 }
@@ -771,7 +750,8 @@ int lbm_conservation(lbm_handle* h, double out[6]) {
 int lbm_step_stats(lbm_handle* h, double out[8]) {
     if (!h || !out) return fail(LBM_ERR_ARG, "null argument");
     double s[NQ];
-    CK(cudaMemcpyAsync(s, h->stats, NQ * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(s, h->stats, (NQ - 1) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(s + 7, h->count(h->cur), sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     int rc = check_status(h);
     for (int k = 0; k < 8; ++k) out[k] = s[k];
     return rc;
@@ -799,7 +779,8 @@ double lbm_bytes_per_step(const lbm_handle* h) {
 }
 
 // Checkpoint layout: magic, nx, ny, precision, walls, a hash of the whole
-// configuration, steps, then the raw stored buffer (18 ghost-padded planes).
+// configuration, steps, then the stored state as 18 ghost-padded planes (f_0 ..
+// f_8, g_0 .. g_8) of nyp lines each.
 static const uint64_t CK_MAGIC = 0x4c424d4c56434b32ull;  // "LBMLVCK2"
 
 // FNV-1a (Fowler, Noll, Vo) over every field of the configuration that
@@ -825,13 +806,47 @@ static uint64_t config_hash(const lbm_config& c) {
     return h;
 }
 
+// The file holds the state as 18 planes (f_0 .. f_8, g_0 .. g_8) of node rows
+// -2 .. ny + 1 (and on to `nyp` rows), each row from 128 bytes before its
+// column 0 to a whole number of 128 bytes that takes the 16 bytes of ghost
+// columns beyond the last.
+struct FilePlanes {
+    size_t px, pitch, nyp, plane;
+    explicit FilePlanes(const lbm_handle* h) {
+        const size_t line = 128 / h->esize;
+        const int min_x = h->storage == S_F64 ? 32 : 64, min_y = h->storage == S_F64 || h->storage == S_F32 ? 16 : 32;
+        px = line;
+        pitch = (px + std::max(h->cfg.nx, min_x) + 16 / h->esize + line - 1) / line * line;
+        nyp = std::max(h->cfg.ny, min_y) + 4;
+        plane = pitch * nyp;
+    }
+};
+// stored strips <-> the file's planes, both on the host: the rows and columns
+// that a step reads
+static void copy_planes(const lbm_handle* h, unsigned char* file, unsigned char* state, bool save) {
+    const Geometry& G = h->L.geo;
+    const FilePlanes F(h);
+    const size_t es = h->esize;
+    const int sw = 1 << G.lsw;
+    for (int p = 0; p < 18; ++p)
+        for (int y = -2; y < G.ny + 2; ++y)
+            for (int x = -GHOST_COLS; x < G.nx + GHOST_COLS;) {
+                const int n = std::min(sw - ((x + sw) & (sw - 1)), G.nx + GHOST_COLS - x);  // up to the strip's end
+                unsigned char* a = file + (p * F.plane + (size_t)(y + 2) * F.pitch + F.px + x) * es;
+                unsigned char* b = state + (size_t)G.at(p, x, y) * es;
+                std::memcpy(save ? a : b, save ? b : a, n * es);
+                x += n;
+            }
+}
+
 int lbm_save(lbm_handle* h, const char* path) {
     if (!h || !path) return fail(LBM_ERR_ARG, "null argument");
     int rc = check_status(h);
     if (rc) return rc;
-    const size_t bytes = (size_t)18 * h->L.geo.plane * h->esize;
-    std::vector<unsigned char> host(bytes);
-    CK(cudaMemcpy(host.data(), h->buf[h->cur], bytes, cudaMemcpyDeviceToHost));
+    const size_t bytes = 18 * FilePlanes(h).plane * h->esize;
+    std::vector<unsigned char> host(bytes), state((size_t)h->L.geo.elems() * h->esize);
+    CK(cudaMemcpy(state.data(), h->buf[h->cur], state.size(), cudaMemcpyDeviceToHost));
+    copy_planes(h, host.data(), state.data(), true);
     FILE* fp = std::fopen(path, "wb");
     if (!fp) return fail(LBM_ERR_IO, std::string("cannot open ") + path);
     int32_t hdr[4] = {h->cfg.nx, h->cfg.ny, h->cfg.precision, h->cfg.walls};
@@ -850,8 +865,8 @@ int lbm_load(lbm_handle* h, const char* path) {
     uint64_t magic = 0, ch = 0;
     int32_t hdr[4];
     int64_t steps = 0;
-    const size_t bytes = (size_t)18 * h->L.geo.plane * h->esize;
-    std::vector<unsigned char> host(bytes);
+    const size_t bytes = 18 * FilePlanes(h).plane * h->esize;
+    std::vector<unsigned char> host(bytes), state((size_t)h->L.geo.elems() * h->esize);
     bool ok = std::fread(&magic, 8, 1, fp) == 1 && std::fread(hdr, sizeof hdr, 1, fp) == 1 &&
               std::fread(&ch, 8, 1, fp) == 1 && std::fread(&steps, 8, 1, fp) == 1;
     if (ok && (magic != CK_MAGIC || hdr[0] != h->cfg.nx || hdr[1] != h->cfg.ny || hdr[2] != h->cfg.precision ||
@@ -868,12 +883,13 @@ int lbm_load(lbm_handle* h, const char* path) {
     std::fclose(fp);
     if (!ok) return fail(LBM_ERR_IO, std::string("read failed: ") + path);
     CK(cudaStreamSynchronize(h->stream));
-    CK(cudaMemcpy(h->buf[0], host.data(), bytes, cudaMemcpyHostToDevice));
+    copy_planes(h, host.data(), state.data(), false);
+    CK(cudaMemcpy(h->buf[0], state.data(), state.size(), cudaMemcpyHostToDevice));
     // the device copy of the step count keys the stochastic rounding of
     // 16-bit storage: a resumed run continues with the same dither
     const double st = (double)steps;
-    CK(cudaMemcpy(h->stats + 7, &st, sizeof st, cudaMemcpyHostToDevice));
     h->cur = 0;
+    CK(cudaMemcpy(h->count(0), &st, sizeof st, cudaMemcpyHostToDevice));
     h->steps = steps;
     return LBM_OK;
 }
@@ -901,16 +917,15 @@ struct lbm_batch {
     long long arena_elems = 0;
     void* arena[2] = {nullptr, nullptr};
     int cur = 0;
-    BatchCase* d_cases[2] = {nullptr, nullptr};  // per tile shape (ntx differs)
-    KC<float>* d_kcs = nullptr;
-    CUtensorMap* d_maps[2] = {nullptr, nullptr};
+    BatchCase* d_cases = nullptr;
     BatchItem* d_items = nullptr;
-    int max_items = 0;
-    std::vector<BatchItem> items[2][3];  // [shape][order]
+    int* d_first = nullptr;
+    int max_items = 0, warps = 0;
+    std::vector<BatchItem> items[2][3];  // [shape][order], the warps' lists one after another
+    std::vector<int> first[2][3];        // where each warp's list begins (and where the last ends)
     float* d_partials = nullptr;
     int* d_status = nullptr;
-    double* d_steps = nullptr;   // step count (device copy, keys stochastic rounding)
-    unsigned* d_done = nullptr;  // finished blocks of the current launch
+    double* d_steps = nullptr;   // step count as of arena 0 and of arena 1 (keys stochastic rounding)
     double* d_rec = nullptr;     // 8 (case record) + 8 (conservation)
     double* scratch = nullptr;   // 18 x largest case
     double* aux_partials = nullptr;
@@ -929,14 +944,12 @@ static BatchLaunch batch_launch(lbm_batch* b) {
     BatchLaunch B;
     B.items = b->d_items;
     B.nitems = (int)b->items[b->shape][b->order].size();
-    B.cases = b->d_cases[b->shape];
-    B.kcs = b->d_kcs;
-    B.maps = b->d_maps[b->shape];
+    B.first = b->d_first;
+    B.warps = b->warps;
+    B.cases = b->d_cases;
     B.partials = b->d_partials;
     B.status = b->d_status;
-    B.sms = b->sms;
     B.steps = b->d_steps;
-    B.done = b->d_done;
     B.rounding = b->cfg[0].rounding;
     B.tile_wait_ns = b->tile_wait_ns;
     return B;
@@ -944,9 +957,8 @@ static BatchLaunch batch_launch(lbm_batch* b) {
 
 static void batch_release(lbm_batch* b) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
-    void* ptrs[] = {b->arena[0], b->arena[1], b->d_cases[0], b->d_cases[1], b->d_kcs, b->d_maps[0], b->d_maps[1],
-                    b->d_items, b->d_partials, b->d_status, b->d_rec, b->scratch, b->aux_partials, b->aux_counter,
-                    b->d_steps, b->d_done};
+    void* ptrs[] = {b->arena[0], b->arena[1], b->d_cases, b->d_items, b->d_first, b->d_partials,
+                    b->d_status, b->d_rec, b->scratch, b->aux_partials, b->aux_counter, b->d_steps};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -954,7 +966,9 @@ static void batch_release(lbm_batch* b) {
 
 static int batch_upload_items(lbm_batch* b) {
     const std::vector<BatchItem>& v = b->items[b->shape][b->order];
+    const std::vector<int>& first = b->first[b->shape][b->order];
     CK(cudaMemcpyAsync(b->d_items, v.data(), v.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, b->stream));
+    CK(cudaMemcpyAsync(b->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
     CK(cudaStreamSynchronize(b->stream));
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
@@ -992,7 +1006,7 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
         int rc = derive(cfgs[i], b->prm[i], b->L[i]);
         if (rc) { delete b; return rc; }
         b->off[i] = total;
-        total += ((18 * b->L[i].geo.plane + 127) / 128) * 128;  // 256-byte aligned case starts
+        total += ((b->L[i].geo.elems() + 127) / 128) * 128;  // 256-byte aligned case starts
         max_n = std::max(max_n, (size_t)cfgs[i].nx * cfgs[i].ny);
     }
     b->arena_elems = total;
@@ -1008,48 +1022,72 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
         if (e != cudaSuccess) { delete b; return cuda_fail(e, "cudaStreamCreate"); }
         b->own_stream = true;
     }
-    // work lists for both tile shapes and the three orders
+    // Work lists. Strips of all cases in one of three orders (case after
+    // case, the largest case first, or strip 0 of every case, then strip 1, ...),
+    // their rows dealt to the warps of one wave: shape 0, every warp an equal
+    // run of consecutive rows; shape 1, items of at most 32 rows in turn.
     std::vector<int> by_size(ncases);
     for (int i = 0; i < ncases; ++i) by_size[i] = i;
     std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int c) {
         return (long long)cfgs[a].nx * cfgs[a].ny > (long long)cfgs[c].nx * cfgs[c].ny;
     });
-    std::vector<BatchCase> hc[2];
-    for (int v = 0; v < 2; ++v) {
-        int bx, by;
-        batch_tile(b->storage, v, &bx, &by);
-        hc[v].resize(ncases);
-        std::vector<int> nt(ncases);
-        for (int i = 0; i < ncases; ++i) {
-            BatchCase& c = hc[v][i];
-            std::memset(&c, 0, sizeof c);
-            c.geo = b->L[i].geo;
-            c.off = b->off[i];
-            c.ntx = (cfgs[i].nx + bx - 1) / bx;
-            c.ntiles = c.ntx * ((cfgs[i].ny + by - 1) / by);
-            float rs = 0.f;
-            for (int q = 0; q < 9; ++q) rs += b->L[i].kf.rest[q];
-            c.rest_sum = rs;
-            nt[i] = c.ntiles;
+    const int sw = march_strip(b->storage);
+    std::vector<BatchItem> strips[3];  // whole strips
+    int max_strips = 0;
+    for (int i = 0; i < ncases; ++i) max_strips = std::max(max_strips, (cfgs[i].nx + sw - 1) / sw);
+    auto add = [&](int o, int i, int s) {
+        if (s * sw < cfgs[i].nx) strips[o].push_back({i, s * sw, 0, cfgs[i].ny});
+    };
+    for (int i = 0; i < ncases; ++i)
+        for (int s = 0; s < max_strips; ++s) add(0, i, s);
+    for (int i : by_size)
+        for (int s = 0; s < max_strips; ++s) add(1, i, s);
+    for (int s = 0; s < max_strips; ++s)
+        for (int i = 0; i < ncases; ++i) add(2, i, s);
+    long long rows = 0;
+    for (const BatchItem& t : strips[0]) rows += t.y1;
+    b->warps = (int)std::min<long long>(batch_warps(b->storage, b->sms), rows);
+    for (int o = 0; o < 3; ++o) {
+        std::vector<BatchItem>&even = b->items[0][o], &dealt = b->items[1][o];
+        std::vector<int>&fe = b->first[0][o], &fd = b->first[1][o];
+        long long at = 0;  // rows before strip t
+        int w = 0;
+        for (const BatchItem& t : strips[o]) {
+            for (int y = 0; y < t.y1;) {
+                while (rows * (w + 1) / b->warps <= at + y) ++w;  // the warp that row y falls to
+                const int e = (int)std::min<long long>(t.y1, rows * (w + 1) / b->warps - at);
+                while ((int)fe.size() <= w) fe.push_back((int)even.size());
+                even.push_back({t.c, t.xs, y, e});
+                y = e;
+            }
+            at += t.y1;
         }
-        for (int i = 0; i < ncases; ++i)
-            for (int t = 0; t < nt[i]; ++t) b->items[v][0].push_back({i, t});
-        for (int i : by_size)
-            for (int t = 0; t < nt[i]; ++t) b->items[v][1].push_back({i, t});
-        int maxt = *std::max_element(nt.begin(), nt.end());
-        for (int t = 0; t < maxt; ++t)
-            for (int i = 0; i < ncases; ++i)
-                if (t < nt[i]) b->items[v][2].push_back({i, t});
-        b->max_items = std::max(b->max_items, (int)b->items[v][0].size());
+        while ((int)fe.size() <= b->warps) fe.push_back((int)even.size());
+        std::vector<BatchItem> cut;
+        for (const BatchItem& t : strips[o]) {
+            const int n = (t.y1 + 31) / 32;
+            for (int j = 0; j < n; ++j) cut.push_back({t.c, t.xs, (int)((long long)t.y1 * j / n), (int)((long long)t.y1 * (j + 1) / n)});
+        }
+        for (int v = 0; v < b->warps; ++v) {
+            fd.push_back((int)dealt.size());
+            for (size_t j = v; j < cut.size(); j += b->warps) dealt.push_back(cut[j]);
+        }
+        fd.push_back((int)dealt.size());
+        b->max_items = std::max({b->max_items, (int)even.size(), (int)dealt.size()});
+    }
+    std::vector<BatchCase> hc(ncases);
+    for (int i = 0; i < ncases; ++i) {
+        std::memset(&hc[i], 0, sizeof hc[i]);
+        hc[i].geo = b->L[i].geo;
+        hc[i].off = b->off[i];
+        hc[i].kf = b->L[i].kf;
+        hc[i].kp = b->L[i].kp;
     }
     const size_t abytes = (size_t)total * b->esize;
     const size_t nb_aux = 4096;
     bool ok = cudaMalloc(&b->arena[0], abytes) == cudaSuccess && cudaMalloc(&b->arena[1], abytes) == cudaSuccess &&
-              cudaMalloc(&b->d_cases[0], ncases * sizeof(BatchCase)) == cudaSuccess &&
-              cudaMalloc(&b->d_cases[1], ncases * sizeof(BatchCase)) == cudaSuccess &&
-              cudaMalloc(&b->d_kcs, ncases * sizeof(KC<float>)) == cudaSuccess &&
-              cudaMalloc(&b->d_maps[0], (size_t)ncases * 4 * sizeof(CUtensorMap)) == cudaSuccess &&
-              cudaMalloc(&b->d_maps[1], (size_t)ncases * 4 * sizeof(CUtensorMap)) == cudaSuccess &&
+              cudaMalloc(&b->d_cases, ncases * sizeof(BatchCase)) == cudaSuccess &&
+              cudaMalloc(&b->d_first, ((size_t)b->warps + 1) * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&b->d_items, (size_t)b->max_items * sizeof(BatchItem)) == cudaSuccess &&
               cudaMalloc(&b->d_partials, (size_t)b->max_items * 8 * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&b->d_status, sizeof(int)) == cudaSuccess &&
@@ -1057,67 +1095,20 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
               cudaMalloc(&b->scratch, 18 * max_n * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&b->aux_partials, nb_aux * NQ * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&b->aux_counter, sizeof(unsigned)) == cudaSuccess &&
-              cudaMalloc(&b->d_steps, sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&b->d_done, sizeof(unsigned)) == cudaSuccess;
+              cudaMalloc(&b->d_steps, 2 * sizeof(double)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         batch_release(b);
         delete b;
         return fail(LBM_ERR_OOM, "device allocation failed");
     }
-    // tensor maps: [case][buffer][f, g] per tile shape
-    EncodeTiled enc = get_encoder();
-    if (!enc) { batch_release(b); delete b; return fail(LBM_ERR_CUDA, "cuTensorMapEncodeTiled unavailable"); }
-    CUtensorMapDataType dt = b->storage == S_F32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                             : b->storage == S_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                   : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    for (int v = 0; v < 2; ++v) {
-        int bx, by;
-        batch_tile(b->storage, v, &bx, &by);
-        std::vector<CUtensorMap> maps((size_t)ncases * 4);
-        for (int i = 0; i < ncases; ++i) {
-            const Geometry& G = b->L[i].geo;
-            const int x0 = G.PX - G.HX;  // map x = 0: the first ghost column
-            // up to the right ghost block: boxes of ragged tiles read the
-            // out-of-bounds fill, not the row padding
-            cuuint64_t dims[3] = {(cuuint64_t)((G.nx > bx ? G.nx : bx) + 2 * G.HX), (cuuint64_t)G.nyp, 18};
-            cuuint64_t strides[2] = {(cuuint64_t)G.pitch * b->esize, (cuuint64_t)G.plane * b->esize};
-            cuuint32_t estr[3] = {1, 1, 1};
-            cuuint32_t boxf[3] = {(cuuint32_t)(bx + 2 * G.HX), (cuuint32_t)(by + 4), 9};
-            cuuint32_t boxg[3] = {(cuuint32_t)(bx + 2 * G.HX), (cuuint32_t)(by + 2), 9};
-            for (int buf = 0; buf < 2; ++buf) {
-                void* base = static_cast<unsigned char*>(b->arena[buf]) + ((size_t)b->off[i] + x0) * b->esize;
-                CUresult r1 = enc(&maps[(i * 2 + buf) * 2], dt, 3, base, dims, strides, boxf, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-                CUresult r2 = enc(&maps[(i * 2 + buf) * 2 + 1], dt, 3, base, dims, strides, boxg, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-                if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS) {
-                    batch_release(b);
-                    delete b;
-                    return fail(LBM_ERR_CUDA, "cuTensorMapEncodeTiled failed for a batch case");
-                }
-            }
-        }
-        e = cudaMemcpy(b->d_maps[v], maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(b->d_cases[v], hc[v].data(), ncases * sizeof(BatchCase), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { batch_release(b); delete b; return cuda_fail(e, "cudaMemcpy"); }
-    }
-    std::vector<KC<float>> kk(ncases);
-    for (int i = 0; i < ncases; ++i) kk[i] = b->L[i].kf;
-    ok = cudaMemcpy(b->d_kcs, kk.data(), ncases * sizeof(KC<float>), cudaMemcpyHostToDevice) == cudaSuccess &&
+    ok = cudaMemcpy(b->d_cases, hc.data(), ncases * sizeof(BatchCase), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(b->arena[0], 0, abytes) == cudaSuccess && cudaMemset(b->arena[1], 0, abytes) == cudaSuccess &&
          cudaMemset(b->d_status, 0, sizeof(int)) == cudaSuccess &&
          cudaMemset(b->d_partials, 0, (size_t)b->max_items * 8 * sizeof(float)) == cudaSuccess &&
          cudaMemset(b->aux_counter, 0, sizeof(unsigned)) == cudaSuccess &&
-         cudaMemset(b->d_steps, 0, sizeof(double)) == cudaSuccess &&
-         cudaMemset(b->d_done, 0, sizeof(unsigned)) == cudaSuccess;
+         cudaMemset(b->d_steps, 0, 2 * sizeof(double)) == cudaSuccess;
     if (!ok) { batch_release(b); delete b; return fail(LBM_ERR_CUDA, "device initialisation failed"); }
-    e = batch_prepare(b->storage);
-    if (e == cudaSuccess) e = prepare_step(b->storage);
-    if (e != cudaSuccess) { batch_release(b); delete b; return cuda_fail(e, "cudaFuncSetAttribute"); }
     int rc = batch_upload_items(b);
     if (rc) { batch_release(b); delete b; return rc; }
     *out = b;
@@ -1151,7 +1142,7 @@ int lbm_batch_set_fields(lbm_batch* b, int32_t i, const double* rho, const doubl
         CK(cudaMemcpyAsync(b->scratch + k * n, src[k], n * sizeof(double), cudaMemcpyHostToDevice, b->stream));
         d[k] = b->scratch + k * n;
     }
-    CK(cudaMemsetAsync(case_buf(b, i, b->cur), 0, (size_t)18 * b->L[i].geo.plane * b->esize, b->stream));
+    CK(cudaMemsetAsync(case_buf(b, i, b->cur), 0, (size_t)b->L[i].geo.elems() * b->esize, b->stream));
     CK(launch_init(b->storage, b->L[i], d[0], d[1], d[2], d[3], case_buf(b, i, b->cur), b->stream));
     return batch_check(b);
 }
@@ -1162,7 +1153,7 @@ static int batch_build_graph(lbm_batch* b) {
     CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < lbm_batch::GRAPH_STEPS && e == cudaSuccess; ++k)
-        e = launch_batch_step(b->storage, b->shape, B, k & 1, b->arena[1 - (k & 1)], b->stream);
+        e = launch_batch_step(b->storage, B, k & 1, b->arena[k & 1], b->arena[1 - (k & 1)], b->stream);
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess) return cuda_fail(e, "batch step launch during capture");
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
@@ -1186,7 +1177,7 @@ int lbm_batch_step(lbm_batch* b, int n) {
             n -= lbm_batch::GRAPH_STEPS;
             continue;
         }
-        CK(launch_batch_step(b->storage, b->shape, B, b->cur, b->arena[1 - b->cur], b->stream));
+        CK(launch_batch_step(b->storage, B, b->cur, b->arena[b->cur], b->arena[1 - b->cur], b->stream));
         b->cur = 1 - b->cur;
         b->steps += 1;
         n -= 1;
@@ -1234,7 +1225,7 @@ int lbm_batch_step_stats(lbm_batch* b, int32_t i, double out[8]) {
     CK(launch_batch_case_record(batch_launch(b), i, b->d_rec, b->stream));
     double s[8], steps = 0.0;
     CK(cudaMemcpyAsync(s, b->d_rec, 8 * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-    CK(cudaMemcpyAsync(&steps, b->d_steps, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    CK(cudaMemcpyAsync(&steps, b->d_steps + b->cur, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     int rc = batch_check(b);
     for (int k = 0; k < 7; ++k) out[k] = s[k];
     out[7] = steps;
@@ -1275,11 +1266,11 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int32_t choice[2], double*
             int rc = lbm_batch_select(b, v, o);
             if (rc) return rc;
             const BatchLaunch B = batch_launch(b);
-            CK(launch_batch_step(b->storage, b->shape, B, b->cur, b->arena[1 - b->cur], b->stream));  // warm-up
+            CK(launch_batch_step(b->storage, B, b->cur, b->arena[b->cur], b->arena[1 - b->cur], b->stream));  // warm-up
             b->cur = 1 - b->cur;
             CK(cudaEventRecord(e0, b->stream));
             for (int k = 0; k < trial_steps; ++k) {
-                CK(launch_batch_step(b->storage, b->shape, B, b->cur, b->arena[1 - b->cur], b->stream));
+                CK(launch_batch_step(b->storage, B, b->cur, b->arena[b->cur], b->arena[1 - b->cur], b->stream));
                 b->cur = 1 - b->cur;
             }
             CK(cudaEventRecord(e1, b->stream));
@@ -1333,7 +1324,7 @@ int lbm_batch_destroy(lbm_batch* b) {
 
 int lbm_internal_fail(int code, const char* msg) { return fail(code, msg); }
 
-size_t lbm_internal_state_bytes(const lbm_handle* h) { return (size_t)18 * h->L.geo.plane * h->esize; }
+size_t lbm_internal_state_bytes(const lbm_handle* h) { return (size_t)h->L.geo.elems() * h->esize; }
 
 int lbm_internal_snapshot(lbm_handle* h, void* dst) {
     CK(cudaMemcpyAsync(dst, h->buf[h->cur], lbm_internal_state_bytes(h), cudaMemcpyDeviceToDevice, h->stream));
@@ -1342,10 +1333,10 @@ int lbm_internal_snapshot(lbm_handle* h, void* dst) {
 
 int lbm_internal_set_fields_fast(lbm_handle* h, const double* fields) {
     const size_t n = (size_t)h->cfg.nx * h->cfg.ny;
-    const size_t bytes = (size_t)18 * h->L.geo.plane * h->esize;
+    const size_t bytes = (size_t)h->L.geo.elems() * h->esize;
     CK(cudaMemsetAsync(h->buf[0], 0, bytes, h->stream));
     CK(launch_init(h->storage, h->L, fields, fields + n, fields + 2 * n, fields + 3 * n, h->buf[0], h->stream, true));
-    h->cur = 0;
+    CK(restart(h));
     return check_status(h);
 }
 
@@ -1375,7 +1366,7 @@ cudaStream_t lbm_internal_stream(const lbm_handle* h) { return h->stream; }
 int lbm_internal_set_steps(lbm_handle* h, int64_t steps) {
     CK(cudaStreamSynchronize(h->stream));
     const double st = (double)steps;
-    CK(cudaMemcpy(h->stats + 7, &st, sizeof st, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->count(h->cur), &st, sizeof st, cudaMemcpyHostToDevice));
     h->steps = steps;
     return LBM_OK;
 }

@@ -1,7 +1,6 @@
 // Internal declarations shared by the host runtime and the kernels of liblbm.
 #pragma once
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,6 +36,7 @@ struct KC {
     C dt_g1, dt_g2, hdt_g1, hdt_g2;  // dt gamma_1, dt gamma_2, dt/2 gamma_1, dt/2 gamma_2
     C c4g1_Cref, c4g2_Cref;          // (4 + gamma_1) C_ref, (4 - gamma_2) C_ref
     C c2_third;      // c^2 / 3
+    C rec_rho, rec_ax, rec_dg;  // total energy: a - 5 kappa / 3, kappa / 3, kappa / 12
     C T_bottom, T_top, T_hot;
     C rho_open, T_open;  // state of the open sides
     C rest[18];      // shifted-storage rest populations (f 0..8, g 9..17)
@@ -44,18 +44,29 @@ struct KC {
 };
 
 // Ghost columns that hold periodic copies: a pull reads one column beyond
-// the lattice and the density of the step's one-node ring pulls from a
-// second; the other columns of the HX-wide ghost block exist only to keep
-// the tile copies 16-byte aligned and are never read.
+// the lattice and the density beside it pulls from a second.
 constexpr int GHOST_COLS = 2;
 
+// The stored state is cut into strips of 32 nodes in x (64 for 16-bit
+// storage), the width of a warp: [strip][row][18 lines][strip width]. A line
+// holds one population of a row of a strip (128 bytes; 256 in FP64), so within
+// a strip every address is a compile-time offset from one pointer. Lines:
+// f_0 .. f_8, g_0 .. g_8. Column x of the lattice is column x + width of the
+// state (the first strip holds the ghost columns left of the lattice), node
+// row y its row y + 2.
+constexpr int ROW_LINES = 18;
+
 struct Geometry {
-    int nx, ny, walls, HX;  // HX: ghost columns on each side (16 bytes)
-    int PX;          // elements before column x = 0 of a row (128 bytes), so
-                     // that row stores start on a cache line
-    int pitch;       // padded row length in elements (a multiple of 128 bytes)
-    int nyp;         // padded number of rows (ny + 4 at least)
-    long long plane; // elements per plane
+    int nx, ny, walls;
+    int lsw;         // log2 of the strip width
+    int nyp;         // rows of a strip (ny + 4)
+    int strips;      // one more on each side than the lattice takes
+    // element of population p (f_i: i, g_i: 9 + i) of the node at (x, y)
+    __host__ __device__ __forceinline__ long long at(int p, int x, int y) const {
+        const int xx = x + (1 << lsw);
+        return (((((long long)(xx >> lsw) * nyp + (y + 2)) * ROW_LINES) + p) << lsw) + (xx & ((1 << lsw) - 1));
+    }
+    __host__ __device__ __forceinline__ long long elems() const { return ((long long)strips * nyp * ROW_LINES) << lsw; }
     int hot_x0, hot_len;
     int sms;         // persistent grid size (one CTA per SM)
     int open;        // open sides: 1 bottom, 2 top, 4 left, 8 right (left and right only together with all)
@@ -72,33 +83,42 @@ struct Launch {
     Geometry geo;
     KC<float> kf;
     KC<double> kd;
+    KC<float2> kp;  // kf in both lanes, for the packed arithmetic of 16-bit storage
     int rounding;  // 16-bit storage: 0 nearest, 1 stochastic
-    // bound in ns on each wait of the step kernel for a tile's copies; 0: the
-    // copies must already have landed when the tile's turn comes (no waiting)
+    // bound in ns on a warp's wait for its first rows; 0: no waiting
     unsigned long long tile_wait_ns;
     int cubic;  // eliminate the cubic velocity terms (periodic single cases)
 };
 
-// default tile-wait bound: 2 s
+// default bound: 2 s
 constexpr unsigned long long TILE_WAIT_NS_DEFAULT = 2000000000ull;
 
 // Storage kinds
 enum { S_F64 = 0, S_F32 = 1, S_F16 = 2, S_BF16 = 3 };
 
-// Host-side launchers (lbm_kernels.cu). All return cudaError_t of the launch.
-// phi: with L.cubic, [2][ny][nx] rho u_x^3 and rho u_y^3 (u over c) of the
-// state entering the step (launch_cubic_phi); otherwise unused
-cudaError_t launch_step(int storage, const Launch& L, const CUtensorMap* tmf, const CUtensorMap* tmg,
-                        void* out, double* partials, double* stats, unsigned* counter, int* status,
-                        cudaStream_t s, const double* phi = nullptr);
+// Host-side launchers. All return cudaError_t of the launch.
 // rho u_x^3 and rho u_y^3 of every node of a state (for the cubic-term
 // elimination): the density field into rho_scratch, then phi [2][ny][nx]
 cudaError_t launch_cubic_phi(int storage, const Launch& L, const void* buf, double* rho_scratch, double* phi,
                              cudaStream_t s);
-void step_tile(int storage, int* bx, int* by, int* hx);
-int step_blocks(int storage, const Geometry& g);
-size_t step_smem_bytes(int storage);
-cudaError_t prepare_step(int storage);  // per-device kernel attributes; call before capture
+// The row-marching step (lbm_march.cu): `groups` blocks of `warps` adjacent
+// strips each across x, `chunks` chunks of rows.
+struct MarchGrid {
+    int groups, warps, chunks;
+    int combine_prev;  // an extra block combines the record of the step before (prev)
+    int combine_here;  // the last block to finish combines this step's record
+};
+int march_strip(int storage);  // width of a warp's strip
+MarchGrid march_grid(int storage, const Geometry& g);
+// partials: [groups * chunks][NQ]; cnt_in, cnt_out: the step count before and
+// after the step (two places, so that every block can read it); phi: with
+// L.cubic, [2][ny][nx] rho u_x^3 and rho u_y^3 (u over c) of the state
+// entering the step (launch_cubic_phi), otherwise unused
+cudaError_t launch_march(int storage, const Launch& L, const void* in, void* out,
+                         const MarchGrid& mg, double* partials, const double* prev, double* stats, const double* cnt_in,
+                         double* cnt_out, unsigned* counter, int* status, cudaStream_t s, const double* phi = nullptr);
+// the record of a finished step whose partials no later step combined
+cudaError_t launch_record_finish(const double* partials, int nblk, double* stats, cudaStream_t s);
 
 // fast: FP32 per-node arithmetic for 32- and 16-bit storage (sums in FP64);
 // FP64 storage always computes in FP64

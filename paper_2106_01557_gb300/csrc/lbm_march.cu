@@ -1,0 +1,173 @@
+// The fused f+g step of a single lattice: the row-marching engine of
+// lbm_march.cuh over strips and chunks of rows, one task per warp.
+//
+// The blocks of one chunk of rows cover adjacent strips, and all chunks run
+// at once (one wave: as many chunks as there are resident blocks), so the
+// sectors two strips share are in the L2 cache when the second one asks.
+//
+// The conservation record of a step (per-block FP64 partial sums) is combined
+// by an extra block of the next step's launch, off the critical path, or,
+// where no step follows in the call, by the last block to finish.
+#include "lbm_march.cuh"
+
+namespace lbm {
+
+namespace {
+
+// stats[q] from the per-block partials [nblk][NQ]: warp w takes the
+// quantities w, w + nw, ...; lane l takes blocks l, l + 32, ... (independent
+// L2 loads), then a butterfly: a fixed order, so the record is the same on
+// every run
+__device__ __forceinline__ void combine_record(const double* partials, int nblk, double* stats, int warp, int nw, int lane) {
+    for (int q = warp; q < 7; q += nw) {
+        double t = 0.0;
+        for (int b = lane; b < nblk; b += 32) {
+            const double pv = __ldcg(partials + (size_t)b * NQ + q);
+            t = (q == 5) ? fmax(t, pv) : t + pv;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double w = __shfl_xor_sync(0xffffffffu, t, o);
+            t = (q == 5) ? fmax(t, w) : t + w;
+        }
+        if (lane == 0) stats[q] = (q == 5) ? sqrt(t) : t;
+    }
+}
+
+// OPEN: the case has open sides; CUBIC: the cubic-term elimination, with
+// phi = rho u_x^3, rho u_y^3 of the entering state (separate instantiations,
+// so that the common path carries none of their code)
+template <class S, class C, bool OPEN, bool CUBIC>
+__global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
+    k_march(const S* __restrict__ in, S* __restrict__ out, const __grid_constant__ Launch L, const MarchGrid mg, double* __restrict__ partials,
+            const double* __restrict__ prev, double* __restrict__ stats, const double* __restrict__ cnt_in,
+            double* __restrict__ cnt_out, unsigned* __restrict__ counter, int* __restrict__ status,
+            const double* __restrict__ phi) {
+    using Cf = MarchCfg<S>;
+    using V = typename std::conditional<Cf::NPL == 2, F2, C>::type;
+    __shared__ C red[MW][7];
+    __shared__ bool last;
+    const Geometry& G = L.geo;
+    const KC<C>& k = kc<C>(L);
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nw = blockDim.x / 32;
+    int block = blockIdx.x;
+    if (mg.combine_prev) {
+        // block 0: the record of the step before this one
+        if (block == 0) {
+            combine_record(prev, mg.groups * mg.chunks, stats, warp, nw, lane);
+            return;
+        }
+        block -= 1;
+    }
+    const int group = block % mg.groups, chunk = block / mg.groups;
+    Strip<S, C> w;
+    w.in = in;
+    w.out = out;
+    w.phi = phi;
+    w.xs = (group * nw + warp) * Cf::SW;
+    w.y0 = (int)((long long)G.ny * chunk / mg.chunks);
+    w.y1 = (int)((long long)G.ny * (chunk + 1) / mg.chunks);
+    Rec<C> acc = {C(0), C(0), C(0), C(0), C(0), C(0), C(0)};
+    if (w.xs < G.nx) {
+        w.wait_ns = L.tile_wait_ns;
+        // stochastic rounding is keyed by the step count
+        w.sr = Store<S, C>::SHIFTED && L.rounding;
+        w.step_key = w.sr ? fmix32((uint32_t)(long long)__ldcg(cnt_in) * 0x9e3779b9u + 0x7f4a7c15u) : 0u;
+        if (!march_rows<S, C, OPEN, CUBIC>(k, march_constants<V>(L), G, w, acc) && lane == 0) atomicOr(status, ST_TIMEOUT);
+    }
+    if (block == 0 && threadIdx.x == 0) *cnt_out = __ldcg(cnt_in) + 1.0;
+
+    // ---- block reduction: compute type within warps, FP64 across warps -----
+    C v[7];
+    reduce_record(acc, v);
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 7; ++q) red[warp][q] = v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {
+        const int q = threadIdx.x;
+        double t = 0.0;
+        for (int j = 0; j < nw; ++j) t = (q == 5) ? fmax(t, (double)red[j][q]) : t + (double)red[j][q];
+        const double cc = (double)k.c;
+        if (q == 1 || q == 2) t *= cc;
+        if (q == 5) t *= cc * cc;
+        partials[(size_t)block * NQ + q] = t;
+        if (q == 6 && t > 0.0) atomicOr(status, ST_NONFINITE);
+    }
+    if (!mg.combine_here) return;
+    __syncthreads();
+    const unsigned nblocks = (unsigned)(mg.groups * mg.chunks);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == nblocks - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    combine_record(partials, (int)nblocks, stats, warp, nw, lane);
+    if (threadIdx.x == 0) *counter = 0u;
+}
+
+__global__ void k_record_finish(const double* __restrict__ partials, int nblk, double* __restrict__ stats) {
+    combine_record(partials, nblk, stats, threadIdx.x / 32, blockDim.x / 32, threadIdx.x % 32);
+}
+
+template <class S, class C>
+cudaError_t march_t(const Launch& L, const void* in, void* out, const MarchGrid& mg,
+                    double* partials, const double* prev, double* stats, const double* cnt_in, double* cnt_out,
+                    unsigned* counter, int* status, cudaStream_t s, const double* phi) {
+    const dim3 grid((unsigned)(mg.groups * mg.chunks + (mg.combine_prev ? 1 : 0))), blk((unsigned)(32 * mg.warps));
+    const S* i = static_cast<const S*>(in);
+    S* o = static_cast<S*>(out);
+    if (L.geo.open)
+        k_march<S, C, true, false><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
+    else if (L.cubic)
+        k_march<S, C, false, true><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
+    else
+        k_march<S, C, false, false><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+int march_strip(int storage) {
+    return storage == S_F64 ? MarchCfg<double>::SW : (storage == S_F32 ? MarchCfg<float>::SW : MarchCfg<__half>::SW);
+}
+
+MarchGrid march_grid(int storage, const Geometry& g) {
+    const int sw = march_strip(storage);
+    const int bps = storage == S_F64 ? MarchCfg<double>::BPS : (storage == S_F32 ? MarchCfg<float>::BPS : MarchCfg<__half>::BPS);
+    const int strips = (g.nx + sw - 1) / sw;
+    MarchGrid m;
+    m.groups = (strips + MW - 1) / MW;
+    m.warps = (strips + m.groups - 1) / m.groups;
+    // as many chunks of rows as fill one wave of resident blocks, which the
+    // block that combines the last record is part of
+    int chunks = (bps * g.sms - 1) / m.groups;
+    if (chunks > g.ny) chunks = g.ny;
+    if (chunks < 1) chunks = 1;
+    m.chunks = chunks;
+    m.combine_prev = m.combine_here = 0;
+    return m;
+}
+
+cudaError_t launch_march(int storage, const Launch& L, const void* in, void* out,
+                         const MarchGrid& mg, double* partials, const double* prev, double* stats, const double* cnt_in,
+                         double* cnt_out, unsigned* counter, int* status, cudaStream_t s, const double* phi) {
+    if (L.cubic && !phi) return cudaErrorInvalidValue;
+    switch (storage) {
+        case S_F64: return march_t<double, double>(L, in, out, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, s, phi);
+        case S_F32: return march_t<float, float>(L, in, out, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, s, phi);
+        case S_F16: return march_t<__half, float>(L, in, out, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, s, phi);
+        case S_BF16: return march_t<__nv_bfloat16, float>(L, in, out, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, s, phi);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_record_finish(const double* partials, int nblk, double* stats, cudaStream_t s) {
+    k_record_finish<<<1, 224, 0, s>>>(partials, nblk, stats);
+    return cudaGetLastError();
+}
+
+}  // namespace lbm

@@ -1,15 +1,12 @@
-// Inline-PTX helpers of the TMA pipelines: shared-memory addresses, the
-// global timer for bounded waits, mbarrier set-up / arrive / try-wait, and
-// 3-D tiled bulk tensor loads into shared memory.
+// Inline-PTX helpers of the asynchronous pipelines: shared-memory addresses, the
+// global timer for bounded waits, mbarrier set-up / arrive / try-wait.
 #pragma once
 
-#include <cuda.h>
 #include <stdint.h>
 
 namespace lbm {
 
-// Bound on any wait for an mbarrier phase: 2 s of wall time (the step
-// kernel's tile waits take theirs from the launch, with this as default).
+// Bound on any wait for an mbarrier phase: 2 s of wall time.
 constexpr uint64_t WAIT_NS = 2000000000ull;
 
 static __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -50,27 +47,5 @@ static __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t par
         : "memory");
     return ok != 0;
 }
-
-// non-blocking test of an mbarrier phase
-static __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-static __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-        : "memory");
-}
-
 
 }  // namespace lbm

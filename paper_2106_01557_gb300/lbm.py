@@ -323,8 +323,8 @@ class Lattice:
         return int(self.lib.lbm_step_count(self.h))
 
     def set_tile_wait(self, ns: int):
-        """Bound (ns) on each wait of the step kernel for a tile's copies;
-        0: no waiting. A wait that runs out is reported by the next
+        """Bound (ns) on the wait of each warp of the step kernel for its first
+        rows; 0: no waiting. A wait that runs out is reported by the next
         synchronising call as LBM_ERR_TIMEOUT."""
         _check(self.lib.lbm_set_tile_wait(self.h, int(ns)))
 
@@ -398,7 +398,7 @@ class Batch:
         return int(self.lib.lbm_batch_step_count(self.h))
 
     def set_tile_wait(self, ns: int):
-        """Bound (ns) on each wait of the batch kernel for an item's copies; 0: no waiting."""
+        """Bound (ns) on each wait of the batch kernel for an item's first rows; 0: no waiting."""
         _check(self.lib.lbm_batch_set_tile_wait(self.h, int(ns)))
 
     def autotune(self, trial_steps=10):
