@@ -25,6 +25,10 @@ struct ConvArgs {
     int res32_c;
     __nv_bfloat16* out16;         // [P][cout] BF16 output, or
     float* out32;                 // [P][cout] FP32 output
+    // launch_conv64 only:
+    int out_relu;                 // max(0, .) of the BF16 output
+    const unsigned long long* mbits;  // [P]: the mask as bits (or null), as an earlier layer's obits
+    unsigned long long* obits;    // [P]: set to the sign bits (> 0) of the BF16 output before its ReLU (or null)
 };
 
 size_t conv_smem_bytes(int cin, int cout);
@@ -33,6 +37,11 @@ cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, in
 // (lbm_conv_tc.cu); bit 0 of the device int *status is set if a wait for
 // the tensor cores ran out of time (the output is then incomplete).
 cudaError_t launch_conv_tc(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms, int* status);
+// The 64 -> 64 layers, warp-specialised (lbm_conv64.cu); outputs and status
+// as launch_conv_tc's.
+cudaError_t launch_conv64(const ConvArgs& a, cudaStream_t s, int sms, int* status);
+// the sign bits of a [P][64] activation, as launch_conv64's obits
+cudaError_t launch_sign_bits(const __nv_bfloat16* x, long long P, unsigned long long* bits, cudaStream_t s);
 // The gradient reductions write per-block partial sums to `part` and add
 // them in block order (no atomics, so results are reproducible bit for
 // bit); grad_scratch_floats(sms) floats serve both.

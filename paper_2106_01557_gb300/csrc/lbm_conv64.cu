@@ -1,0 +1,543 @@
+// 3x3 periodic convolution 64 -> 64 of the surrogate on the 5th-generation
+// tensor cores, warp-specialised: forward layers and input gradients.
+//
+// The output is cut into rows of 128 pixels (one MMA M); a CTA walks down
+// 128-pixel strips, each a contiguous run of rows. Roles, handing over by
+// mbarriers only (every wait bounded in time):
+//   warp 0        tensor copies of the input rows into a ring of C6_SLOTS
+//                 slots: 128 pixels, and 8 more on each side of which one is
+//                 the periodic halo (8-pixel boxes start on the 1024-byte
+//                 atoms of the 128-byte swizzle; narrow strips are filled by
+//                 8-pixel boxes only);
+//   warps 12-15   apply ReLU to a slot in place (where the layer wants it);
+//   warp 1        issues the MMAs, input-stationary: input row li feeds output
+//                 rows li - 2, li - 1 and li through taps dy = +1, 0, -1, whose
+//                 weights sit side by side in N, so one MMA (M = 128 pixels, N =
+//                 3 x 64, K = 16) applies one (dx, 16-channel) step to three
+//                 output rows. Output row t accumulates in block t % 8 of tensor
+//                 memory (64 columns); a step is cut in two where the blocks
+//                 wrap around. The epilogue leaves a block zeroed, so every MMA
+//                 accumulates. Each output sums its 36 K-steps in the order
+//                 (dy, dx, channel chunk);
+//   warps 4-11    two epilogue groups of 4 warps take the output rows in turn:
+//                 tensor memory -> registers (a thread is a pixel), bias, mask,
+//                 residual, ReLU, BF16, into one of the group's two staging
+//                 rows, from where one tensor store writes it. The residual row
+//                 is brought into the same staging row by a tensor copy, one row
+//                 of the group ahead. Masks are kept as one bit per channel: 8
+//                 bytes per pixel instead of the 128 of the activation whose sign
+//                 they are, written by the forward layer that computes it.
+//
+// What bounds it (1024 x 1024, one image): 268 MB per layer without and 402 MB
+// with the residual, 40 and 59 us at the measured copy bandwidth, against 35 us
+// of MMAs; without the residual copies the 12 layers of a forward pass take 133
+// us less, without any epilogue 230 us less. A forward pass takes 1269 us where
+// the layers with two block barriers per row and copies by the threads took
+// 1889, a training step on 8 x 256 x 256 3310 instead of 4625. The descriptors
+// have to be warp-uniform: with one lane walking the rows each MMA cost its
+// thread about 130 cycles (1428 us per forward pass).
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <mutex>
+
+#include "lbm_conv.h"
+#include "lbm_ptx.cuh"
+#include "lbm_tc.cuh"
+
+namespace lbm {
+namespace {
+
+constexpr int C6_W = 128;                  // pixels per output row segment (MMA M)
+constexpr int C6_SLOTS = 4;                // input-row ring
+constexpr int C6_BLK = 8;                  // accumulator blocks in tensor memory
+constexpr int C6_THREADS = 512;
+constexpr int C6_SLOT = (C6_W + 16) * 128;  // 8 halo pixels on each side
+constexpr int C6_ROW = C6_W * 128;          // a staged row
+constexpr int C6_WDX = 3 * 64 * 128;        // weights of one dx
+constexpr int C6_OFF_IN = 3 * C6_WDX;
+constexpr int C6_OFF_OUT = C6_OFF_IN + C6_SLOTS * C6_SLOT;
+constexpr int C6_BYTES = C6_OFF_OUT + 4 * C6_ROW + 1024;
+static_assert(C6_BYTES <= 227 * 1024 && C6_SLOT % 1024 == 0 && C6_WDX % 1024 == 0, "shared memory");
+
+struct C6Maps {
+    CUtensorMap in, in8, out, out8, res, res8;  // boxes of 128 and of 8 pixels
+};
+
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* tm, int x, int row, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(0), "r"(x), "r"(row), "r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void tma_store(const CUtensorMap* tm, int x, int row, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     reinterpret_cast<uint64_t>(tm)),
+                 "r"(0), "r"(x), "r"(row), "r"(src)
+                 : "memory");
+}
+
+// Wait for a phase of bar, bounded; false after the bound, or once another
+// role has given up (dead is set for all).
+__device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (!mbar_try_wait(bar, parity)) {
+        if (*dead || globaltimer_ns() - t0 > WAIT_NS) {
+            *dead = 1;
+            return false;
+        }
+    }
+    return true;
+}
+
+// the same for a converged warp: one outcome for all lanes
+__device__ __forceinline__ bool role_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
+    return __all_sync(0xffffffffu, role_wait(bar, parity, dead));
+}
+
+__global__ void __launch_bounds__(C6_THREADS, 1)
+    k_conv64(const __grid_constant__ C6Maps tm, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
+             int N, int H, int W, int in_relu, int out_relu, int with_res, const uint2* __restrict__ mbits,
+             uint2* __restrict__ obits, int* __restrict__ status) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full[C6_SLOTS], ready[C6_SLOTS], empty[C6_SLOTS], acc_full[C6_BLK], acc_empty[C6_BLK],
+        side[2][2];
+    __shared__ uint32_t tmem_base;
+    __shared__ __align__(16) float s_bias[64];
+    __shared__ int dead_flag;
+    volatile int* dead = &dead_flag;
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
+
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < C6_SLOTS; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&ready[s], 4);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < C6_BLK; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 4);
+        }
+        for (int b = 0; b < 4; ++b) mbar_init(&side[b / 2][b % 2], 1);
+        fence_mbar_init();
+        dead_flag = 0;
+    }
+    if (tid < 64) s_bias[tid] = bias ? bias[tid] : 0.f;
+    // weights [9 taps (dy, dx)][co][ci] -> [3 dx][n = block (dy = +1, 0, -1) * 64 + co][64 ci], 16-byte
+    // chunks swizzled by the row
+    for (int e = tid; e < 9 * 64 * 8; e += C6_THREADS) {
+        const int kg = e % 8, co = (e / 8) % 64, tap = e / 512;
+        const int n = (2 - tap / 3) * 64 + co;
+        *reinterpret_cast<uint4*>(smem + (tap % 3) * C6_WDX + n * 128 + ((kg ^ (n & 7)) * 16)) =
+            *reinterpret_cast<const uint4*>(w + ((size_t)tap * 64 + co) * 64 + kg * 8);
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    if (warp >= 4 && warp < 8) {  // every accumulator block starts zeroed
+#pragma unroll 1
+        for (int c = 0; c < 512; c += 32) tc_st_zero32(tmem + ((uint32_t)(32 * (warp % 4)) << 16) + (uint32_t)c);
+        tc_wait_st();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+
+    const int tiles_x = (W + C6_W - 1) / C6_W;
+    const long long rows_total = (long long)N * tiles_x * H;
+    const long long r_begin = rows_total * blockIdx.x / gridDim.x, r_end = rows_total * (blockIdx.x + 1) / gridDim.x;
+    // the CTA's runs: rows y0 .. y0 + L - 1 of a strip starting at x0 with nv
+    // pixels in image n; q0 input rows and t0 output rows came before
+    struct Run {
+        int y0, L, x0, nv, n;
+    };
+    auto run_at = [&](long long r) {
+        Run u;
+        u.y0 = (int)(r % H);
+        const long long strip = r / H;
+        u.x0 = (int)(strip % tiles_x) * C6_W;
+        u.n = (int)(strip / tiles_x);
+        u.L = (int)((long long)(H - u.y0) < r_end - r ? (long long)(H - u.y0) : r_end - r);
+        u.nv = W - u.x0 < C6_W ? W - u.x0 : C6_W;
+        return u;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            unsigned q = 0;  // input rows issued
+            bool ok = true;
+            for (long long r = r_begin; r < r_end && ok;) {
+                const Run u = run_at(r);
+                r += u.L;
+                const int xl = u.x0 == 0 ? W - 8 : u.x0 - 8, xr = u.x0 + u.nv == W ? 0 : u.x0 + u.nv;
+                for (int li = 0; li < u.L + 2; ++li, ++q) {
+                    const unsigned s = q % C6_SLOTS;
+                    if (q >= C6_SLOTS && !role_wait(&empty[s], (q / C6_SLOTS - 1) & 1u, dead)) {
+                        ok = false;
+                        break;
+                    }
+                    int gy = u.y0 - 1 + li;
+                    gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
+                    const int row = u.n * H + gy;
+                    const uint32_t dst = sbase + C6_OFF_IN + s * C6_SLOT;
+                    mbar_arrive_expect_tx(&full[s], (uint32_t)(u.nv + 16) * 128u);
+                    tma_load(dst, &tm.in8, xl, row, &full[s]);
+                    if (u.nv == C6_W) {
+                        tma_load(dst + 1024, &tm.in, u.x0, row, &full[s]);
+                    } else {
+                        for (int x = 0; x < u.nv; x += 8) tma_load(dst + 1024 + x * 128, &tm.in8, u.x0 + x, row, &full[s]);
+                    }
+                    tma_load(dst + 1024 + u.nv * 128, &tm.in8, xr, row, &full[s]);
+                }
+            }
+            // every copy issued lands before the shared memory is given up
+            for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) {
+                const unsigned p = q - 1 - j;
+                const uint64_t t1 = globaltimer_ns();
+                while (!mbar_try_wait(&full[p % C6_SLOTS], (p / C6_SLOTS) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
+            }
+        }
+    } else if (warp == 1) {
+        // The whole warp walks the rows, so that descriptors and addresses are
+        // warp-uniform; one elected lane issues.
+        // D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 = 1), K-major, M >> 4 at bits 24-28; N >> 3 (bits 17-22)
+        // per MMA
+        const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(C6_W >> 4) << 24);
+        const uint64_t b_desc = sdesc_sw128(sbase);
+        const uint64_t a_desc = sdesc_sw128(sbase + C6_OFF_IN + 1024 - 128);
+        const uint32_t ahi = (uint32_t)(a_desc >> 32), bhi = (uint32_t)(b_desc >> 32);
+        unsigned q = 0, t0 = 0;
+        bool ok = true;
+        for (long long r = r_begin; r < r_end && ok;) {
+            const Run u = run_at(r);
+            r += u.L;
+            for (int li = 0; li < u.L + 2; ++li, ++q) {
+                const unsigned s = q % C6_SLOTS;
+                if (li < u.L) {  // the block that output row li starts in
+                    const unsigned t = t0 + li;
+                    if (t >= C6_BLK && !role_wait_warp(&acc_empty[t % C6_BLK], (t / C6_BLK - 1) & 1u, dead)) {
+                        ok = false;
+                        break;
+                    }
+                }
+                if (!role_wait_warp(in_relu ? &ready[s] : &full[s], (q / C6_SLOTS) & 1u, dead)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                // output rows tlo .. thi, in one MMA per step, or two where the
+                // accumulator blocks wrap around to block 0 at row wr
+                const int tlo = li - 2 > 0 ? li - 2 : 0, thi = li < u.L - 1 ? li : u.L - 1;
+                const int to_wrap = C6_BLK - (int)((t0 + tlo) % C6_BLK);  // rows up to the wrap
+                const int wr = tlo + to_wrap <= thi ? tlo + to_wrap : thi + 1;
+                const uint32_t d0 = tmem + ((t0 + tlo) % C6_BLK) * 64u;
+                const uint32_t b0 = (uint32_t)b_desc + (uint32_t)((tlo - li + 2) * 64 * 128 >> 4);
+                const uint32_t b1 = (uint32_t)b_desc + (uint32_t)((wr - li + 2) * 64 * 128 >> 4);
+                const uint32_t i0 = idesc0 | ((uint32_t)(wr - tlo) * 8u << 17), i1 = idesc0 | ((uint32_t)(thi + 1 - wr) * 8u << 17);
+                const uint32_t a0 = (uint32_t)a_desc + ((s * C6_SLOT) >> 4);
+                const bool two = wr <= thi;
+                if (elect_one()) {
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                        for (int kc = 0; kc < 4; ++kc)
+                            tc_mma_acc(d0, a0 + ((dx * 128 + kc * 32) >> 4), ahi, b0 + ((dx * C6_WDX + kc * 32) >> 4), bhi, i0);
+                    if (two) {
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                            for (int kc = 0; kc < 4; ++kc)
+                                tc_mma_acc(tmem, a0 + ((dx * 128 + kc * 32) >> 4), ahi, b1 + ((dx * C6_WDX + kc * 32) >> 4), bhi,
+                                           i1);
+                    }
+                    tc_commit(&empty[s]);
+                    if (li >= 2) tc_commit(&acc_full[(t0 + li - 2) % C6_BLK]);
+                }
+                __syncwarp();
+            }
+            t0 += u.L;
+        }
+        // the MMAs issued are done with the slots before the block ends
+        for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) {
+            const unsigned p = q - 1 - j;
+            const uint64_t t1 = globaltimer_ns();
+            while (!mbar_try_wait(&empty[p % C6_SLOTS], (p / C6_SLOTS) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
+        }
+    } else if (warp >= 12) {
+        if (in_relu) {
+            const int rt = tid - 12 * 32;
+            unsigned q = 0;
+            bool ok = true;
+            for (long long r = r_begin; r < r_end && ok;) {
+                const Run u = run_at(r);
+                r += u.L;
+                // pixels -1 .. nv of the strip, 8 vectors each
+                const int nvec = (u.nv + 2) * 8;
+                for (int li = 0; li < u.L + 2; ++li, ++q) {
+                    const unsigned s = q % C6_SLOTS;
+                    if (!role_wait(&full[s], (q / C6_SLOTS) & 1u, dead)) {
+                        ok = false;
+                        break;
+                    }
+                    uint4* v = reinterpret_cast<uint4*>(smem + C6_OFF_IN + s * C6_SLOT + 1024 - 128);
+#pragma unroll 4
+                    for (int e = rt; e < nvec; e += 128) v[e] = relu8(v[e]);
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ready[s]);
+                }
+            }
+        }
+    } else if (warp >= 4) {
+        const int grp = (warp - 4) / 4;
+        const int px = 32 * (warp % 4) + lane;  // pixel = tensor-memory lane
+        const uint32_t t_lane = tmem + ((uint32_t)(32 * (warp % 4)) << 16);
+        const bool leader = warp == 4 + 4 * grp && lane == 0;
+        // the group's output rows, one after another through the CTA's runs
+        struct Rows {
+            long long r;  // where the next run starts
+            Run u;
+            int t;        // row of the run
+            unsigned t0;  // output rows of the CTA before the run
+            bool more;
+        };
+        auto settle = [&](Rows& c) {  // on to the next run while the row lies beyond this one
+            while (c.more && c.t >= c.u.L) {
+                c.t0 += c.u.L;
+                if (c.r >= r_end) {
+                    c.more = false;
+                } else {
+                    c.u = run_at(c.r);
+                    c.r += c.u.L;
+                    c.t = (int)((c.t0 ^ (unsigned)grp) & 1u);
+                }
+            }
+        };
+        Rows c;
+        c.more = r_begin < r_end;
+        if (c.more) {
+            c.u = run_at(r_begin);
+            c.r = r_begin + c.u.L;
+            c.t = grp;
+            c.t0 = 0;
+            settle(c);
+        }
+        auto stage = [&](unsigned k) { return C6_OFF_OUT + (2 * grp + (int)(k & 1u)) * C6_ROW; };
+        // the residual of a row into its staging row (leader)
+        auto bring = [&](const Rows& d, unsigned k) {
+            const int row = d.u.n * H + d.u.y0 + d.t;
+            uint64_t* bar = &side[grp][k & 1u];
+            const uint32_t dst = sbase + stage(k);
+            mbar_arrive_expect_tx(bar, (uint32_t)d.u.nv * 128u);
+            if (d.u.nv == C6_W) {
+                tma_load(dst, &tm.res, d.u.x0, row, bar);
+            } else {
+                for (int x = 0; x < d.u.nv; x += 8) tma_load(dst + x * 128, &tm.res8, d.u.x0 + x, row, bar);
+            }
+        };
+        unsigned k = 0, brought = 0;  // rows of the group done; residuals asked for (leader)
+        if (with_res && leader && c.more) {
+            bring(c, 0);
+            brought = 1;
+        }
+        while (c.more) {
+            const unsigned tt = c.t0 + c.t;
+            const size_t pix = ((size_t)c.u.n * H + c.u.y0 + c.t) * W + c.u.x0 + px;
+            uint2 mw = make_uint2(0xffffffffu, 0xffffffffu);
+            if (mbits && px < c.u.nv) mw = __ldg(mbits + pix);
+            if (!role_wait(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
+            __syncwarp();
+            tc_fence_after();
+            float v[64];
+            tc_ld32(t_lane + (tt % C6_BLK) * 64u, v);
+            tc_ld32(t_lane + (tt % C6_BLK) * 64u + 32u, v + 32);
+            tc_wait_ld(v);
+            tc_st_zero32(t_lane + (tt % C6_BLK) * 64u);
+            tc_st_zero32(t_lane + (tt % C6_BLK) * 64u + 32u);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[tt % C6_BLK]);
+            if (with_res && !role_wait(&side[grp][k & 1u], (k >> 1) & 1u, dead)) break;
+            unsigned char* orow = smem + stage(k) + px * 128;
+            uint32_t bits[2] = {0u, 0u};
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float* x = v + 8 * q;
+                const int at = (q ^ (px & 7)) * 16;
+#pragma unroll
+                for (int j = 0; j < 8; j += 4) {
+                    const float4 b = *reinterpret_cast<const float4*>(s_bias + 8 * q + j);
+                    x[j] += b.x;
+                    x[j + 1] += b.y;
+                    x[j + 2] += b.z;
+                    x[j + 3] += b.w;
+                }
+                if (mbits) {
+                    // bit j of a word: channel 2 j of its 32, bit 16 + j: channel 2 j + 1
+                    const uint32_t m = q < 4 ? mw.x : mw.y;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (!(m & (1u << (4 * (q & 3) + j)))) x[2 * j] = 0.f;
+                        if (!(m & (0x10000u << (4 * (q & 3) + j)))) x[2 * j + 1] = 0.f;
+                    }
+                }
+                if (with_res) {
+                    const uint4 m = *reinterpret_cast<const uint4*>(orow + at);
+                    const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(&m);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) x[j] += __bfloat162float(mh[j]);
+                }
+                uint4 o;
+                __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+                if (obits) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        bits[q / 4] |= __hgt2_mask(oh[j], __floats2bfloat162_rn(0.f, 0.f)) & (0x10001u << (4 * (q & 3) + j));
+                }
+                if (out_relu) o = relu8(o);
+                *reinterpret_cast<uint4*>(orow + at) = o;
+            }
+            if (obits && px < c.u.nv) obits[pix] = make_uint2(bits[0], bits[1]);
+            Rows d = c;  // the row after this one
+            d.t += 2;
+            settle(d);
+            if (leader) {
+                // the other staging row is free once the store before has been read
+                bulk_wait_read0();
+                if (with_res && d.more) {
+                    bring(d, k + 1);
+                    ++brought;
+                }
+            }
+            fence_proxy_async();
+            group_sync(grp);
+            if (leader) {
+                const int row = c.u.n * H + c.u.y0 + c.t;
+                const uint32_t src = sbase + stage(k);
+                if (c.u.nv == C6_W) {
+                    tma_store(&tm.out, c.u.x0, row, src);
+                } else {
+                    for (int x = 0; x < c.u.nv; x += 8) tma_store(&tm.out8, c.u.x0 + x, row, src + x * 128);
+                }
+                bulk_commit();
+            }
+            c = d;
+            ++k;
+        }
+        if (leader) {
+            // after a wait that ran out: the residuals still in flight
+            for (unsigned j = k; j < brought; ++j) {
+                const uint64_t t1 = globaltimer_ns();
+                while (!mbar_try_wait(&side[grp][j & 1u], (j >> 1) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
+            }
+            bulk_wait_all();
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (tid == 0 && dead_flag) atomicOr(status, 1);
+    if (warp == 2) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// The sign bits of an activation no layer of this kernel has written (the
+// lift layer's): one 32-channel word per thread.
+__global__ void k_sign_bits(const uint4* __restrict__ x, long long words, uint32_t* __restrict__ bits) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < words; i += (long long)gridDim.x * blockDim.x) {
+        uint32_t b = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 v = __ldg(x + 4 * i + q);
+            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b |= __hgt2_mask(h[j], __floats2bfloat162_rn(0.f, 0.f)) & (0x10001u << (4 * q + j));
+        }
+        bits[i] = b;
+    }
+}
+
+using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiled get_encoder() {
+    static EncodeTiled fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiled>(p);
+    });
+    return fn;
+}
+
+}  // namespace
+
+// [rows][W][64] BF16: boxes of `px` pixels of one row, 128-byte swizzle
+cudaError_t encode_rows64(const void* base, long long rows, int W, int px, CUtensorMap* m) {
+    EncodeTiled enc = get_encoder();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t dims[3] = {64, (cuuint64_t)W, (cuuint64_t)rows}, strides[2] = {128, (cuuint64_t)W * 128};
+    const cuuint32_t box[3] = {64, (cuuint32_t)px, 1}, ones[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, ones,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? cudaSuccess
+               : cudaErrorInvalidValue;
+}
+
+cudaError_t launch_sign_bits(const __nv_bfloat16* x, long long P, unsigned long long* bits, cudaStream_t s) {
+    long long g = (2 * P + 255) / 256;
+    if (g > 8192) g = 8192;
+    k_sign_bits<<<(unsigned)g, 256, 0, s>>>(reinterpret_cast<const uint4*>(x), 2 * P, reinterpret_cast<uint32_t*>(bits));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_conv64(const ConvArgs& a, cudaStream_t s, int sms, int* status) {
+    if (a.N < 1 || a.H < 1 || a.W < 16 || a.W % 16 != 0 || !status || sms < 1 || !a.out16) return cudaErrorInvalidValue;
+    const long long rows = (long long)a.N * a.H, tiles = rows * ((a.W + C6_W - 1) / C6_W);
+    if (rows >= (1ll << 31)) return cudaErrorInvalidValue;
+    C6Maps m;
+    const void* res = a.res16 ? a.res16 : a.in;
+    const struct {
+        const void* p;
+        CUtensorMap *wide, *narrow;
+    } t[3] = {{a.in, &m.in, &m.in8}, {a.out16, &m.out, &m.out8}, {res, &m.res, &m.res8}};
+    for (const auto& e : t) {
+        cudaError_t rc = encode_rows64(e.p, rows, a.W, C6_W, e.wide);
+        if (rc == cudaSuccess) rc = encode_rows64(e.p, rows, a.W, 8, e.narrow);
+        if (rc != cudaSuccess) return rc;
+    }
+    const cudaError_t e = cudaFuncSetAttribute(k_conv64, cudaFuncAttributeMaxDynamicSharedMemorySize, C6_BYTES);
+    if (e != cudaSuccess) return e;
+    const int grid = tiles < sms ? (int)tiles : sms;
+    k_conv64<<<grid, C6_THREADS, C6_BYTES, s>>>(m, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.out_relu, a.res16 != nullptr,
+                                               reinterpret_cast<const uint2*>(a.mbits), reinterpret_cast<uint2*>(a.obits),
+                                               status);
+    return cudaGetLastError();
+}
+
+}  // namespace lbm

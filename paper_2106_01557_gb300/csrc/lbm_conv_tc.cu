@@ -1,4 +1,5 @@
-// 3x3 periodic convolution of the surrogate on the 5th-generation tensor
+// 3x3 periodic convolution of the surrogate's lift and projection layers (16 ->
+// 64, 64 -> 16 channels; lbm_conv64.cu has the 64 -> 64 layers) on the 5th-generation tensor
 // cores: tcgen05.mma (kind::f16: BF16 operands in shared memory, FP32
 // accumulators in tensor memory), completion tracked by tcgen05.commit on an
 // mbarrier (every wait bounded in time).
@@ -59,6 +60,7 @@
 
 #include "lbm_conv.h"
 #include "lbm_ptx.cuh"
+#include "lbm_tc.cuh"
 
 namespace lbm {
 namespace {
@@ -111,56 +113,6 @@ struct TcCfg {
     static_assert(BYTES <= 227 * 1024, "shared memory");
 };
 
-// shared-memory matrix descriptor: start >> 4 (bits 0-13), LBO >> 4 (16-29),
-// SBO >> 4 (32-45), fixed version 0b001 (46-48), no swizzle (61-63 = 0)
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
-
-// the same for a K-major operand in 128-byte swizzled rows: 8-row atoms of
-// 1024 bytes (SBO), LBO unused (16), swizzle mode 2 (bits 61-63)
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
-           (2ull << 61);
-}
-
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum)
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-// N consecutive FP32 columns (N = 8 or 16) of this thread's tensor-memory lane
-template <int N>
-__device__ __forceinline__ void tc_ld(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    if constexpr (N == 16) {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(taddr));
-    } else {
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(taddr));
-    }
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 // barrier of the epilogue threads only (the issue warp does not wait)
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI_THREADS) : "memory"); }
 
@@ -178,14 +130,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-__device__ __forceinline__ uint4 relu8(uint4 v) {
-    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&v);
-    const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) h[j] = __hmax2(h[j], z);
-    return v;
-}
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
@@ -780,7 +724,6 @@ cudaError_t launch_wgrad_tc(int cin, int cout, const __nv_bfloat16* in, const __
 cudaError_t launch_conv_tc(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms, int* status) {
     if (a.N < 1 || a.H < 1 || a.W < 16 || a.W % 16 != 0 || !status || sms < 1) return cudaErrorInvalidValue;
     if (cin == 16 && cout == 64) return conv_tc_t<16, 64>(a, s, sms, status);
-    if (cin == 64 && cout == 64) return conv_tc_t<64, 64>(a, s, sms, status);
     if (cin == 64 && cout == 16) return conv_tc_t<64, 16>(a, s, sms, status);
     return cudaErrorInvalidValue;
 }

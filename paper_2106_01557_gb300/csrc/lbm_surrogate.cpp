@@ -62,6 +62,10 @@ struct lbm_surrogate {
     __nv_bfloat16* dy16 = nullptr; // [P][16]
     std::vector<__nv_bfloat16*> h;   // B + 1 activations [P][C]
     std::vector<__nv_bfloat16*> z1;  // B activations
+    // sign bits of h[b] and z1[b] ([P] words each, b = 0 .. B - 1 consecutive):
+    // the masks of the backward pass (tensor-core path)
+    unsigned long long* hbits = nullptr;
+    unsigned long long* zbits = nullptr;
     __nv_bfloat16* g0 = nullptr;     // gradient buffers [P][C]
     __nv_bfloat16* g1 = nullptr;
     __nv_bfloat16* g2 = nullptr;
@@ -92,7 +96,8 @@ static void release_acts(lbm_surrogate* s) {
     for (auto* p : s->z1) s_free(p);
     s->h.clear();
     s->z1.clear();
-    s_free(s->g0); s_free(s->g1); s_free(s->g2);
+    s_free(s->g0); s_free(s->g1); s_free(s->g2); s_free(s->hbits); s_free(s->zbits);
+    s->hbits = s->zbits = nullptr;
     s->x16 = nullptr; s->x32 = s->t32 = s->y32 = nullptr; s->dy16 = s->g0 = s->g1 = s->g2 = nullptr;
     s->cap = 0;
 }
@@ -121,7 +126,9 @@ static int ensure_acts(lbm_surrogate* s, long long P, bool train) {
     }
     if (ok && train)
         ok = cudaMalloc(&s->g0, a) == cudaSuccess && cudaMalloc(&s->g1, a) == cudaSuccess &&
-             cudaMalloc(&s->g2, a) == cudaSuccess;
+             cudaMalloc(&s->g2, a) == cudaSuccess &&
+             cudaMalloc(&s->hbits, (size_t)P * s->cfg.blocks * 8) == cudaSuccess &&
+             cudaMalloc(&s->zbits, (size_t)P * s->cfg.blocks * 8) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         release_acts(s);
@@ -146,7 +153,9 @@ static ConvArgs cargs(const __nv_bfloat16* in, const __nv_bfloat16* w, const flo
 
 // 3x3 convolution on the configured path
 static int conv(lbm_surrogate* s, int cin, int cout, const ConvArgs& a) {
-    if (s->cfg.conv_path == 0) {
+    if (s->cfg.conv_path == 0 && cin == 64 && cout == 64) {
+        SCK(launch_conv64(a, s->stream, s->sms, s->d_status));
+    } else if (s->cfg.conv_path == 0) {
         SCK(launch_conv_tc(cin, cout, a, s->stream, s->sms, s->d_status));
     } else {
         SCK(launch_conv(cin, cout, a, s->stream, s->sms));
@@ -191,10 +200,12 @@ static int check_status(lbm_surrogate* s) {
 // forward pass; with train = true every activation is kept for backward
 static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
     const int B = s->cfg.blocks, C = s->cfg.channels;
+    const long long P = (long long)N * H * W;
     const Layer& lift = s->layers[0];
     ConvArgs a = cargs(s->x16, lift.w16, lift.b, N, H, W, 0);
     a.out16 = s->h[0];
     CONV(16, C, a);
+    if (train && s->cfg.conv_path == 0) SCK(launch_sign_bits(s->h[0], P, s->hbits, s->stream));
     for (int b = 0; b < B; ++b) {
         const Layer& L1 = s->layers[1 + 2 * b];
         const Layer& L2 = s->layers[2 + 2 * b];
@@ -203,10 +214,16 @@ static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
         __nv_bfloat16* z = train ? s->z1[b] : s->z1[0];
         a = cargs(hin, L1.w16, L1.b, N, H, W, 1);
         a.out16 = z;
+        // z1 only ever enters through its ReLU and its sign: the tensor-core
+        // path stores max(0, z1), so that its readers need not apply it again
+        const int tc = s->cfg.conv_path == 0;
+        a.out_relu = tc;
+        if (tc && train) a.obits = s->zbits + b * P;
         CONV(C, C, a);
-        a = cargs(z, L2.w16, L2.b, N, H, W, 1);
+        a = cargs(z, L2.w16, L2.b, N, H, W, !tc);
         a.res16 = hin;
         a.out16 = hout;
+        if (tc && train && b + 1 < B) a.obits = s->hbits + (b + 1) * P;
         CONV(C, C, a);
     }
     const Layer& proj = s->layers.back();
@@ -220,6 +237,7 @@ static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
 
 static int run_backward(lbm_surrogate* s, int N, int H, int W) {
     const int B = s->cfg.blocks, C = s->cfg.channels;
+    const bool tc = s->cfg.conv_path == 0;
     const long long P = (long long)N * H * W;
     for (Layer& L : s->layers) {
         SCK(cudaMemsetAsync(L.gw, 0, (size_t)L.nw() * 4, s->stream));
@@ -239,16 +257,18 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
         Layer& L1 = s->layers[1 + 2 * b];
         Layer& L2 = s->layers[2 + 2 * b];
         // h_{b+1} = h_b + conv2(relu(z1)); d z2 = d h_{b+1}
-        WGRAD(C, C, s->z1[b], dh, 1, L2.gw);
+        WGRAD(C, C, s->z1[b], dh, s->cfg.conv_path != 0, L2.gw);
         SCK(launch_bgrad(dh, P, C, L2.gb, s->gpart, s->stream));
         a = cargs(dh, L2.wflip, nullptr, N, H, W, 0);
-        a.mask = s->z1[b];
+        if (tc) a.mbits = s->zbits + b * P;
+        else a.mask = s->z1[b];
         a.out16 = s->g1;  // d z1
         CONV(C, C, a);
         WGRAD(C, C, s->h[b], s->g1, 1, L1.gw);
         SCK(launch_bgrad(s->g1, P, C, L1.gb, s->gpart, s->stream));
         a = cargs(s->g1, L1.wflip, nullptr, N, H, W, 0);
-        a.mask = s->h[b];
+        if (tc) a.mbits = s->hbits + b * P;
+        else a.mask = s->h[b];
         a.res16 = dh;
         a.out16 = spare;  // d h_b = d h_{b+1} + conv1^T(d z1) * [h_b > 0]
         CONV(C, C, a);
