@@ -60,7 +60,7 @@ template <int CIN, int COUT>
 __global__ void __launch_bounds__(CT, 1)
     k_conv(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
            int N, int H, int W, int in_relu, const __nv_bfloat16* __restrict__ mask,
-           const __nv_bfloat16* __restrict__ res16, const float* __restrict__ res32, int res32_c,
+           const __nv_bfloat16* __restrict__ res16, const float* __restrict__ res32,
            __nv_bfloat16* __restrict__ out16, float* __restrict__ out32) {
     using SMc = ConvSmem<CIN, COUT>;
     constexpr int PS = SMc::PS;
@@ -141,13 +141,14 @@ __global__ void __launch_bounds__(CT, 1)
                         v0 += __bfloat162float(r.x);
                         v1 += __bfloat162float(r.y);
                     }
-                    if (res32) {
-                        if (co < res32_c) v0 += res32[p * res32_c + co];
-                        if (co + 1 < res32_c) v1 += res32[p * res32_c + co + 1];
-                    }
                     if (out32) {
-                        out32[p * COUT + co] = v0;
-                        out32[p * COUT + co + 1] = v1;
+                        if (co >= 4) continue;
+                        if (res32) {
+                            v0 += res32[p * 4 + co];
+                            v1 += res32[p * 4 + co + 1];
+                        }
+                        out32[p * 4 + co] = v0;
+                        out32[p * 4 + co + 1] = v1;
                     } else {
                         *reinterpret_cast<__nv_bfloat162*>(out16 + p * COUT + co) = __floats2bfloat162_rn(v0, v1);
                     }
@@ -301,21 +302,40 @@ __global__ void __launch_bounds__(WT)
     }
 }
 
-// dw[tp][co][ci] += sum over blocks b = 0, 1, ... of the partials, tap
-// tp = 3 (dy + 1) + dx + 1 (the order of the sum is fixed)
-__global__ void k_wgrad_sum(const float* __restrict__ part, int nblk, int cc, float* __restrict__ dw) {
-    const int n = 9 * cc;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        const int tp = e / cc, rem = e % cc;
-        const int by = tp / 3, tl = tp % 3;
-        float s = 0.f;
+// dw[tp][co][ci] = the sum over blocks of the partials, tap tp = 3 (dy + 1) +
+// dx + 1, four weights per thread: thread row ty adds blocks ty, ty + 8, ... in
+// that order, then the eight rows are added in order (a fixed order).
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float4* __restrict__ part, int nblk, int n4, float4* __restrict__ dw) {
+    __shared__ float4 s[8][32];
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+    const int e = blockIdx.x * 32 + tx;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < n4) {
 #pragma unroll 8
-        for (int b = 0; b < nblk; ++b) s += part[(((size_t)b * 3 + by) * 3 + tl) * cc + rem];
-        dw[e] += s;
+        for (int b = ty; b < nblk; b += 8) {
+            const float4 v = __ldcg(part + (size_t)b * n4 + e);
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+    }
+    s[ty][tx] = a;
+    __syncthreads();
+    if (ty == 0 && e < n4) {
+#pragma unroll
+        for (int j = 1; j < 8; ++j) {
+            const float4 v = s[j][tx];
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+        dw[e] = a;
     }
 }
 
-// Bias gradient db[c] += sum_p dOut[p][c] (C a multiple of 8, C <= 256):
+// Bias gradient db[c] = sum_p dOut[p][c] (C a multiple of 8, C <= 256):
 // thread = one 8-channel group of a pixel (16-byte loads, coalesced across
 // the block), per-thread sums reduced per channel group in shared memory.
 __global__ void k_bgrad(const __nv_bfloat16* __restrict__ dout, long long P, int C, float* __restrict__ part) {
@@ -343,7 +363,7 @@ __global__ void k_bgrad(const __nv_bfloat16* __restrict__ dout, long long P, int
     }
 }
 
-// db[c] += sum over blocks b = 0, 1, ... of part[b][c]
+// db[c] = sum over blocks b = 0, 1, ... of part[b][c]
 // One warp per channel: lane l adds the partials of blocks l, l + 32, ...
 // in that order, then a butterfly over the lanes; lane 0's result is the
 // same on every run (a fixed order, not a sequential one)
@@ -354,10 +374,10 @@ __global__ void k_bgrad_sum(const float* __restrict__ part, int nblk, int C, flo
     for (int b = lane; b < nblk; b += 32) t += part[(size_t)b * C + c];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) db[c] += t;
+    if (lane == 0) db[c] = t;
 }
 
-// *out += sum over i = 0 .. n-1 of part[i], by one warp in a fixed order
+// *out = sum over i = 0 .. n-1 of part[i], by one warp in a fixed order
 // (lane l: i = l, l + 32, ...; then a butterfly)
 __global__ void k_sum_in_order(const double* __restrict__ part, int n, double* __restrict__ out) {
     const int lane = threadIdx.x;
@@ -366,31 +386,44 @@ __global__ void k_sum_in_order(const double* __restrict__ part, int n, double* _
     for (int i = lane; i < n; i += 32) t += part[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) *out += t;
+    if (lane == 0) *out = t;
 }
 
 // loss = mean over P pixels and 4 channels of (out - target)^2; dout = d loss / d out.
-// With the mass-conserving output layer (csum not null) the density gradient
-// is projected: minus its per-image mean, which equals
-// 2 (mean(x_rho) - mean(target_rho)) / (4 P); csum[n] = sum over image n of
-// (x_rho - target_rho), HW pixels per image.
-__global__ void k_mse(const float* __restrict__ out, const float* __restrict__ target, long long P,
-                      __nv_bfloat16* __restrict__ dout, double* __restrict__ part, const double* __restrict__ csum,
-                      long long HW) {
+// With the mass-conserving output layer (sums not null) out_rho is first
+// shifted by -sums[n] / HW (image n), and the density gradient is projected:
+// minus its per-image mean, which equals 2 (mean(x_rho) - mean(target_rho)) /
+// (4 P); sums[N + n] = sum over image n of (x_rho - target_rho), HW pixels per
+// image. Grid y: images. Bound by memory (P x 64 bytes); with 64-bit divisions
+// and 2-byte stores per pixel it took 47 us on 8 x 256 x 256.
+__global__ void k_mse(const float4* __restrict__ out, const float4* __restrict__ target, int N, long long HW,
+                      uint4* __restrict__ dout, double* __restrict__ part, const double* __restrict__ sums) {
     __shared__ double s[256];
     double acc = 0.0;
+    const long long P = HW * N;
     const float scale = 2.0f / (float)(P * 4);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-        const float shift = csum ? (float)(csum[p / HW] / (double)HW) : 0.f;
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            float d = 0.f;
-            if (c < 4) {
-                d = out[p * 16 + c] - target[p * 4 + c];
-                acc += (double)d * d;
-            }
-            dout[p * 16 + c] = __float2bfloat16(c < 4 ? scale * (c == 0 ? d - shift : d) : 0.f);
-        }
+    __shared__ double means[2];
+    for (int n = blockIdx.y; n < N; n += gridDim.y) {
+    __syncthreads();
+    if (threadIdx.x < 2) means[threadIdx.x] = sums ? sums[threadIdx.x * N + n] / (double)HW : 0.0;
+    __syncthreads();
+    const double mean = means[0];
+    const float shift = (float)means[1];
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < HW; q += (long long)gridDim.x * blockDim.x) {
+        const long long p = n * HW + q;
+        const float4 o = out[p], t = target[p];
+        const float d0 = (sums ? (float)((double)o.x - mean) : o.x) - t.x, d1 = o.y - t.y, d2 = o.z - t.z, d3 = o.w - t.w;
+        acc += (double)d0 * d0;
+        acc += (double)d1 * d1;
+        acc += (double)d2 * d2;
+        acc += (double)d3 * d3;
+        const __nv_bfloat162 a = __floats2bfloat162_rn(scale * (d0 - shift), scale * d1), b = __floats2bfloat162_rn(scale * d2, scale * d3);
+        uint4 v = make_uint4(0, 0, 0, 0);
+        memcpy(&v.x, &a, 4);
+        memcpy(&v.y, &b, 4);
+        dout[2 * p] = v;
+        dout[2 * p + 1] = make_uint4(0, 0, 0, 0);
+    }
     }
     s[threadIdx.x] = acc;
     __syncthreads();
@@ -398,77 +431,100 @@ __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t
         if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = s[0] / (double)(P * 4);
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s[0] / (double)(P * 4);
 }
 
-// Adam on FP32 master weights of one convolution ([9][COUT][CIN] and bias),
-// then the BF16 forward copy and the flipped, transposed copy used for the
-// input gradient: wf[8 - tap][ci][co] = w[tap][co][ci].
-__global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ gw, int n, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float gi = gw[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// Adam on FP32 master weights of all layers in one launch (grid y = layers):
+// the update, then the BF16 forward copy and the flipped, transposed copy used
+// for the input gradient: wf[8 - tap][ci][co] = w[tap][co][ci]. Without
+// `update` only the copies. (42 launches of one layer's update or copy took 95 + 69 us.)
+__global__ void k_adam_refresh(const LayerDesc* __restrict__ layers, float* __restrict__ w, float* __restrict__ m,
+                               float* __restrict__ v, const float* __restrict__ g, __nv_bfloat16* __restrict__ w16,
+                               __nv_bfloat16* __restrict__ wflip, int update, float lr, float b1, float b2, float eps,
+                               float c1, float c2) {
+    const LayerDesc d = layers[blockIdx.y];
+    const int nw = 9 * d.cout * d.cin;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + d.cout; i += gridDim.x * blockDim.x) {
+        const long long e = d.off + i;  // the layer's weights, then its biases
+        float wi = w[e];
+        if (update) {
+            const float gi = g[e];
+            const float mi = b1 * m[e] + (1.f - b1) * gi;
+            const float vi = b2 * v[e] + (1.f - b2) * gi * gi;
+            m[e] = mi;
+            v[e] = vi;
+            wi -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+            w[e] = wi;
+        }
+        if (i < nw) {
+            const int ci = i % d.cin, co = (i / d.cin) % d.cout, tap = i / (d.cin * d.cout);
+            const float val = (ci < d.cin_real && co < d.cout_real) ? wi : 0.f;  // padding stays zero
+            const __nv_bfloat16 b = __float2bfloat16(val);
+            w16[d.off16 + i] = b;
+            wflip[d.off16 + ((long long)(8 - tap) * d.cin + ci) * d.cout + co] = b;
+        }
     }
 }
 
-__global__ void k_refresh(const float* __restrict__ w, int cin, int cout, int cin_real, int cout_real,
-                          __nv_bfloat16* __restrict__ w16, __nv_bfloat16* __restrict__ wflip) {
-    const int n = 9 * cout * cin;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int ci = i % cin, co = (i / cin) % cout, tap = i / (cin * cout);
-        const float val = (ci < cin_real && co < cout_real) ? w[i] : 0.f;  // padding stays zero
-        const __nv_bfloat16 b = __float2bfloat16(val);
-        w16[i] = b;
-        if (wflip) wflip[((size_t)(8 - tap) * cin + ci) * cout + co] = b;
-    }
-}
-
-// fields -> normalised network input: 16 BF16 channels (4 used) and an FP32
-// copy of the 4 channels for the output residual
+// fields -> normalised network input: 16 BF16 channels (4 used; x16 may be
+// null) and an FP32 copy of the 4 channels. One pixel per thread, 16-byte
+// stores (with 2-byte stores: 100 us at 1024 x 1024, four times its memory time).
 __global__ void k_pack(const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
-                       const double* __restrict__ T, long long P, NormConsts nc, __nv_bfloat16* __restrict__ x16,
-                       float* __restrict__ x32) {
+                       const double* __restrict__ T, long long P, NormConsts nc, uint4* __restrict__ x16,
+                       float4* __restrict__ x32) {
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-        const float v[4] = {(float)((rho[p] - nc.off[0]) * nc.inv_scale[0]), (float)((ux[p] - nc.off[1]) * nc.inv_scale[1]),
-                            (float)((uy[p] - nc.off[2]) * nc.inv_scale[2]), (float)((T[p] - nc.off[3]) * nc.inv_scale[3])};
-#pragma unroll
-        for (int c = 0; c < 16; ++c) x16[p * 16 + c] = __float2bfloat16(c < 4 ? v[c] : 0.f);
-        if (x32)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) x32[p * 4 + c] = v[c];
+        const float4 v = make_float4((float)((rho[p] - nc.off[0]) * nc.inv_scale[0]), (float)((ux[p] - nc.off[1]) * nc.inv_scale[1]),
+                                     (float)((uy[p] - nc.off[2]) * nc.inv_scale[2]), (float)((T[p] - nc.off[3]) * nc.inv_scale[3]));
+        x32[p] = v;
+        if (x16) {
+            const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+            uint4 o = make_uint4(0, 0, 0, 0);
+            memcpy(&o.x, &a, 4);
+            memcpy(&o.y, &b, 4);
+            x16[2 * p] = o;
+            x16[2 * p + 1] = make_uint4(0, 0, 0, 0);
+        }
     }
 }
 
-__global__ void k_unpack(const float* __restrict__ y, long long P, NormConsts nc, double* __restrict__ rho,
-                         double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ T) {
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-        rho[p] = nc.off[0] + (double)y[p * 16 + 0] * nc.scale[0];
-        ux[p] = nc.off[1] + (double)y[p * 16 + 1] * nc.scale[1];
-        uy[p] = nc.off[2] + (double)y[p * 16 + 2] * nc.scale[2];
-        T[p] = nc.off[3] + (double)y[p * 16 + 3] * nc.scale[3];
+// network output [P][4] -> fields, the density of image n (HW pixels; grid y =
+// images) first shifted by -sums[n] / HW (sums not null)
+__global__ void k_unpack(const float4* __restrict__ y, long long HW, const double* __restrict__ sums, NormConsts nc,
+                         int N, double* __restrict__ rho, double* __restrict__ ux, double* __restrict__ uy,
+                         double* __restrict__ T) {
+    __shared__ double s_mean;
+    for (int n = blockIdx.y; n < N; n += gridDim.y) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_mean = sums ? sums[n] / (double)HW : 0.0;  // (FP64 divisions are slow here: one per block)
+    __syncthreads();
+    const double mean = s_mean;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < HW; q += (long long)gridDim.x * blockDim.x) {
+        const long long p = n * HW + q;
+        const float4 v = y[p];
+        const float r = sums ? (float)((double)v.x - mean) : v.x;
+        rho[p] = nc.off[0] + (double)r * nc.scale[0];
+        ux[p] = nc.off[1] + (double)v.y * nc.scale[1];
+        uy[p] = nc.off[2] + (double)v.z * nc.scale[2];
+        T[p] = nc.off[3] + (double)v.w * nc.scale[3];
+    }
     }
 }
 
 // Mass-conserving output layer: per image n, sums[n] = sum of
 // (y_rho - x_rho) and, with a target, sums[N + n] = sum of (x_rho - t_rho);
-// then y_rho -= sums[n] / HW. y: [P][16], x, t: [P][4]; grid y = images.
+// its readers shift y_rho by -sums[n] / HW. y, x, t: [P][4]; grid y = images.
 // Each block writes its two partial sums to part[n][block][2];
 // k_mass_sums adds them in block order.
-__global__ void k_mass_stats(const float* __restrict__ y, const float* __restrict__ x, const float* __restrict__ t,
+__global__ void k_mass_stats(const float4* __restrict__ y, const float4* __restrict__ x, const float4* __restrict__ t,
                              int N, long long HW, double* __restrict__ part) {
     __shared__ double s[2][256];
     const int n = blockIdx.y;
     double a = 0.0, b = 0.0;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < HW; q += (long long)gridDim.x * blockDim.x) {
         const long long p = n * HW + q;
-        a += (double)y[p * 16] - (double)x[p * 4];
-        if (t) b += (double)x[p * 4] - (double)t[p * 4];
+        const double xr = (double)x[p].x;
+        a += (double)y[p].x - xr;
+        if (t) b += xr - (double)t[p].x;
     }
     s[0][threadIdx.x] = a;
     s[1][threadIdx.x] = b;
@@ -506,11 +562,6 @@ __global__ void k_mass_sums(const double* __restrict__ part, int N, int nblk, in
         sums[n] = a;
         if (with_t) sums[N + n] = b;
     }
-}
-
-__global__ void k_mass_apply(float* __restrict__ y, long long P, long long HW, const double* __restrict__ sums) {
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x)
-        y[p * 16] = (float)((double)y[p * 16] - sums[p / HW] / (double)HW);
 }
 
 // counts over a field set [4][P] of one W-wide periodic image: cnt[0] nodes
@@ -588,7 +639,7 @@ cudaError_t conv_t(const ConvArgs& a, cudaStream_t s, int sms) {
     const int tiles = a.N * ((a.H + TH - 1) / TH) * ((a.W + TW - 1) / TW);
     const int grid = tiles < sms ? tiles : sms;
     k_conv<CIN, COUT><<<grid, CT, SMc::BYTES, s>>>(a.in, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.mask, a.res16,
-                                                   a.res32, a.res32_c, a.out16, a.out32);
+                                                   a.res32, a.out16, a.out32);
     return cudaGetLastError();
 }
 
@@ -607,8 +658,8 @@ cudaError_t wgrad_t(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, i
     if (gx > chunks) gx = chunks;
     if (gx < 1) gx = 1;
     k_wgrad<CIN, COUT><<<dim3((unsigned)gx, 3), WT, 2 * Cf::STAGE, s>>>(in, dout, N, H, W, in_relu, part);
-    k_wgrad_sum<<<(9 * COUT * CIN + 255) / 256, 256, 0, s>>>(part, (int)gx, COUT * CIN, dw);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, (int)gx, COUT * CIN, dw, s);
 }
 
 }  // namespace
@@ -634,17 +685,15 @@ cudaError_t launch_field_change(const double* a, const double* b, long long P, u
     return cudaGetLastError();
 }
 
-cudaError_t launch_mass_layer(float* y, const float* x, const float* t, int N, long long HW, double* sums,
+cudaError_t launch_mass_layer(const float* y, const float* x, const float* t, int N, long long HW, double* sums,
                               double* part, cudaStream_t s) {
     if (N < 1 || HW < 1) return cudaErrorInvalidValue;
     long long gx = (HW + 255) / 256;
     if (gx > MASS_BLOCKS) gx = MASS_BLOCKS;
-    k_mass_stats<<<dim3((unsigned)gx, (unsigned)N), 256, 0, s>>>(y, x, t, N, HW, part);
+    k_mass_stats<<<dim3((unsigned)gx, (unsigned)N), 256, 0, s>>>(reinterpret_cast<const float4*>(y),
+                                                                 reinterpret_cast<const float4*>(x),
+                                                                 reinterpret_cast<const float4*>(t), N, HW, part);
     k_mass_sums<<<(32 * N + 127) / 128, 128, 0, s>>>(part, N, (int)gx, t != nullptr, sums);
-    const long long P = (long long)N * HW;
-    long long g = (P + 255) / 256;
-    if (g > 2048) g = 2048;
-    k_mass_apply<<<(unsigned)g, 256, 0, s>>>(y, P, HW, sums);
     return cudaGetLastError();
 }
 
@@ -679,7 +728,10 @@ cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_
 
 cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, cudaStream_t s) {
     if (nblk < 1 || cc < 1) return cudaErrorInvalidValue;
-    k_wgrad_sum<<<(9 * cc + 255) / 256, 256, 0, s>>>(part, nblk, cc, dw);
+    if (cc % 4 != 0) return cudaErrorInvalidValue;
+    const int n4 = 9 * cc / 4;
+    k_wgrad_sum<<<(n4 + 31) / 32, 256, 0, s>>>(reinterpret_cast<const float4*>(part), nblk, n4,
+                                              reinterpret_cast<float4*>(dw));
     return cudaGetLastError();
 }
 
@@ -693,26 +745,24 @@ cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* d
     return cudaGetLastError();
 }
 
-cudaError_t launch_mse(const float* out, const float* target, long long P, __nv_bfloat16* dout, double* loss,
-                       const double* csum, long long HW, double* part, cudaStream_t s) {
-    if (csum && HW < 1) return cudaErrorInvalidValue;
-    long long g = (P + 255) / 256;
-    if (g > MSE_BLOCKS) g = MSE_BLOCKS;
-    k_mse<<<(unsigned)g, 256, 0, s>>>(out, target, P, dout, part, csum, HW);
-    k_sum_in_order<<<1, 32, 0, s>>>(part, (int)g, loss);
+cudaError_t launch_mse(const float* out, const float* target, int N, long long HW, __nv_bfloat16* dout, double* loss,
+                       const double* sums, double* part, cudaStream_t s) {
+    if (N < 1 || HW < 1) return cudaErrorInvalidValue;
+    const int ny = N < MSE_BLOCKS ? N : MSE_BLOCKS;
+    long long g = (HW + 255) / 256;
+    if (g > MSE_BLOCKS / ny) g = MSE_BLOCKS / ny;
+    k_mse<<<dim3((unsigned)g, (unsigned)ny), 256, 0, s>>>(reinterpret_cast<const float4*>(out),
+                                                        reinterpret_cast<const float4*>(target), N, HW,
+                                                        reinterpret_cast<uint4*>(dout), part, sums);
+    k_sum_in_order<<<1, 32, 0, s>>>(part, (int)g * ny, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int n, float lr, float b1, float b2, float eps,
-                        float c1, float c2, cudaStream_t s) {
-    k_adam<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(w, m, v, g, n, lr, b1, b2, eps, c1, c2);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_refresh(const float* w, int cin, int cout, int cin_real, int cout_real, __nv_bfloat16* w16,
-                           __nv_bfloat16* wflip, cudaStream_t s) {
-    const int n = 9 * cin * cout;
-    k_refresh<<<(n + 255) / 256, 256, 0, s>>>(w, cin, cout, cin_real, cout_real, w16, wflip);
+cudaError_t launch_adam_refresh(const LayerDesc* layers, int nlayers, float* w, float* m, float* v, const float* g,
+                                __nv_bfloat16* w16, __nv_bfloat16* wflip, int update, float lr, float b1, float b2, float eps,
+                                float c1, float c2, cudaStream_t s) {
+    if (nlayers < 1) return cudaErrorInvalidValue;
+    k_adam_refresh<<<dim3(36, (unsigned)nlayers), 256, 0, s>>>(layers, w, m, v, g, w16, wflip, update, lr, b1, b2, eps, c1, c2);
     return cudaGetLastError();
 }
 
@@ -720,15 +770,17 @@ cudaError_t launch_pack(const double* rho, const double* ux, const double* uy, c
                         const NormConsts& nc, __nv_bfloat16* x16, float* x32, cudaStream_t s) {
     long long g = (P + 255) / 256;
     if (g > 4096) g = 4096;
-    k_pack<<<(unsigned)g, 256, 0, s>>>(rho, ux, uy, T, P, nc, x16, x32);
+    k_pack<<<(unsigned)g, 256, 0, s>>>(rho, ux, uy, T, P, nc, reinterpret_cast<uint4*>(x16), reinterpret_cast<float4*>(x32));
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack(const float* y, long long P, const NormConsts& nc, double* rho, double* ux, double* uy,
-                          double* T, cudaStream_t s) {
-    long long g = (P + 255) / 256;
-    if (g > 4096) g = 4096;
-    k_unpack<<<(unsigned)g, 256, 0, s>>>(y, P, nc, rho, ux, uy, T);
+cudaError_t launch_unpack(const float* y, int N, long long HW, const double* sums, const NormConsts& nc, double* rho,
+                          double* ux, double* uy, double* T, cudaStream_t s) {
+    if (N < 1 || HW < 1) return cudaErrorInvalidValue;
+    const int ny = N < 1024 ? N : 1024;
+    long long g = (HW + 255) / 256;
+    if (g > 1216) g = 1216;
+    k_unpack<<<dim3((unsigned)g, (unsigned)ny), 256, 0, s>>>(reinterpret_cast<const float4*>(y), HW, sums, nc, N, rho, ux, uy, T);
     return cudaGetLastError();
 }
 

@@ -21,10 +21,9 @@ struct ConvArgs {
     int in_relu;                  // apply max(0, .) to the input
     const __nv_bfloat16* mask;    // [P][cout]: zero where mask <= 0 (or null)
     const __nv_bfloat16* res16;   // [P][cout] added (or null)
-    const float* res32;           // [P][res32_c] added to the first res32_c channels (or null)
-    int res32_c;
+    const float* res32;           // [P][4] added to out32 (or null)
     __nv_bfloat16* out16;         // [P][cout] BF16 output, or
-    float* out32;                 // [P][cout] FP32 output
+    float* out32;                 // [P][4] FP32 output of the first four channels
     // launch_conv64 only:
     int out_relu;                 // max(0, .) of the BF16 output
     const unsigned long long* mbits;  // [P]: the mask as bits (or null), as an earlier layer's obits
@@ -53,7 +52,7 @@ cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_
 // bit 0 of *status as for launch_conv_tc.
 cudaError_t launch_wgrad_tc(int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
                             int in_relu, float* dw, float* part, cudaStream_t s, int sms, int* status);
-// dw[9][cc] += the sum over blocks 0 .. nblk - 1 (in that order) of the
+// dw[9][cc] = the sum over blocks 0 .. nblk - 1 (in a fixed order) of the
 // partials part[nblk][3 dy][3 dx][cc]
 cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, cudaStream_t s);
 cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* db, float* part, cudaStream_t s);
@@ -61,24 +60,30 @@ cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* d
 constexpr int MASS_BLOCKS = 256;
 // loss partials: part holds MSE_BLOCKS doubles
 constexpr int MSE_BLOCKS = 1024;
-// csum (may be null): per-image sums of (x_rho - target_rho) of the
-// mass-conserving output layer, HW pixels per image
-cudaError_t launch_mse(const float* out, const float* target, long long P, __nv_bfloat16* dout, double* loss,
-                       const double* csum, long long HW, double* part, cudaStream_t s);
-// Mass-conserving output layer on y [N*HW][16] given the input x [N*HW][4]:
-// y_rho -= mean over each image of (y_rho - x_rho). With a target t, also
-// sums[N + n] = sum over image n of (x_rho - t_rho) for launch_mse.
-// sums: 2 N doubles of scratch.
-cudaError_t launch_mass_layer(float* y, const float* x, const float* t, int N, long long HW, double* sums,
+// Mass-conserving output layer on y [N*HW][4] given the input x [N*HW][4]:
+// sums[n] = sum over image n of (y_rho - x_rho), by whose mean the readers of y
+// shift its density. With a target t, also sums[N + n] = sum over image n of
+// (x_rho - t_rho) for launch_mse. sums: 2 N doubles.
+cudaError_t launch_mass_layer(const float* y, const float* x, const float* t, int N, long long HW, double* sums,
                               double* part, cudaStream_t s);
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int n, float lr, float b1, float b2, float eps,
-                        float c1, float c2, cudaStream_t s);
-cudaError_t launch_refresh(const float* w, int cin, int cout, int cin_real, int cout_real, __nv_bfloat16* w16,
-                           __nv_bfloat16* wflip, cudaStream_t s);
+// loss of N images of HW pixels and its gradient; sums:
+// launch_mass_layer's, or null without the mass-conserving output layer
+cudaError_t launch_mse(const float* out, const float* target, int N, long long HW, __nv_bfloat16* dout, double* loss,
+                       const double* sums, double* part, cudaStream_t s);
+// A layer in the flat parameter arrays: weights [9][cout][cin] at off, then
+// the biases; its BF16 copies at off16
+struct LayerDesc {
+    int cin, cout, cin_real, cout_real;
+    long long off, off16;
+};
+// the BF16 copies of every layer, after an Adam step (update)
+cudaError_t launch_adam_refresh(const LayerDesc* layers, int nlayers, float* w, float* m, float* v, const float* g,
+                                __nv_bfloat16* w16, __nv_bfloat16* wflip, int update, float lr, float b1, float b2, float eps,
+                                float c1, float c2, cudaStream_t s);
 cudaError_t launch_pack(const double* rho, const double* ux, const double* uy, const double* T, long long P,
                         const NormConsts& nc, __nv_bfloat16* x16, float* x32, cudaStream_t s);
-cudaError_t launch_unpack(const float* y, long long P, const NormConsts& nc, double* rho, double* ux, double* uy,
-                          double* T, cudaStream_t s);
+cudaError_t launch_unpack(const float* y, int N, long long HW, const double* sums, const NormConsts& nc, double* rho,
+                          double* ux, double* uy, double* T, cudaStream_t s);
 
 // cnt[4]: liquid nodes (rho > mid), unphysical nodes, liquid-vapour edges
 // of the periodic W-wide image f [4][P], and nodes whose phase differs from

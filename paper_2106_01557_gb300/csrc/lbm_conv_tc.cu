@@ -102,9 +102,8 @@ struct TcCfg {
     static constexpr int EPI_CH = EPI_COLS / NC;        // tcgen05.ld per thread and row
     static constexpr int CPP = COUT / 4;                // 16-byte FP32 chunks per pixel in the tile
     static constexpr int SWZ = (CPP < 8 ? CPP : 8) - 1; // chunk swizzle mask
-    static constexpr int N16 = TC_TW * COUT / 8, N32 = TC_TW * COUT / 4;  // 16-byte output chunks of a row
+    static constexpr int N16 = TC_TW * COUT / 8;        // 16-byte BF16 output chunks of a row
     static constexpr int O16 = (N16 + TC_EPI_THREADS - 1) / TC_EPI_THREADS;  // BF16 chunks per thread
-    static constexpr int O32 = (N32 + TC_EPI_THREADS - 1) / TC_EPI_THREADS;  // FP32 chunks per thread
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && 3 * COUT <= 256, "tcgen05 f16 shape");
     static_assert((TMEM_COLS & (TMEM_COLS - 1)) == 0 && TC_NBLK >= 4, "accumulator blocks");
     static_assert(WDX % 1024 == 0, "swizzle atoms of the weights start on 1024-byte boundaries");
@@ -135,7 +134,7 @@ template <int CIN, int COUT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
               int N, int H, int W, int in_relu, const __nv_bfloat16* __restrict__ mask,
-              const __nv_bfloat16* __restrict__ res16, const float* __restrict__ res32, int res32_c,
+              const __nv_bfloat16* __restrict__ res16, const float* __restrict__ res32,
               __nv_bfloat16* __restrict__ out16, float* __restrict__ out32, int* __restrict__ status) {
     using Cf = TcCfg<CIN, COUT>;
     extern __shared__ unsigned char smem_raw[];
@@ -354,11 +353,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
                         for (int q = 0; q < 8; ++q) v[q] += __bfloat162float(rh[q]);
                     }
-                    if (res32) {
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (g8 * 8 + q < res32_c) v[q] += res32[(row0 + p) * res32_c + g8 * 8 + q];
-                    }
                     uint4 ov;
                     __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
@@ -366,19 +360,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     *reinterpret_cast<uint4*>(out16 + (row0 + p) * COUT + g8 * 8) = ov;
                 }
             } else {
-#pragma unroll
-                for (int j = 0; j < Cf::O32; ++j) {
-                    const int i = tid + j * TC_EPI_THREADS;
-                    const int p = i / (COUT / 4), k = i % (COUT / 4);
-                    if (i >= Cf::N32 || p >= nvalid) continue;
-                    float4 v = *reinterpret_cast<const float4*>(tile + p * COUT + 4 * (k ^ (p & Cf::SWZ)));
+                // the first four channels, one 16-byte chunk per pixel
+                if (tid < TC_TW && tid < nvalid) {
+                    const size_t p = row0 + tid;
+                    float4 v = *reinterpret_cast<const float4*>(tile + tid * COUT + 4 * (0 ^ (tid & Cf::SWZ)));
                     if (res32) {
-                        if (4 * k + 0 < res32_c) v.x += res32[(row0 + p) * res32_c + 4 * k + 0];
-                        if (4 * k + 1 < res32_c) v.y += res32[(row0 + p) * res32_c + 4 * k + 1];
-                        if (4 * k + 2 < res32_c) v.z += res32[(row0 + p) * res32_c + 4 * k + 2];
-                        if (4 * k + 3 < res32_c) v.w += res32[(row0 + p) * res32_c + 4 * k + 3];
+                        const float4 x = *reinterpret_cast<const float4*>(res32 + p * 4);
+                        v.x += x.x;
+                        v.y += x.y;
+                        v.z += x.z;
+                        v.w += x.w;
                     }
-                    *reinterpret_cast<float4*>(out32 + (row0 + p) * COUT + 4 * k) = v;
+                    *reinterpret_cast<float4*>(out32 + p * 4) = v;
                 }
             }
         };
@@ -692,7 +685,7 @@ cudaError_t conv_tc_t(const ConvArgs& a, cudaStream_t s, int sms, int* status) {
     const long long rows = (long long)a.N * a.H * ((a.W + TC_TW - 1) / TC_TW);
     const int grid = rows < sms ? (int)rows : sms;
     k_conv_tc<CIN, COUT><<<grid, TC_THREADS, Cf::BYTES, s>>>(a.in, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.mask,
-                                                             a.res16, a.res32, a.res32_c, a.out16, a.out32, status);
+                                                             a.res16, a.res32, a.out16, a.out32, status);
     return cudaGetLastError();
 }
 

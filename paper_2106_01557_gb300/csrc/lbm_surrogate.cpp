@@ -32,14 +32,11 @@ int sfail(int code, const std::string& m) { return lbm_internal_fail(code, m.c_s
 struct Layer {
     int cin, cout;            // padded channel counts (16 or C)
     int cin_real, cout_real;  // 4 or C
+    // in the flat arrays of all layers:
     float* w = nullptr;       // FP32 master [9][cout][cin]
     float* b = nullptr;       // [cout]
     float* gw = nullptr;
     float* gb = nullptr;
-    float* mw = nullptr;
-    float* vw = nullptr;
-    float* mb = nullptr;
-    float* vb = nullptr;
     __nv_bfloat16* w16 = nullptr;    // forward copy
     __nv_bfloat16* wflip = nullptr;  // [9][cin][cout], taps reversed: input gradient
     int nw() const { return 9 * cin * cout; }
@@ -51,6 +48,13 @@ struct lbm_surrogate {
     lbm_surrogate_config cfg;
     NormConsts nc;
     std::vector<Layer> layers;  // lift, (b1, b2) x B, proj
+    // parameters, their gradients and Adam moments, and the BF16 copies of all
+    // layers, each in one array: per layer the weights, then the biases
+    size_t nflat = 0;
+    float *theta = nullptr, *grad = nullptr, *mom1 = nullptr, *mom2 = nullptr;
+    __nv_bfloat16 *w16 = nullptr, *wflip = nullptr;
+    LayerDesc* d_layers = nullptr;
+    float* h_flat = nullptr;    // pinned, nflat
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int sms = 0;
@@ -58,7 +62,7 @@ struct lbm_surrogate {
     __nv_bfloat16* x16 = nullptr;  // [P][16]
     float* x32 = nullptr;          // [P][4]
     float* t32 = nullptr;          // [P][4] targets
-    float* y32 = nullptr;          // [P][16]
+    float* y32 = nullptr;          // [P][4]
     __nv_bfloat16* dy16 = nullptr; // [P][16]
     std::vector<__nv_bfloat16*> h;   // B + 1 activations [P][C]
     std::vector<__nv_bfloat16*> z1;  // B activations
@@ -110,7 +114,7 @@ static int ensure_acts(lbm_surrogate* s, long long P, bool train) {
     const int C = s->cfg.channels;
     const size_t a = (size_t)P * C * sizeof(__nv_bfloat16);
     bool ok = cudaMalloc(&s->x16, (size_t)P * 16 * 2) == cudaSuccess && cudaMalloc(&s->x32, (size_t)P * 4 * 4) == cudaSuccess &&
-              cudaMalloc(&s->t32, (size_t)P * 4 * 4) == cudaSuccess && cudaMalloc(&s->y32, (size_t)P * 16 * 4) == cudaSuccess &&
+              cudaMalloc(&s->t32, (size_t)P * 4 * 4) == cudaSuccess && cudaMalloc(&s->y32, (size_t)P * 4 * 4) == cudaSuccess &&
               cudaMalloc(&s->dy16, (size_t)P * 16 * 2) == cudaSuccess;
     const int nh = train ? s->cfg.blocks + 1 : 2;
     for (int i = 0; ok && i < nh; ++i) {
@@ -229,7 +233,6 @@ static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
     const Layer& proj = s->layers.back();
     a = cargs(train ? s->h[B] : s->h[B & 1], proj.w16, proj.b, N, H, W, 1);
     a.res32 = s->x32;
-    a.res32_c = 4;
     a.out32 = s->y32;
     CONV(C, 16, a);
     return LBM_OK;
@@ -239,10 +242,6 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
     const int B = s->cfg.blocks, C = s->cfg.channels;
     const bool tc = s->cfg.conv_path == 0;
     const long long P = (long long)N * H * W;
-    for (Layer& L : s->layers) {
-        SCK(cudaMemsetAsync(L.gw, 0, (size_t)L.nw() * 4, s->stream));
-        SCK(cudaMemsetAsync(L.gb, 0, (size_t)L.cout * 4, s->stream));
-    }
     // projection: its input is relu(h_B)
     Layer& proj = s->layers.back();
     WGRAD(C, 16, s->h[B], s->dy16, 1, proj.gw);
@@ -280,8 +279,8 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
     return LBM_OK;
 }
 
-// the mass-conserving output layer on y32 (with the targets: also the sums
-// the projected loss gradient needs)
+// the sums of the mass-conserving output layer on y32 (with the targets: also
+// those the projected loss gradient needs)
 static int mass_layer(lbm_surrogate* s, int N, long long HW, const float* t32) {
     if (!s->cfg.conserve_mass) return LBM_OK;
     if (N > s->msum_cap) {
@@ -340,19 +339,29 @@ int lbm_surrogate_create(const lbm_surrogate_config* cfg, lbm_surrogate** out) {
         s->layers.push_back({C, C, C, C});
     }
     s->layers.push_back({C, 16, C, 4});
+    std::vector<LayerDesc> desc;
+    size_t n16 = 0;
+    for (const Layer& L : s->layers) {
+        desc.push_back({L.cin, L.cout, L.cin_real, L.cout_real, (long long)s->nflat, (long long)n16});
+        s->nflat += (size_t)L.nw() + L.cout;  // multiples of 16 elements
+        n16 += (size_t)L.nw();
+    }
     bool ok = true;
-    for (Layer& L : s->layers) {
-        const size_t nw = (size_t)L.nw();
-        ok = ok && cudaMalloc(&L.w, nw * 4) == cudaSuccess && cudaMalloc(&L.gw, nw * 4) == cudaSuccess &&
-             cudaMalloc(&L.mw, nw * 4) == cudaSuccess && cudaMalloc(&L.vw, nw * 4) == cudaSuccess &&
-             cudaMalloc(&L.b, L.cout * 4) == cudaSuccess && cudaMalloc(&L.gb, L.cout * 4) == cudaSuccess &&
-             cudaMalloc(&L.mb, L.cout * 4) == cudaSuccess && cudaMalloc(&L.vb, L.cout * 4) == cudaSuccess &&
-             cudaMalloc(&L.w16, nw * 2) == cudaSuccess && cudaMalloc(&L.wflip, nw * 2) == cudaSuccess;
-        if (ok) {
-            cudaMemset(L.w, 0, nw * 4); cudaMemset(L.mw, 0, nw * 4); cudaMemset(L.vw, 0, nw * 4);
-            cudaMemset(L.b, 0, L.cout * 4); cudaMemset(L.mb, 0, L.cout * 4); cudaMemset(L.vb, 0, L.cout * 4);
-            cudaMemset(L.w16, 0, nw * 2); cudaMemset(L.wflip, 0, nw * 2);
-        }
+    for (float** q : {&s->theta, &s->grad, &s->mom1, &s->mom2})
+        ok = ok && cudaMalloc(q, s->nflat * 4) == cudaSuccess && cudaMemset(*q, 0, s->nflat * 4) == cudaSuccess;
+    for (__nv_bfloat16** q : {&s->w16, &s->wflip})
+        ok = ok && cudaMalloc(q, n16 * 2) == cudaSuccess && cudaMemset(*q, 0, n16 * 2) == cudaSuccess;
+    ok = ok && cudaMalloc(&s->d_layers, desc.size() * sizeof(LayerDesc)) == cudaSuccess &&
+         cudaMemcpy(s->d_layers, desc.data(), desc.size() * sizeof(LayerDesc), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMallocHost(&s->h_flat, s->nflat * 4) == cudaSuccess;
+    for (size_t i = 0; ok && i < desc.size(); ++i) {
+        Layer& L = s->layers[i];
+        L.w = s->theta + desc[i].off;
+        L.b = L.w + L.nw();
+        L.gw = s->grad + desc[i].off;
+        L.gb = L.gw + L.nw();
+        L.w16 = s->w16 + desc[i].off16;
+        L.wflip = s->wflip + desc[i].off16;
     }
     ok = ok && cudaMalloc(&s->d_loss, sizeof(double)) == cudaSuccess &&
          cudaMalloc(&s->d_lpart, MSE_BLOCKS * sizeof(double)) == cudaSuccess &&
@@ -375,55 +384,63 @@ int64_t lbm_surrogate_num_params(const lbm_surrogate* s) {
     return n;
 }
 
-// parameter order <-> padded device layout
-static int copy_params(lbm_surrogate* s, float* host, bool to_device, bool grads) {
-    size_t off = 0;
-    for (Layer& L : s->layers) {
-        std::vector<float> wpad((size_t)L.nw()), bpad((size_t)L.cout);
-        if (!to_device) {
-            SCK(cudaMemcpy(wpad.data(), grads ? L.gw : L.w, wpad.size() * 4, cudaMemcpyDeviceToHost));
-            SCK(cudaMemcpy(bpad.data(), grads ? L.gb : L.b, bpad.size() * 4, cudaMemcpyDeviceToHost));
-        } else {
-            std::fill(wpad.begin(), wpad.end(), 0.f);
-            std::fill(bpad.begin(), bpad.end(), 0.f);
+// the caller's parameter order <-> the padded flat layout (h_flat)
+static void pad_params(lbm_surrogate* s, float* host, bool to_flat) {
+    size_t off = 0, at = 0;
+    for (const Layer& L : s->layers) {
+        float* w = s->h_flat + at;
+        for (int r = 0; r < 9 * L.cout; ++r) {
+            const int o = r % L.cout;
+            float* row = w + (size_t)r * L.cin;
+            if (o >= L.cout_real) {
+                if (to_flat) std::fill(row, row + L.cin, 0.f);
+                continue;
+            }
+            if (to_flat) {
+                std::memcpy(row, host + off, L.cin_real * sizeof(float));
+                std::fill(row + L.cin_real, row + L.cin, 0.f);
+            } else {
+                std::memcpy(host + off, row, L.cin_real * sizeof(float));
+            }
+            off += L.cin_real;
         }
-        for (int t = 0; t < 9; ++t)
-            for (int o = 0; o < L.cout_real; ++o)
-                for (int i = 0; i < L.cin_real; ++i) {
-                    float& dev = wpad[((size_t)t * L.cout + o) * L.cin + i];
-                    float& hv = host[off + ((size_t)t * L.cout_real + o) * L.cin_real + i];
-                    if (to_device) dev = hv; else hv = dev;
-                }
-        off += 9ull * L.cout_real * L.cin_real;
-        for (int o = 0; o < L.cout_real; ++o) {
-            if (to_device) bpad[o] = host[off + o]; else host[off + o] = bpad[o];
+        float* b = w + L.nw();
+        if (to_flat) {
+            std::fill(b, b + L.cout, 0.f);
+            std::memcpy(b, host + off, L.cout_real * sizeof(float));
+        } else {
+            std::memcpy(host + off, b, L.cout_real * sizeof(float));
         }
         off += L.cout_real;
-        if (to_device) {
-            SCK(cudaMemcpy(L.w, wpad.data(), wpad.size() * 4, cudaMemcpyHostToDevice));
-            SCK(cudaMemcpy(L.b, bpad.data(), bpad.size() * 4, cudaMemcpyHostToDevice));
-            SCK(launch_refresh(L.w, L.cin, L.cout, L.cin_real, L.cout_real, L.w16, L.wflip, s->stream));
-        }
+        at += (size_t)L.nw() + L.cout;
     }
+}
+
+// one flat array (parameters or gradients) in the caller's order
+static int read_flat(lbm_surrogate* s, const float* dev, float* host) {
+    SCK(cudaMemcpyAsync(s->h_flat, dev, s->nflat * 4, cudaMemcpyDeviceToHost, s->stream));
     SCK(cudaStreamSynchronize(s->stream));
+    pad_params(s, host, false);
     return LBM_OK;
 }
 
 int lbm_surrogate_set_params(lbm_surrogate* s, const float* params) {
     if (!s || !params) return sfail(LBM_ERR_ARG, "null argument");
     s->step_count = 0;
-    for (Layer& L : s->layers) {
-        SCK(cudaMemset(L.mw, 0, (size_t)L.nw() * 4));
-        SCK(cudaMemset(L.vw, 0, (size_t)L.nw() * 4));
-        SCK(cudaMemset(L.mb, 0, (size_t)L.cout * 4));
-        SCK(cudaMemset(L.vb, 0, (size_t)L.cout * 4));
-    }
-    return copy_params(s, const_cast<float*>(params), true, false);
+    SCK(cudaStreamSynchronize(s->stream));
+    pad_params(s, const_cast<float*>(params), true);
+    SCK(cudaMemsetAsync(s->mom1, 0, s->nflat * 4, s->stream));
+    SCK(cudaMemsetAsync(s->mom2, 0, s->nflat * 4, s->stream));
+    SCK(cudaMemcpyAsync(s->theta, s->h_flat, s->nflat * 4, cudaMemcpyHostToDevice, s->stream));
+    SCK(launch_adam_refresh(s->d_layers, (int)s->layers.size(), s->theta, s->mom1, s->mom2, s->grad, s->w16, s->wflip, 0, 0.f,
+                            0.f, 0.f, 0.f, 1.f, 1.f, s->stream));
+    SCK(cudaStreamSynchronize(s->stream));
+    return LBM_OK;
 }
 
 int lbm_surrogate_get_params(lbm_surrogate* s, float* params) {
     if (!s || !params) return sfail(LBM_ERR_ARG, "null argument");
-    return copy_params(s, params, false, false);
+    return read_flat(s, s->theta, params);
 }
 
 static int check_dims(int N, int H, int W) {
@@ -444,7 +461,8 @@ int lbm_surrogate_forward(lbm_surrogate* s, const double* in, int32_t N, int32_t
     if (rc) return rc;
     rc = mass_layer(s, N, (long long)H * W, nullptr);
     if (rc) return rc;
-    SCK(launch_unpack(s->y32, P, s->nc, out, out + P, out + 2 * P, out + 3 * P, s->stream));
+    SCK(launch_unpack(s->y32, N, (long long)H * W, s->cfg.conserve_mass ? s->d_msum : nullptr, s->nc, out, out + P,
+                      out + 2 * P, out + 3 * P, s->stream));
     SCK(cudaStreamSynchronize(s->stream));
     return check_status(s);
 }
@@ -456,15 +474,14 @@ static int loss_and_backward(lbm_surrogate* s, const double* in, const double* t
     if (rc) return rc;
     rc = pack_inputs(s, in, P, s->x32, s->x16);
     if (rc) return rc;
-    // targets: the normalised 4 fields (the BF16 copy is scratch)
-    SCK(launch_pack(target, target + P, target + 2 * P, target + 3 * P, P, s->nc, s->dy16, s->t32, s->stream));
+    // targets: the normalised 4 fields
+    SCK(launch_pack(target, target + P, target + 2 * P, target + 3 * P, P, s->nc, nullptr, s->t32, s->stream));
     rc = run_forward(s, N, H, W, true);
     if (rc) return rc;
     rc = mass_layer(s, N, (long long)H * W, s->t32);
     if (rc) return rc;
-    SCK(cudaMemsetAsync(s->d_loss, 0, sizeof(double), s->stream));
-    SCK(launch_mse(s->y32, s->t32, P, s->dy16, s->d_loss, s->cfg.conserve_mass ? s->d_msum + N : nullptr,
-                   (long long)H * W, s->d_lpart, s->stream));
+    SCK(launch_mse(s->y32, s->t32, N, (long long)H * W, s->dy16, s->d_loss, s->cfg.conserve_mass ? s->d_msum : nullptr,
+                   s->d_lpart, s->stream));
     rc = run_backward(s, N, H, W);
     if (rc) return rc;
     if (loss) {
@@ -481,7 +498,7 @@ int lbm_surrogate_loss_grad(lbm_surrogate* s, const double* in, const double* ta
     if (rc) return rc;
     rc = loss_and_backward(s, in, target, N, H, W, loss);
     if (rc) return rc;
-    if (grads) return copy_params(s, grads, false, true);
+    if (grads) return read_flat(s, s->grad, grads);
     return LBM_OK;
 }
 
@@ -496,11 +513,8 @@ int lbm_surrogate_train_step(lbm_surrogate* s, const double* in, const double* t
     s->step_count += 1;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float c1 = 1.f - std::pow(b1, (float)s->step_count), c2 = 1.f - std::pow(b2, (float)s->step_count);
-    for (Layer& L : s->layers) {
-        SCK(launch_adam(L.w, L.mw, L.vw, L.gw, L.nw(), (float)lr, b1, b2, eps, c1, c2, s->stream));
-        SCK(launch_adam(L.b, L.mb, L.vb, L.gb, L.cout, (float)lr, b1, b2, eps, c1, c2, s->stream));
-        SCK(launch_refresh(L.w, L.cin, L.cout, L.cin_real, L.cout_real, L.w16, L.wflip, s->stream));
-    }
+    SCK(launch_adam_refresh(s->d_layers, (int)s->layers.size(), s->theta, s->mom1, s->mom2, s->grad, s->w16, s->wflip, 1,
+                            (float)lr, b1, b2, eps, c1, c2, s->stream));
     SCK(cudaStreamSynchronize(s->stream));
     return LBM_OK;
 }
@@ -671,10 +685,9 @@ int lbm_surrogate_rollout(lbm_surrogate* s, lbm_handle* h, int32_t njumps, int32
 int lbm_surrogate_destroy(lbm_surrogate* s) {
     if (!s) return LBM_OK;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    for (Layer& L : s->layers) {
-        s_free(L.w); s_free(L.b); s_free(L.gw); s_free(L.gb); s_free(L.mw); s_free(L.vw); s_free(L.mb);
-        s_free(L.vb); s_free(L.w16); s_free(L.wflip);
-    }
+    s_free(s->theta); s_free(s->grad); s_free(s->mom1); s_free(s->mom2); s_free(s->w16); s_free(s->wflip);
+    s_free(s->d_layers);
+    if (s->h_flat) cudaFreeHost(s->h_flat);
     release_acts(s);
     s_free(s->d_loss); s_free(s->d_cnt); s_free(s->d_status); s_free(s->d_msum); s_free(s->d_mpart); s_free(s->d_lpart); s_free(s->gpart); s_free(s->fields); s_free(s->pred); s_free(s->ver); s_free(s->d_chg); s_free(s->snapshot);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
