@@ -207,7 +207,9 @@ __global__ void __launch_bounds__(WT)
     const int g = lane / 4, t = lane % 4;
     const int dy = (int)blockIdx.y - 1;
     const int tiles_x = (W + WCH - 1) / WCH;
-    const long long nchunks = (long long)N * H * tiles_x;
+    // this block's run of the input rows of all strips, strip after strip
+    const long long rows = (long long)N * H * tiles_x;
+    const long long r_begin = rows * blockIdx.x / gridDim.x, r_end = rows * (blockIdx.x + 1) / gridDim.x;
     const int mt = warp % Cf::MT, nt0 = (warp / Cf::MT) * Cf::NPW;
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(wg_smem);
     float acc[3][Cf::NPW][4];
@@ -218,14 +220,14 @@ __global__ void __launch_bounds__(WT)
 
     // copy chunk ch into stage st (one commit group per call, empty past the end)
     auto load = [&](long long ch, int st) {
-        if (ch < nchunks) {
-            const int x0 = (int)(ch % tiles_x) * WCH;
-            const long long ry = ch / tiles_x;  // n * H + y
-            const int y = (int)(ry % H), n = (int)(ry / H);
-            int yy = y + dy;
-            yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+        if (ch < r_end) {
+            const int yy = (int)(ch % H);  // input row
+            const long long strip = ch / H;
+            const int x0 = (int)(strip % tiles_x) * WCH, n = (int)(strip / tiles_x);
+            int y = yy - dy;  // dOut row
+            y = y < 0 ? y + H : (y >= H ? y - H : y);
             const uint32_t sd = sbase + st * Cf::STAGE, sx = sd + Cf::D_BYTES;
-            const __nv_bfloat16* drow = dout + (size_t)ry * W * COUT;
+            const __nv_bfloat16* drow = dout + ((size_t)n * H + y) * W * COUT;
             const __nv_bfloat16* xrow = in + ((size_t)n * H + yy) * W * CIN;
             for (int e = tid; e < WCH * (COUT / 8); e += WT) {
                 const int px = e / (COUT / 8), c8 = e % (COUT / 8);
@@ -255,11 +257,11 @@ __global__ void __launch_bounds__(WT)
         }
     };
 
-    long long ch = blockIdx.x;
+    long long ch = r_begin;
     load(ch, 0);
-    for (int it = 0; ch < nchunks; ch += gridDim.x, ++it) {
+    for (int it = 0; ch < r_end; ++ch, ++it) {
         const int st = it & 1;
-        load(ch + gridDim.x, st ^ 1);
+        load(ch + 1, st ^ 1);
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         if (in_relu) relu_tile(st);
         __syncthreads();
@@ -305,8 +307,22 @@ __global__ void __launch_bounds__(WT)
 // dw[tp][co][ci] = the sum over blocks of the partials, tap tp = 3 (dy + 1) +
 // dx + 1, four weights per thread: thread row ty adds blocks ty, ty + 8, ... in
 // that order, then the eight rows are added in order (a fixed order).
-__global__ void __launch_bounds__(256) k_wgrad_sum(const float4* __restrict__ part, int nblk, int n4, float4* __restrict__ dw) {
+// The last block, where there is a bias gradient, adds its partials [nblk][64]
+// the same way: row j of four adds blocks j, j + 4, ...
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float4* __restrict__ part, int nblk, int n4, float4* __restrict__ dw,
+                                                   const float* __restrict__ bpart, float* __restrict__ db) {
     __shared__ float4 s[8][32];
+    if (db && blockIdx.x == gridDim.x - 1) {
+        float* t = reinterpret_cast<float*>(s);
+        const int c = threadIdx.x % 64, j = threadIdx.x / 64;
+        float a = 0.f;
+#pragma unroll 4
+        for (int b = j; b < nblk; b += 4) a += __ldcg(bpart + (size_t)b * 64 + c);
+        t[threadIdx.x] = a;
+        __syncthreads();
+        if (j == 0) db[c] = ((a + t[64 + c]) + t[128 + c]) + t[192 + c];
+        return;
+    }
     const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
     const int e = blockIdx.x * 32 + tx;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -360,6 +376,39 @@ __global__ void k_bgrad(const __nv_bfloat16* __restrict__ dout, long long P, int
         float t = 0.f;
         for (int k = 0; k < per; ++k) t += s[k * G8 + g8][q];
         part[(size_t)blockIdx.x * C + c] = t;
+    }
+}
+
+// The same of 64 channels, over the blocks' runs of rows and in the order in
+// which k_wgrad64 sums it (128 threads: 8 channels of pixels sub, sub + 16, ...).
+__global__ void __launch_bounds__(128) k_bgrad64(const __nv_bfloat16* __restrict__ dout, int N, int H, int W, float* __restrict__ part) {
+    __shared__ float s[16][64];
+    const int c8 = threadIdx.x % 8, sub = threadIdx.x / 8;
+    const int tiles_x = (W + WCH - 1) / WCH;
+    const long long rows = (long long)N * H * tiles_x;
+    const long long r_end = rows * (blockIdx.x + 1) / gridDim.x;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (long long r = rows * blockIdx.x / gridDim.x; r < r_end; ++r) {
+        const long long strip = r / H;
+        const int x0 = (int)(strip % tiles_x) * WCH;
+        const __nv_bfloat16* row = dout + ((strip / tiles_x * H + r % H) * W + x0) * 64 + c8 * 8;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int px = sub + 16 * i;
+            if (x0 + px >= W) break;
+            const uint4 v = *reinterpret_cast<const uint4*>(row + (size_t)px * 64);
+            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] += __bfloat162float(h[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s[sub][c8 * 8 + c] = acc[c];
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        float t = 0.f;
+        for (int j = 0; j < 16; ++j) t += s[j][threadIdx.x];
+        part[(size_t)blockIdx.x * 64 + threadIdx.x] = t;
     }
 }
 
@@ -654,12 +703,14 @@ cudaError_t wgrad_t(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, i
         set = true;
     }
     const long long chunks = (long long)N * H * ((W + WCH - 1) / WCH);
-    long long gx = (2 * sms) / 3;  // with the three filter rows: two CTAs per SM, as in the tcgen05 path
+    // with the three filter rows two CTAs per SM; the 64 -> 64 layers' rows are
+    // split as the tcgen05 path splits them
+    long long gx = CIN == 64 && COUT == 64 ? wgrad64_blocks(N, H, W, sms) : (2 * sms) / 3;
     if (gx > chunks) gx = chunks;
     if (gx < 1) gx = 1;
     k_wgrad<CIN, COUT><<<dim3((unsigned)gx, 3), WT, 2 * Cf::STAGE, s>>>(in, dout, N, H, W, in_relu, part);
     const cudaError_t e = cudaGetLastError();
-    return e != cudaSuccess ? e : launch_wgrad_sum(part, (int)gx, COUT * CIN, dw, s);
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, (int)gx, COUT * CIN, dw, nullptr, nullptr, s);
 }
 
 }  // namespace
@@ -713,8 +764,7 @@ cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, in
 }
 
 size_t grad_scratch_floats(int sms) {
-    const size_t gx = (size_t)(2 * sms + 2) / 3;
-    const size_t w = gx * 9 * 64 * 64, b = (size_t)608 * 256;
+    const size_t w = (size_t)sms * (9 * 64 * 64 + 64), b = (size_t)608 * 256;
     return w > b ? w : b;
 }
 
@@ -726,13 +776,24 @@ cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, cudaStream_t s) {
-    if (nblk < 1 || cc < 1) return cudaErrorInvalidValue;
-    if (cc % 4 != 0) return cudaErrorInvalidValue;
+cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, cudaStream_t s) {
+    if (nblk < 1 || cc < 0 || cc % 4 != 0 || (cc == 0 && !db)) return cudaErrorInvalidValue;
     const int n4 = 9 * cc / 4;
-    k_wgrad_sum<<<(n4 + 31) / 32, 256, 0, s>>>(reinterpret_cast<const float4*>(part), nblk, n4,
-                                              reinterpret_cast<float4*>(dw));
+    k_wgrad_sum<<<(n4 + 31) / 32 + (db ? 1 : 0), 256, 0, s>>>(reinterpret_cast<const float4*>(part), nblk, n4,
+                                                             reinterpret_cast<float4*>(dw), bpart, db);
     return cudaGetLastError();
+}
+
+int wgrad64_blocks(int N, int H, int W, int sms) {
+    const long long rows = (long long)N * H * ((W + WCH - 1) / WCH);
+    return rows < sms ? (int)rows : sms;
+}
+
+cudaError_t launch_bgrad64(const __nv_bfloat16* dout, int N, int H, int W, float* db, float* part, cudaStream_t s, int sms) {
+    const int g = wgrad64_blocks(N, H, W, sms);
+    k_bgrad64<<<g, 128, 0, s>>>(dout, N, H, W, part);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, g, 0, nullptr, part, db, s);
 }
 
 cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* db, float* part, cudaStream_t s) {

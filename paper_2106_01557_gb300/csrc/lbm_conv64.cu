@@ -44,18 +44,16 @@
 #include <mutex>
 
 #include "lbm_conv.h"
+#include "lbm_conv64.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_tc.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int C6_W = 128;                  // pixels per output row segment (MMA M)
 constexpr int C6_SLOTS = 4;                // input-row ring
 constexpr int C6_BLK = 8;                  // accumulator blocks in tensor memory
 constexpr int C6_THREADS = 512;
-constexpr int C6_SLOT = (C6_W + 16) * 128;  // 8 halo pixels on each side
-constexpr int C6_ROW = C6_W * 128;          // a staged row
 constexpr int C6_WDX = 3 * 64 * 128;        // weights of one dx
 constexpr int C6_OFF_IN = 3 * C6_WDX;
 constexpr int C6_OFF_OUT = C6_OFF_IN + C6_SLOTS * C6_SLOT;
@@ -65,39 +63,6 @@ static_assert(C6_BYTES <= 227 * 1024 && C6_SLOT % 1024 == 0 && C6_WDX % 1024 == 
 struct C6Maps {
     CUtensorMap in, in8, out, out8, res, res8;  // boxes of 128 and of 8 pixels
 };
-
-__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* tm, int x, int row, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(tm)), "r"(0), "r"(x), "r"(row), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void tma_store(const CUtensorMap* tm, int x, int row, uint32_t src) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                     reinterpret_cast<uint64_t>(tm)),
-                 "r"(0), "r"(x), "r"(row), "r"(src)
-                 : "memory");
-}
-
-// Wait for a phase of bar, bounded; false after the bound, or once another
-// role has given up (dead is set for all).
-__device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*dead || globaltimer_ns() - t0 > WAIT_NS) {
-            *dead = 1;
-            return false;
-        }
-    }
-    return true;
-}
-
-// the same for a converged warp: one outcome for all lanes
-__device__ __forceinline__ bool role_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
-    return __all_sync(0xffffffffu, role_wait(bar, parity, dead));
-}
 
 __global__ void __launch_bounds__(C6_THREADS, 1)
     k_conv64(const __grid_constant__ C6Maps tm, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
@@ -157,24 +122,10 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
     __syncthreads();
     tc_fence_after();
 
-    const int tiles_x = (W + C6_W - 1) / C6_W;
-    const long long rows_total = (long long)N * tiles_x * H;
-    const long long r_begin = rows_total * blockIdx.x / gridDim.x, r_end = rows_total * (blockIdx.x + 1) / gridDim.x;
-    // the CTA's runs: rows y0 .. y0 + L - 1 of a strip starting at x0 with nv
-    // pixels in image n; q0 input rows and t0 output rows came before
-    struct Run {
-        int y0, L, x0, nv, n;
-    };
-    auto run_at = [&](long long r) {
-        Run u;
-        u.y0 = (int)(r % H);
-        const long long strip = r / H;
-        u.x0 = (int)(strip % tiles_x) * C6_W;
-        u.n = (int)(strip / tiles_x);
-        u.L = (int)((long long)(H - u.y0) < r_end - r ? (long long)(H - u.y0) : r_end - r);
-        u.nv = W - u.x0 < C6_W ? W - u.x0 : C6_W;
-        return u;
-    };
+    const StripRuns R(N, H, W);
+    const long long r_begin = R.rows * blockIdx.x / gridDim.x, r_end = R.rows * (blockIdx.x + 1) / gridDim.x;
+    using Run = StripRun;
+    auto run_at = [&](long long r) { return R.at(r, r_end); };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -190,26 +141,20 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
                         ok = false;
                         break;
                     }
-                    int gy = u.y0 - 1 + li;
-                    gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
-                    const int row = u.n * H + gy;
+                    const int row = u.n * H + R.wrap(u.y0 - 1 + li);
                     const uint32_t dst = sbase + C6_OFF_IN + s * C6_SLOT;
                     mbar_arrive_expect_tx(&full[s], (uint32_t)(u.nv + 16) * 128u);
-                    tma_load(dst, &tm.in8, xl, row, &full[s]);
+                    tma_load_rows(dst, &tm.in8, xl, row, &full[s]);
                     if (u.nv == C6_W) {
-                        tma_load(dst + 1024, &tm.in, u.x0, row, &full[s]);
+                        tma_load_rows(dst + 1024, &tm.in, u.x0, row, &full[s]);
                     } else {
-                        for (int x = 0; x < u.nv; x += 8) tma_load(dst + 1024 + x * 128, &tm.in8, u.x0 + x, row, &full[s]);
+                        for (int x = 0; x < u.nv; x += 8) tma_load_rows(dst + 1024 + x * 128, &tm.in8, u.x0 + x, row, &full[s]);
                     }
-                    tma_load(dst + 1024 + u.nv * 128, &tm.in8, xr, row, &full[s]);
+                    tma_load_rows(dst + 1024 + u.nv * 128, &tm.in8, xr, row, &full[s]);
                 }
             }
             // every copy issued lands before the shared memory is given up
-            for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) {
-                const unsigned p = q - 1 - j;
-                const uint64_t t1 = globaltimer_ns();
-                while (!mbar_try_wait(&full[p % C6_SLOTS], (p / C6_SLOTS) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
-            }
+            for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) land(&full[(q - 1 - j) % C6_SLOTS], ((q - 1 - j) / C6_SLOTS) & 1u);
         }
     } else if (warp == 1) {
         // The whole warp walks the rows, so that descriptors and addresses are
@@ -272,11 +217,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
             t0 += u.L;
         }
         // the MMAs issued are done with the slots before the block ends
-        for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) {
-            const unsigned p = q - 1 - j;
-            const uint64_t t1 = globaltimer_ns();
-            while (!mbar_try_wait(&empty[p % C6_SLOTS], (p / C6_SLOTS) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
-        }
+        for (unsigned j = 0; j < C6_SLOTS && j < q; ++j) land(&empty[(q - 1 - j) % C6_SLOTS], ((q - 1 - j) / C6_SLOTS) & 1u);
     } else if (warp >= 12) {
         if (in_relu) {
             const int rt = tid - 12 * 32;
@@ -344,9 +285,9 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
             const uint32_t dst = sbase + stage(k);
             mbar_arrive_expect_tx(bar, (uint32_t)d.u.nv * 128u);
             if (d.u.nv == C6_W) {
-                tma_load(dst, &tm.res, d.u.x0, row, bar);
+                tma_load_rows(dst, &tm.res, d.u.x0, row, bar);
             } else {
-                for (int x = 0; x < d.u.nv; x += 8) tma_load(dst + x * 128, &tm.res8, d.u.x0 + x, row, bar);
+                for (int x = 0; x < d.u.nv; x += 8) tma_load_rows(dst + x * 128, &tm.res8, d.u.x0 + x, row, bar);
             }
         };
         unsigned k = 0, brought = 0;  // rows of the group done; residuals asked for (leader)
@@ -432,9 +373,9 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
                 const int row = c.u.n * H + c.u.y0 + c.t;
                 const uint32_t src = sbase + stage(k);
                 if (c.u.nv == C6_W) {
-                    tma_store(&tm.out, c.u.x0, row, src);
+                    tma_store_rows(&tm.out, c.u.x0, row, src);
                 } else {
-                    for (int x = 0; x < c.u.nv; x += 8) tma_store(&tm.out8, c.u.x0 + x, row, src + x * 128);
+                    for (int x = 0; x < c.u.nv; x += 8) tma_store_rows(&tm.out8, c.u.x0 + x, row, src + x * 128);
                 }
                 bulk_commit();
             }
@@ -443,10 +384,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
         }
         if (leader) {
             // after a wait that ran out: the residuals still in flight
-            for (unsigned j = k; j < brought; ++j) {
-                const uint64_t t1 = globaltimer_ns();
-                while (!mbar_try_wait(&side[grp][j & 1u], (j >> 1) & 1u) && globaltimer_ns() - t1 < WAIT_NS) {}
-            }
+            for (unsigned j = k; j < brought; ++j) land(&side[grp][j & 1u], (j >> 1) & 1u);
             bulk_wait_all();
         }
     }
@@ -496,7 +434,6 @@ EncodeTiled get_encoder() {
 
 }  // namespace
 
-// [rows][W][64] BF16: boxes of `px` pixels of one row, 128-byte swizzle
 cudaError_t encode_rows64(const void* base, long long rows, int W, int px, CUtensorMap* m) {
     EncodeTiled enc = get_encoder();
     if (!enc) return cudaErrorNotSupported;

@@ -167,21 +167,27 @@ static int conv(lbm_surrogate* s, int cin, int cout, const ConvArgs& a) {
     return LBM_OK;
 }
 
-// weight gradient: the 64 -> 64 layers on tcgen05 with the tensor-core path
-static int wgrad(lbm_surrogate* s, int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N,
-                 int H, int W, int relu, float* gw) {
-    if (s->cfg.conv_path == 0 && cin == 64 && cout == 64) {
-        SCK(launch_wgrad_tc(cin, cout, in, dout, N, H, W, relu, gw, s->gpart, s->stream, s->sms, s->d_status));
-    } else {
-        SCK(launch_wgrad(cin, cout, in, dout, N, H, W, relu, gw, s->gpart, s->stream, s->sms));
+// weight and bias gradients of a layer
+static int wgrad(lbm_surrogate* s, const Layer& L, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
+                 int relu) {
+    if (L.cin == 64 && L.cout == 64) {
+        if (s->cfg.conv_path == 0) {
+            SCK(launch_wgrad64(in, dout, N, H, W, relu, L.gw, L.gb, s->gpart, s->stream, s->sms, s->d_status));
+            return LBM_OK;
+        }
+        SCK(launch_wgrad(64, 64, in, dout, N, H, W, relu, L.gw, s->gpart, s->stream, s->sms));
+        SCK(launch_bgrad64(dout, N, H, W, L.gb, s->gpart, s->stream, s->sms));
+        return LBM_OK;
     }
+    SCK(launch_wgrad(L.cin, L.cout, in, dout, N, H, W, relu, L.gw, s->gpart, s->stream, s->sms));
+    SCK(launch_bgrad(dout, (long long)N * H * W, L.cout, L.gb, s->gpart, s->stream));
     return LBM_OK;
 }
 
-#define WGRAD(cin, cout, in, dout, relu, gw)                          \
-    do {                                                              \
-        int rc_ = wgrad(s, cin, cout, in, dout, N, H, W, relu, gw);   \
-        if (rc_) return rc_;                                          \
+#define WGRAD(L, in, dout, relu)                          \
+    do {                                                  \
+        int rc_ = wgrad(s, L, in, dout, N, H, W, relu);   \
+        if (rc_) return rc_;                              \
     } while (0)
 
 #define CONV(cin, cout, a)                \
@@ -244,8 +250,7 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
     const long long P = (long long)N * H * W;
     // projection: its input is relu(h_B)
     Layer& proj = s->layers.back();
-    WGRAD(C, 16, s->h[B], s->dy16, 1, proj.gw);
-    SCK(launch_bgrad(s->dy16, P, 16, proj.gb, s->gpart, s->stream));
+    WGRAD(proj, s->h[B], s->dy16, 1);
     ConvArgs a = cargs(s->dy16, proj.wflip, nullptr, N, H, W, 0);
     a.mask = s->h[B];
     a.out16 = s->g0;  // d h_B
@@ -256,15 +261,13 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
         Layer& L1 = s->layers[1 + 2 * b];
         Layer& L2 = s->layers[2 + 2 * b];
         // h_{b+1} = h_b + conv2(relu(z1)); d z2 = d h_{b+1}
-        WGRAD(C, C, s->z1[b], dh, s->cfg.conv_path != 0, L2.gw);
-        SCK(launch_bgrad(dh, P, C, L2.gb, s->gpart, s->stream));
+        WGRAD(L2, s->z1[b], dh, !tc);
         a = cargs(dh, L2.wflip, nullptr, N, H, W, 0);
         if (tc) a.mbits = s->zbits + b * P;
         else a.mask = s->z1[b];
         a.out16 = s->g1;  // d z1
         CONV(C, C, a);
-        WGRAD(C, C, s->h[b], s->g1, 1, L1.gw);
-        SCK(launch_bgrad(s->g1, P, C, L1.gb, s->gpart, s->stream));
+        WGRAD(L1, s->h[b], s->g1, 1);
         a = cargs(s->g1, L1.wflip, nullptr, N, H, W, 0);
         if (tc) a.mbits = s->hbits + b * P;
         else a.mask = s->h[b];
@@ -274,8 +277,7 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
         std::swap(dh, spare);
     }
     Layer& lift = s->layers[0];
-    WGRAD(16, C, s->x16, dh, 0, lift.gw);
-    SCK(launch_bgrad(dh, P, C, lift.gb, s->gpart, s->stream));
+    WGRAD(lift, s->x16, dh, 0);
     return LBM_OK;
 }
 

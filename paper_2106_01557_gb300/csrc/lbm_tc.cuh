@@ -23,6 +23,14 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
            (2ull << 61);
 }
 
+// MN-major operand in 128-byte swizzled rows (one row per K index): atoms of
+// 8 K rows (SBO = 1024 bytes); lbo: byte offset between the 64-wide halves
+// along M or N; swizzle mode 2 (bits 61-63)
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
+           ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+
 __device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
