@@ -2,7 +2,7 @@
 // temperature advance together, one launch per time step. Every warp marches
 // the rows of its list of items (case, strip, rows) with the engine of
 // lbm_march.cuh; the host deals the items so that the warps of one wave of
-// resident blocks get equal work. A case's constants (temperature-dependent
+// resident blocks get equal work, neighbouring strips to neighbouring warps. A case's constants (temperature-dependent
 // c, dt, c_s, G^2/c, rho_v/rho_l, C_ref, shift) and geometry are copied into
 // the warp's shared memory when an item starts.
 // Per-item FP32 partial sums of the conservation record go to a table from
@@ -14,13 +14,25 @@ namespace lbm {
 
 namespace {
 
+// Warps per block and blocks per SM. A case's constants come from shared
+// memory instead of the launch's constant bank, so a warp needs registers for
+// them: with the 168 of three blocks per SM the 16-bit form spills (256 boxes
+// of 64 to 512 a side, FP16 storage: 445 us per step with 12 warps per SM, 342
+// with 8, 500 with 9 or 10, which share the four schedulers unevenly).
 template <class S>
-__global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS) k_batch_step(const BatchLaunch B, int from, const S* __restrict__ arena_in, S* __restrict__ arena_out) {
+struct BatchCfg {
+    static constexpr int W = 4;
+    static constexpr int BPS = sizeof(S) == 2 ? 2 : 4;
+};
+
+template <class S>
+__global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch_step(const BatchLaunch B, int from, const S* __restrict__ arena_in, S* __restrict__ arena_out) {
     using Cf = MarchCfg<S>;
     using V = typename std::conditional<Cf::NPL == 2, F2, float>::type;
-    __shared__ BatchCase s_case[MW];
+    constexpr int W = BatchCfg<S>::W;
+    __shared__ BatchCase s_case[W];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int gw = blockIdx.x * MW + warp;
+    const int gw = blockIdx.x * W + warp;
     if (blockIdx.x == 0 && threadIdx.x == 0) B.steps[1 - from] = __ldcg(&B.steps[from]) + 1.0;
     if (gw >= B.warps) return;
     BatchCase& cs = s_case[warp];
@@ -88,14 +100,14 @@ __global__ void k_batch_case_record(const BatchItem* __restrict__ items, int nit
 
 template <class S>
 cudaError_t launch_bt(const BatchLaunch& B, int from, const void* in, void* out, cudaStream_t s) {
-    k_batch_step<S><<<(B.warps + MW - 1) / MW, 32 * MW, 0, s>>>(B, from, static_cast<const S*>(in), static_cast<S*>(out));
+    k_batch_step<S><<<(B.warps + BatchCfg<S>::W - 1) / BatchCfg<S>::W, 32 * BatchCfg<S>::W, 0, s>>>(B, from, static_cast<const S*>(in), static_cast<S*>(out));
     return cudaGetLastError();
 }
 
 }  // namespace
 
 int batch_warps(int storage, int sms) {
-    return MW * sms * (storage == S_F32 ? MarchCfg<float>::BPS : MarchCfg<__half>::BPS);
+    return sms * (storage == S_F32 ? BatchCfg<float>::W * BatchCfg<float>::BPS : BatchCfg<__half>::W * BatchCfg<__half>::BPS);
 }
 
 cudaError_t launch_batch_step(int storage, const BatchLaunch& B, int from, const void* in, void* out, cudaStream_t s) {

@@ -1022,58 +1022,100 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
         if (e != cudaSuccess) { delete b; return cuda_fail(e, "cudaStreamCreate"); }
         b->own_stream = true;
     }
-    // Work lists. Strips of all cases in one of three orders (case after
-    // case, the largest case first, or strip 0 of every case, then strip 1, ...),
-    // their rows dealt to the warps of one wave: shape 0, every warp an equal
-    // run of consecutive rows; shape 1, items of at most 32 rows in turn.
+    // Work lists: strips of the cases in one of three orders (case after case,
+    // the largest case first, or strip 0 of every case, then strip 1, ...),
+    // their rows dealt to the warps of one wave. Shape 0: every warp an equal
+    // run of rows. Shape 1: items of at most 32 rows in turn.
+    // The strips of a case read each other's edge columns, so in the first two
+    // orders they are cut at the same rows and given to neighbouring warps,
+    // which find these columns in L1 and L2: for shape 0 the cases with s
+    // strips are stacked to one column s strips wide, and s warps at a time
+    // take the next run of its rows; what is left of a column, less than a
+    // run, is dealt strip by strip to the warps that remain. (40 cases of
+    // 256 x 256, FP32: 108.7 us per step strip by strip, 80.4 us so.)
     std::vector<int> by_size(ncases);
     for (int i = 0; i < ncases; ++i) by_size[i] = i;
     std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int c) {
         return (long long)cfgs[a].nx * cfgs[a].ny > (long long)cfgs[c].nx * cfgs[c].ny;
     });
     const int sw = march_strip(b->storage);
-    std::vector<BatchItem> strips[3];  // whole strips
+    auto strips_of = [&](int i) { return (cfgs[i].nx + sw - 1) / sw; };
     int max_strips = 0;
-    for (int i = 0; i < ncases; ++i) max_strips = std::max(max_strips, (cfgs[i].nx + sw - 1) / sw);
-    auto add = [&](int o, int i, int s) {
-        if (s * sw < cfgs[i].nx) strips[o].push_back({i, s * sw, 0, cfgs[i].ny});
-    };
-    for (int i = 0; i < ncases; ++i)
-        for (int s = 0; s < max_strips; ++s) add(0, i, s);
-    for (int i : by_size)
-        for (int s = 0; s < max_strips; ++s) add(1, i, s);
-    for (int s = 0; s < max_strips; ++s)
-        for (int i = 0; i < ncases; ++i) add(2, i, s);
     long long rows = 0;
-    for (const BatchItem& t : strips[0]) rows += t.y1;
+    for (int i = 0; i < ncases; ++i) {
+        max_strips = std::max(max_strips, strips_of(i));
+        rows += (long long)strips_of(i) * cfgs[i].ny;
+    }
     b->warps = (int)std::min<long long>(batch_warps(b->storage, b->sms), rows);
     for (int o = 0; o < 3; ++o) {
-        std::vector<BatchItem>&even = b->items[0][o], &dealt = b->items[1][o];
-        std::vector<int>&fe = b->first[0][o], &fd = b->first[1][o];
-        long long at = 0;  // rows before strip t
-        int w = 0;
-        for (const BatchItem& t : strips[o]) {
-            for (int y = 0; y < t.y1;) {
-                while (rows * (w + 1) / b->warps <= at + y) ++w;  // the warp that row y falls to
-                const int e = (int)std::min<long long>(t.y1, rows * (w + 1) / b->warps - at);
-                while ((int)fe.size() <= w) fe.push_back((int)even.size());
-                even.push_back({t.c, t.xs, y, e});
+        std::vector<std::vector<BatchItem>> even(b->warps), dealt(b->warps);
+        std::vector<BatchItem> rest, cut;  // items left for single warps; items of at most 32 rows
+        int w = 0;                         // warps that have their rows
+        auto pieces = [&](int i, int s0, int s1) {
+            const int ny = cfgs[i].ny, n = (ny + 31) / 32;
+            for (int j = 0; j < n; ++j)
+                for (int s = s0; s < s1; ++s)
+                    cut.push_back({i, s * sw, (int)((long long)ny * j / n), (int)((long long)ny * (j + 1) / n)});
+        };
+        if (o < 2) {
+            std::vector<std::vector<int>> column(max_strips + 1);
+            for (int j = 0; j < ncases; ++j) {
+                const int i = o == 0 ? j : by_size[j];
+                column[strips_of(i)].push_back(i);
+                pieces(i, 0, strips_of(i));
+            }
+            for (int s = max_strips; s > 0; --s) {
+                long long height = 0;
+                for (int i : column[s]) height += cfgs[i].ny;
+                const int runs = (int)(height * b->warps / rows);
+                long long at = 0;  // rows of the column below case i
+                int run = 0;
+                for (int i : column[s]) {
+                    for (int y = 0; y < cfgs[i].ny;) {
+                        while (run < runs && rows * (run + 1) / b->warps <= at + y) ++run;  // the run that row y falls to
+                        const int e = run < runs ? (int)std::min<long long>(cfgs[i].ny, rows * (run + 1) / b->warps - at) : cfgs[i].ny;
+                        for (int j = 0; j < s; ++j) {
+                            const BatchItem t = {i, j * sw, y, e};
+                            if (run < runs) even[w + run * s + j].push_back(t);
+                            else rest.push_back(t);
+                        }
+                        y = e;
+                    }
+                    at += cfgs[i].ny;
+                }
+                w += runs * s;
+            }
+        } else {
+            for (int s = 0; s < max_strips; ++s)
+                for (int i = 0; i < ncases; ++i)
+                    if (s < strips_of(i)) {
+                        rest.push_back({i, s * sw, 0, cfgs[i].ny});
+                        pieces(i, s, s + 1);
+                    }
+        }
+        long long left = 0, at = 0;
+        for (const BatchItem& t : rest) left += t.y1 - t.y0;
+        const int free = b->warps - w;  // (left > 0 only with free > 0: the runs are equal shares rounded down)
+        int v = 0;
+        for (const BatchItem& t : rest) {
+            for (int y = t.y0; y < t.y1;) {
+                while (left * (v + 1) / free <= at + (y - t.y0)) ++v;
+                const int e = (int)std::min<long long>(t.y1, left * (v + 1) / free - at + t.y0);
+                even[w + v].push_back({t.c, t.xs, y, e});
                 y = e;
             }
-            at += t.y1;
+            at += t.y1 - t.y0;
         }
-        while ((int)fe.size() <= b->warps) fe.push_back((int)even.size());
-        std::vector<BatchItem> cut;
-        for (const BatchItem& t : strips[o]) {
-            const int n = (t.y1 + 31) / 32;
-            for (int j = 0; j < n; ++j) cut.push_back({t.c, t.xs, (int)((long long)t.y1 * j / n), (int)((long long)t.y1 * (j + 1) / n)});
+        for (size_t j = 0; j < cut.size(); ++j) dealt[j % b->warps].push_back(cut[j]);
+        for (int shape = 0; shape < 2; ++shape) {
+            std::vector<BatchItem>& list = b->items[shape][o];
+            for (const std::vector<BatchItem>& t : shape ? dealt : even) {
+                b->first[shape][o].push_back((int)list.size());
+                list.insert(list.end(), t.begin(), t.end());
+            }
+            b->first[shape][o].push_back((int)list.size());
+            b->max_items = std::max(b->max_items, (int)list.size());
         }
-        for (int v = 0; v < b->warps; ++v) {
-            fd.push_back((int)dealt.size());
-            for (size_t j = v; j < cut.size(); j += b->warps) dealt.push_back(cut[j]);
-        }
-        fd.push_back((int)dealt.size());
-        b->max_items = std::max({b->max_items, (int)even.size(), (int)dealt.size()});
     }
     std::vector<BatchCase> hc(ncases);
     for (int i = 0; i < ncases; ++i) {
