@@ -20,7 +20,8 @@ namespace lbm {
 
 namespace {
 
-constexpr int AUX_NT = 256;
+constexpr int AUX_NT = 256;    // threads of a block that adds up a record
+constexpr int FIELD_NT = 64;    // of the passes that have one node per thread
 
 template <class S>
 __device__ __forceinline__ double load_d(const S* buf, const Geometry& G, int p, int x, int y, double rest) {
@@ -35,19 +36,13 @@ __device__ __forceinline__ S to_store(double v, double rest) {
     else return (S)v;
 }
 
-// load_d / to_store in the compute type C (identical to them for C = double)
+// load_d in the compute type C (identical to it for C = double)
 template <class S, class C>
 __device__ __forceinline__ C load_c(const S* buf, const Geometry& G, int p, int x, int y, C rest) {
     const S v = buf[G.at(p, x, y)];
     if constexpr (sizeof(S) == 2) return rest + (C)Store<S, float>::ld(v, 0.0f);
     else return (C)v;
 }
-template <class S, class C>
-__device__ __forceinline__ S to_store_c(C v, C rest) {
-    if constexpr (sizeof(S) == 2) return Store<S, float>::st((float)(v - rest), 0.0f);
-    else return (S)v;
-}
-
 __device__ __forceinline__ int ex_of(int i) {
     return (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
 }
@@ -66,6 +61,55 @@ __device__ __forceinline__ void scatter(S* buf, const Geometry& G, int p, int i,
     put<S>(buf, G, p, xs, ys, v);
 }
 
+// What the kernels of whole fields below have in common. A node's neighbours
+// in the state lie at constant offsets from its row in three columns, so one
+// 64-bit address is formed per column and not one per population.
+template <class S>
+struct NodeAt {
+    static constexpr int SW = sizeof(S) == 2 ? 64 : 32;  // strip width
+    static constexpr int ROW = ROW_LINES * SW;
+    int x, y;
+    long long idx;     // y nx + x
+    long long col[3];  // line 0 of row y in columns x - 1, x, x + 1
+    bool inner;        // three or more nodes from every edge: no neighbour wraps, no copies
+    __device__ __forceinline__ NodeAt(const Geometry& G, long long i) : idx(i) {
+        y = (int)((uint32_t)i / (uint32_t)G.nx);  // (a lattice has at most 2^31 nodes)
+        x = (int)((uint32_t)i - (uint32_t)y * (uint32_t)G.nx);
+#pragma unroll
+        for (int d = -1; d <= 1; ++d) col[d + 1] = G.at(0, x + d, y);
+        inner = x >= 3 && x < G.nx - 3 && y >= 3 && y < G.ny - 3;
+    }
+    // element that population i of the DF whose lines begin at p is pulled from
+    __device__ __forceinline__ long long from(int p, int i) const { return col[1 - EX(i)] + ((p + i) * SW - EY(i) * ROW); }
+    static __device__ constexpr int EX(int i) { return (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0); }
+    static __device__ constexpr int EY(int i) { return (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0); }
+    // the density of the node and its neighbours as the pair force sees them
+    template <class C>
+    __device__ __forceinline__ void densities(const double* __restrict__ rho, const Geometry& G, double rho_open, C rn[9]) const;
+    // the pulled values of a DF, without the rest populations
+    template <class C>
+    __device__ __forceinline__ void pull(const S* __restrict__ buf, int p, C l[9]) const {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const S v = __ldg(buf + from(p, i));
+            if constexpr (sizeof(S) == 8) l[i] = v;
+            else l[i] = widen<C>(Store<S, float>::raw(v));
+        }
+    }
+    // float to C. To FP64 by integer arithmetic, exact: the conversion unit
+    // takes a warp's worth every 16 cycles, as FP64 arithmetic does.
+    template <class C>
+    static __device__ __forceinline__ C widen(float v) {
+        if constexpr (sizeof(C) == 4) {
+            return v;
+        } else {
+            const uint32_t u = __float_as_uint(v), a = u << 1;
+            if (a - 0x01000000u >= 0xfe000000u) return (double)v;  // zero, subnormal, infinite or NaN
+            return __hiloint2double((int)((u & 0x80000000u) | ((a >> 4) + 0x38000000u)), (int)(u << 29));
+        }
+    }
+};
+
 // density at (x, y) as the pair force sees it: the open sides' fixed
 // density beyond them, the adjacent fluid node's beyond a wall, periodic
 // images elsewhere
@@ -77,44 +121,119 @@ __device__ __forceinline__ double rho_nb(const double* rho, const Geometry& G, d
     return rho[(long long)y * G.nx + x];
 }
 
+template <class S>
+template <class C>
+__device__ __forceinline__ void NodeAt<S>::densities(const double* __restrict__ rho, const Geometry& G, double rho_open,
+                                                     C rn[9]) const {
+    if (inner) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) rn[i] = (C)__ldg(rho + idx + EX(i) + EY(i) * G.nx);
+    } else {
+#pragma unroll 1
+        for (int dy = -1; dy <= 1; ++dy) {
+            const double a = rho_nb(rho, G, rho_open, x - 1, y + dy), b = rho_nb(rho, G, rho_open, x, y + dy),
+                         c = rho_nb(rho, G, rho_open, x + 1, y + dy);
+            if (dy < 0) { rn[7] = (C)a; rn[4] = (C)b; rn[8] = (C)c; }
+            else if (dy == 0) { rn[3] = (C)a; rn[0] = (C)b; rn[1] = (C)c; }
+            else { rn[6] = (C)a; rn[2] = (C)b; rn[5] = (C)c; }
+        }
+    }
+}
+
+// M^-1 m for m = (m0, m1, m2, jx, -jx, jy, -jy, m7, m8)
+template <class C>
+__device__ __forceinline__ void populations_jj(C m0, C m1, C m2, C jx, C jy, C m7, C m8, C l[9]) {
+    const C a0 = ninth(m0);
+    const C axis = a0 - m1 * C(1.0 / 36.0) - m2 * C(1.0 / 18.0);
+    const C diag = a0 + m1 * C(1.0 / 18.0) + m2 * C(1.0 / 36.0);
+    l[0] = a0 + (m2 - m1) * C(1.0 / 9.0);
+    const C ap = axis + m7 * C(0.25), am = axis - m7 * C(0.25);
+    l[1] = ap + jx * C(1.0 / 3.0);
+    l[3] = ap - jx * C(1.0 / 3.0);
+    l[2] = am + jy * C(1.0 / 3.0);
+    l[4] = am - jy * C(1.0 / 3.0);
+    const C dp = diag + m8 * C(0.25), dm = diag - m8 * C(0.25), js = jx + jy, jd = jx - jy;
+    l[5] = dp + js * C(1.0 / 12.0);
+    l[7] = dp - js * C(1.0 / 12.0);
+    l[8] = dm + jd * C(1.0 / 12.0);
+    l[6] = dm - jd * C(1.0 / 12.0);
+}
+
+// Populations of the state (rho, u, T). In FP64 bound by the FP64 arithmetic
+// (1/64 of the FP32 rate): no division but the equation of state's, the
+// rest populations of shifted storage come off as three moments, and the
+// moments m_4 = -m_3, m_6 = -m_5, n_7 = n_8 = 0 are used as such. 256 x 256,
+// FP32 storage, FP64 arithmetic: 37.7 us before (180 FP64 operations and 8
+// divisions per node, blocks of 256), 28.7 (147, 64). At 4096 x 1024 in FP32
+// the fields in and out take 436 us instead of 606, in FP16 408 instead of 757
+// (64-bit index divisions and one 64-bit address per population before).
 template <class S, class C>
-__global__ void k_init(const Launch L, const double* __restrict__ rho, const double* __restrict__ ux,
+__global__ void __launch_bounds__(FIELD_NT) k_init(const __grid_constant__ Launch L, const double* __restrict__ rho, const double* __restrict__ ux,
                        const double* __restrict__ uy, const double* __restrict__ T, S* __restrict__ buf) {
     const Geometry& G = L.geo;
     const KC<C>& k = kc<C>(L);
-    const long long n = (long long)G.nx * G.ny;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx % G.nx), y = (int)(idx / G.nx);
-        NodeMacro<C> s;
-        C rn[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) rn[i] = (C)rho_nb(rho, G, (double)L.kd.rho_open, x + ex_of(i), y + ey_of(i));
-        const C r = (C)rho[idx], vx = (C)ux[idx], vy = (C)uy[idx];
-        s.rho = r;
-        s.inv_rho = C(1) / r;
-        s.gx = (rn[1] - rn[3]) / C(3) + ((rn[5] - rn[7]) + (rn[8] - rn[6])) / C(12);
-        s.gy = (rn[2] - rn[4]) / C(3) + ((rn[5] - rn[7]) + (rn[6] - rn[8])) / C(12);
-        s.Fhx = k.G2c * r * s.gx + r * k.axc;
-        s.Fhy = k.G2c * r * s.gy + r * k.ayc;
-        s.uhx = vx / k.c;
-        s.uhy = vy / k.c;
-        s.q = k.c2 * (s.Fhx * s.uhx + s.Fhy * s.uhy);
-        s.T = (C)T[idx];
-        s.rek = r * k.cv * s.T + C(0.5) * r * (vx * vx + vy * vy);
-        C meq[9], Fm[9], neq[9], qm[9], m[9], nn[9], f[9], g[9];
-        equilibria(k, s, meq, Fm, neq, qm, L.cubic != 0);
+    const long long at = blockIdx.x * (long long)FIELD_NT + threadIdx.x;
+    if (at >= (long long)G.nx * G.ny) return;
+    const NodeAt<S> d(G, at);
+    NodeMacro<C> s;
+    C rn[9];
+    d.densities(rho, G, L.kd.rho_open, rn);
+    const C r = rn[0], vx = (C)__ldg(ux + at) * k.c_inv, vy = (C)__ldg(uy + at) * k.c_inv;
+    const C third = C(1.0 / 3.0), twelfth = C(1.0 / 12.0);
+    s.rho = r;
+    s.gx = third * (rn[1] - rn[3]) + twelfth * ((rn[5] - rn[7]) + (rn[8] - rn[6]));
+    s.gy = third * (rn[2] - rn[4]) + twelfth * ((rn[5] - rn[7]) + (rn[6] - rn[8]));
+    s.Fhx = k.G2c * r * s.gx + r * k.axc;
+    s.Fhy = k.G2c * r * s.gy + r * k.ayc;
+    s.uhx = vx;
+    s.uhy = vy;
+    s.q = k.c2 * (s.Fhx * vx + s.Fhy * vy);
+    s.T = (C)__ldg(T + at);
+    s.rek = r * (k.cv * s.T + C(0.5) * k.c2 * (vx * vx + vy * vy));
+    C f[9], g[9];
+    if (L.cubic) {
+        C meq[9], Fm[9], neq[9], qm[9];
+        equilibria(k, s, meq, Fm, neq, qm, true);
 #pragma unroll
         for (int j = 0; j < 9; ++j) {
-            m[j] = meq[j] - k.half_dt * Fm[j];
-            nn[j] = neq[j] - k.half_dt * qm[j];
+            meq[j] -= k.half_dt * Fm[j];
+            neq[j] -= k.half_dt * qm[j];
         }
-        populations9(m, f);
-        populations9(nn, g);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            meq[j] -= k.mrest[j];
+            neq[j] -= k.nrest[j];
+        }
+        populations9(meq, f);
+        populations9(neq, g);
+    } else {
+        // m^eq - dt/2 F_m and n^eq - dt/2 q_m (SM Eq. S3, S4), written out
+        const C pbe = p_BE(k, r, s.T), eta = pbe * k.cs2_inv - r;
+        const C rux = r * vx, ruy = r * vy;
+        const C A3 = C(3) * ((rux * vx + ruy * vy) - k.dt * (s.Fhx * vx + s.Fhy * vy));
+        const C jx = rux - k.half_dt * s.Fhx, jy = ruy - k.half_dt * s.Fhy;
+        const C m7 = (rux - k.dt * s.Fhx) * vx - (ruy - k.dt * s.Fhy) * vy;
+        const C m8 = jx * vy - k.half_dt * s.Fhy * vx;
+        populations_jj(r - k.mrest[0], (C(2) * (eta - r) + A3) - k.mrest[1], (r + k.beta * eta - A3) - k.mrest[2], jx, jy, m7, m8, f);
+        const C hq = k.half_dt * s.q, h = (s.rek + pbe) - hq;
+        populations_jj((s.rek - hq) - k.nrest[0], (C(-4) * s.rek + k.c4g1_Cref * s.T - k.g1 * hq) - k.nrest[1],
+                       (C(4) * s.rek - k.c4g2_Cref * s.T - k.g2 * hq) - k.nrest[2], h * vx, h * vy, C(0), C(0), g);
+    }
+    auto as_stored = [](C v) {
+        if constexpr (sizeof(S) == 2) return Store<S, float>::st((float)v, 0.0f);
+        else return (S)v;
+    };
+    if (d.inner) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            scatter<S>(buf, G, i, i, x, y, to_store_c<S, C>(f[i], (C)L.kf.rest[i]));
-            scatter<S>(buf, G, 9 + i, i, x, y, to_store_c<S, C>(g[i], (C)L.kf.rest[9 + i]));
+            buf[d.from(0, i)] = as_stored(f[i]);
+            buf[d.from(9, i)] = as_stored(g[i]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            scatter<S>(buf, G, i, i, d.x, d.y, as_stored(f[i]));
+            scatter<S>(buf, G, 9 + i, i, d.x, d.y, as_stored(g[i]));
         }
     }
 }
@@ -152,17 +271,15 @@ __global__ void k_get_pops(const Launch L, const S* __restrict__ buf, double* __
 }
 
 template <class S, class C>
-__global__ void k_rho(const Launch L, const S* __restrict__ buf, double* __restrict__ rho) {
+__global__ void __launch_bounds__(FIELD_NT) k_rho(const __grid_constant__ Launch L, const S* __restrict__ buf, double* __restrict__ rho) {
     const Geometry& G = L.geo;
-    const long long n = (long long)G.nx * G.ny;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx % G.nx), y = (int)(idx / G.nx);
-        C r = C(0);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) r += load_c<S, C>(buf, G, i, x - ex_of(i), y - ey_of(i), (C)L.kf.rest[i]);
-        rho[idx] = (double)r;
-    }
+    const long long at = blockIdx.x * (long long)FIELD_NT + threadIdx.x;
+    if (at >= (long long)G.nx * G.ny) return;
+    const NodeAt<S> d(G, at);
+    C l[9], m[9];
+    d.pull(buf, 0, l);
+    moments_of<sizeof(S) == 2>(l, kc<C>(L).mrest, m);
+    rho[at] = (double)m[0];
 }
 
 // rho u_x^3 and rho u_y^3 (u over c) of every node, phi [2][ny][nx], for
@@ -191,48 +308,46 @@ __global__ void k_phi(const Launch L, const S* __restrict__ buf, const double* _
     }
 }
 
-// Macroscopic fields (Eq. 13, 14) and, if partials != NULL, the FP64
-// conservation record reduced deterministically into stats[0..6].
-template <class S, class C>
-__global__ void __launch_bounds__(AUX_NT) k_moments(const Launch L, const S* __restrict__ buf,
-                                                    const double* __restrict__ rho_f, double* __restrict__ o_rho,
-                                                    double* __restrict__ o_ux, double* __restrict__ o_uy,
-                                                    double* __restrict__ o_T, double* __restrict__ partials,
-                                                    double* __restrict__ stats, unsigned* __restrict__ counter) {
+// Macroscopic fields (Eq. 13, 14; 14.5 us at 256 x 256 in FP64) and, with RECORD, the FP64 conservation
+// record reduced deterministically into stats[0..6].
+template <class S, class C, bool RECORD>
+__global__ void __launch_bounds__(RECORD ? AUX_NT : FIELD_NT)
+    k_moments(const __grid_constant__ Launch L, const S* __restrict__ buf, const double* __restrict__ rho_f, double* __restrict__ o_rho,
+              double* __restrict__ o_ux, double* __restrict__ o_uy, double* __restrict__ o_T,
+              double* __restrict__ partials, double* __restrict__ stats, unsigned* __restrict__ counter) {
     const Geometry& G = L.geo;
     const KC<C>& k = kc<C>(L);
     const long long n = (long long)G.nx * G.ny;
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx % G.nx), y = (int)(idx / G.nx);
+        const NodeAt<S> d(G, idx);
         C f[9], g[9], rn[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            f[i] = load_c<S, C>(buf, G, i, x - ex_of(i), y - ey_of(i), (C)L.kf.rest[i]);
-            g[i] = load_c<S, C>(buf, G, 9 + i, x - ex_of(i), y - ey_of(i), (C)L.kf.rest[9 + i]);
-            rn[i] = (C)rho_nb(rho_f, G, (double)L.kd.rho_open, x + ex_of(i), y + ey_of(i));
-        }
+        d.pull(buf, 0, f);
+        d.pull(buf, 9, g);
+        d.densities(rho_f, G, L.kd.rho_open, rn);
         NodeMacro<C> s;
-        node_macro(k, f, g, rn, s);
+        node_macro<sizeof(S) == 2>(k, f, g, rn, s);
         if (o_rho) o_rho[idx] = (double)s.rho;
         if (o_ux) o_ux[idx] = (double)(s.uhx * k.c);
         if (o_uy) o_uy[idx] = (double)(s.uhy * k.c);
         if (o_T) o_T[idx] = (double)s.T;
-        const C lap = C(2) * (((rn[1] + rn[2]) + (rn[3] + rn[4])) / C(3) +
-                              ((rn[5] + rn[6]) + (rn[7] + rn[8])) / C(12) - (C(5) / C(3)) * s.rho);
-        acc[0] += (double)s.rho;
-        acc[1] += (double)(s.rho * s.uhx * k.c);
-        acc[2] += (double)(s.rho * s.uhy * k.c);
-        acc[3] += (double)s.rek;
-        acc[4] += (double)(s.rek - k.a * s.rho * s.rho - k.half_kappa * s.rho * lap);
-        acc[5] = fmax(acc[5], (double)(k.c2 * (s.uhx * s.uhx + s.uhy * s.uhy)));
-        // as the step kernel counts them: density, temperature, velocity (NaN included)
-        if (!(s.rho > C(0) && s.rho < C(1e30) && s.T > C(0) && s.T < C(1e30) &&
-              s.uhx * s.uhx + s.uhy * s.uhy < C(1e30)))
-            acc[6] += 1.0;
+        if constexpr (RECORD) {
+            const C ax = (rn[1] + rn[2]) + (rn[3] + rn[4]), dg = (rn[5] + rn[6]) + (rn[7] + rn[8]);
+            const C u2 = s.uhx * s.uhx + s.uhy * s.uhy;
+            acc[0] += (double)s.rho;
+            acc[1] += (double)(s.rho * s.uhx);
+            acc[2] += (double)(s.rho * s.uhy);
+            acc[3] += (double)s.rek;
+            acc[4] += (double)(s.rek - s.rho * (k.rec_rho * s.rho + k.rec_ax * ax + k.rec_dg * dg));
+            acc[5] = fmax(acc[5], (double)u2);
+            if (bad_node(s.rho, s.T, u2)) acc[6] += 1.0;  // as the step kernel counts them
+        }
     }
-    if (!partials) return;
+    if constexpr (!RECORD) return;
+    acc[1] *= L.kd.c;
+    acc[2] *= L.kd.c;
+    acc[5] *= L.kd.c2;
     __shared__ double red[AUX_NT / 32][7];
     __shared__ bool last;
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
@@ -293,6 +408,8 @@ int aux_blocks(const Geometry& g) {
     return (int)(b < 4096 ? b : 4096);
 }
 
+int field_blocks(const Geometry& g) { return (int)(((long long)g.nx * g.ny + FIELD_NT - 1) / FIELD_NT); }
+
 template <class S>
 struct AuxT {
     // fast: FP32 per-node arithmetic (32- and 16-bit storage only)
@@ -300,17 +417,17 @@ struct AuxT {
                             void* buf, cudaStream_t s, bool fast) {
         if constexpr (sizeof(S) < 8) {
             if (fast) {
-                k_init<S, float><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, rho, ux, uy, T, static_cast<S*>(buf));
+                k_init<S, float><<<field_blocks(L.geo), FIELD_NT, 0, s>>>(L, rho, ux, uy, T, static_cast<S*>(buf));
                 return cudaGetLastError();
             }
         }
-        k_init<S, double><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, rho, ux, uy, T, static_cast<S*>(buf));
+        k_init<S, double><<<field_blocks(L.geo), FIELD_NT, 0, s>>>(L, rho, ux, uy, T, static_cast<S*>(buf));
         return cudaGetLastError();
     }
     // in the step's compute type: FP64 for FP64 storage, FP32 otherwise
     static cudaError_t phi(const Launch& L, const void* buf, double* rho_scratch, double* out, cudaStream_t s) {
         using C = typename std::conditional<sizeof(S) == 8, double, float>::type;
-        k_rho<S, C><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch);
+        k_rho<S, C><<<field_blocks(L.geo), FIELD_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch);
         k_phi<S, C><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch, out);
         return cudaGetLastError();
     }
@@ -322,21 +439,24 @@ struct AuxT {
         k_get_pops<S><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), f, g);
         return cudaGetLastError();
     }
+    template <class C>
+    static cudaError_t moments_in(const Launch& L, const S* buf, double* rho_scratch, double* rho, double* ux,
+                                  double* uy, double* T, double* partials, double* stats, unsigned* counter,
+                                  cudaStream_t s) {
+        k_rho<S, C><<<field_blocks(L.geo), FIELD_NT, 0, s>>>(L, buf, rho_scratch);
+        if (partials)
+            k_moments<S, C, true><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, buf, rho_scratch, rho, ux, uy, T, partials, stats, counter);
+        else
+            k_moments<S, C, false><<<field_blocks(L.geo), FIELD_NT, 0, s>>>(L, buf, rho_scratch, rho, ux, uy, T, nullptr, nullptr, nullptr);
+        return cudaGetLastError();
+    }
     static cudaError_t moments(const Launch& L, const void* buf, double* rho_scratch, double* rho, double* ux,
                                double* uy, double* T, double* partials, double* stats, unsigned* counter,
                                cudaStream_t s, bool fast) {
-        if constexpr (sizeof(S) < 8) {
-            if (fast) {
-                k_rho<S, float><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch);
-                k_moments<S, float><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch,
-                                                                        rho, ux, uy, T, partials, stats, counter);
-                return cudaGetLastError();
-            }
-        }
-        k_rho<S, double><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch);
-        k_moments<S, double><<<aux_blocks(L.geo), AUX_NT, 0, s>>>(L, static_cast<const S*>(buf), rho_scratch, rho, ux,
-                                                                 uy, T, partials, stats, counter);
-        return cudaGetLastError();
+        const S* b = static_cast<const S*>(buf);
+        if constexpr (sizeof(S) < 8)
+            if (fast) return moments_in<float>(L, b, rho_scratch, rho, ux, uy, T, partials, stats, counter, s);
+        return moments_in<double>(L, b, rho_scratch, rho, ux, uy, T, partials, stats, counter, s);
     }
 };
 

@@ -249,6 +249,13 @@ __device__ __forceinline__ void node_macro(const K& k, const C f[9], const C g[9
     macro_of(k, rn, s);
 }
 
+// a non-positive or non-finite density or temperature, or a velocity that
+// runs away (the comparisons also catch NaN)
+template <class C>
+__device__ __forceinline__ bool bad_node(C rho, C T, C u2) {
+    return !(rho > C(0) && rho < C(1e30) && T > C(0) && T < C(1e30) && u2 < C(1e30));
+}
+
 // p_BE = p_EOS + a rho^2 with Eq. 17
 template <class C, class K>
 __device__ __forceinline__ C p_BE(const K& k, C rho, C T) {

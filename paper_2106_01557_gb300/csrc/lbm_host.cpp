@@ -327,6 +327,7 @@ static int derive(const lbm_config& c, lbm_params& p, Launch& L) {
         k.c2 = cast(p.c * p.c);
         k.dt = cast(p.dt);
         k.half_dt = cast(0.5 * p.dt);
+        k.c_inv = cast(1.0 / p.c);
         k.G2c = cast(p.G2 / p.c);
         k.axc = cast(c.accel_x / p.c);
         k.ayc = cast(c.accel_y / p.c);

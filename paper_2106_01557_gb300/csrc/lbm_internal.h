@@ -18,6 +18,7 @@ constexpr int NQ = 8;
 template <class C>
 struct KC {
     C c, c2, dt, half_dt;
+    C c_inv;         // 1 / c
     C G2c;           // G^2 / c   (F^ = F / c)
     C axc, ayc;      // a / c
     C a, half_kappa; // Eq. 16 a and kappa / 2 (total-energy diagnostic)

@@ -125,13 +125,6 @@ __device__ __forceinline__ float vsum(F2 a) { return a.v.x + a.v.y; }
 __device__ __forceinline__ float vmax(float a, float b) { return a > b ? a : b; }
 __device__ __forceinline__ double vmax(double a, double b) { return a > b ? a : b; }
 __device__ __forceinline__ float vmax(float a, F2 b) { return vmax(a, vmax(b.v.x, b.v.y)); }
-// a non-positive or non-finite density or temperature, or a velocity that
-// runs away (the comparisons also catch NaN)
-template <class C>
-__device__ __forceinline__ bool bad_node(C rho, C T, C u2) {
-    return !(rho > C(0) && rho < C(1e30) && T > C(0) && T < C(1e30) && u2 < C(1e30));
-}
-
 // Conservation record of the entering state at a node, or a node pair whose
 // second node lies in the lattice if v1. The total energy rho e_k - a rho^2 -
 // kappa / 2 rho lap(rho), lap = 2 (axes / 3 + diagonals / 12 - 5 rho / 3).
