@@ -172,6 +172,7 @@ struct lbm_handle {
     double* stats = nullptr;     // NQ (step) + NQ (moments) + the step count as of buffer 0 and of buffer 1
     unsigned* counter = nullptr; // 2 counters
     int* status = nullptr;
+    int* h_status = nullptr;  // pinned: its copy after a call
     double* scratch = nullptr;   // 9 * 2 * n doubles (populations / fields)
     size_t scratch_elems = 0;
     cudaStream_t stream = nullptr;
@@ -445,6 +446,7 @@ static void release(lbm_handle* h) {
     if (h->stats) cudaFree(h->stats);
     if (h->counter) cudaFree(h->counter);
     if (h->status) cudaFree(h->status);
+    if (h->h_status) cudaFreeHost(h->h_status);
     if (h->scratch) cudaFree(h->scratch);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
@@ -484,6 +486,7 @@ int lbm_init(const lbm_config* cfg, lbm_handle** out) {
               cudaMalloc(&h->stats, (2 * NQ + 2) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&h->counter, 2 * sizeof(unsigned)) == cudaSuccess &&
               cudaMalloc(&h->status, sizeof(int)) == cudaSuccess &&
+              cudaMallocHost(&h->h_status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&h->scratch, h->scratch_elems * sizeof(double)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -581,11 +584,13 @@ int lbm_maxwell(const lbm_config* cfg, double Tr, double out[3]) {
 }
 
 static int check_status(lbm_handle* h) {
+    // one wait: the status word comes with the call's other work (a blocking
+    // copy after it took 8 us more)
+    CK(cudaMemcpyAsync(h->h_status, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    int st = 0;
-    CK(cudaMemcpy(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost));
+    const int st = *h->h_status;
     if (st) {
-        CK(cudaMemset(h->status, 0, sizeof(int)));
+        CK(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
         if (st & ST_TIMEOUT) return fail(LBM_ERR_TIMEOUT, "a device-side wait exceeded its bound");
         if (st & ST_NONFINITE) return fail(LBM_ERR_DIVERGED, "non-finite or non-positive density or temperature");
     }
@@ -926,6 +931,7 @@ struct lbm_batch {
     std::vector<int> first[2][3];        // where each warp's list begins (and where the last ends)
     float* d_partials = nullptr;
     int* d_status = nullptr;
+    int* h_status = nullptr;  // pinned: its copy after a call
     double* d_steps = nullptr;   // step count as of arena 0 and of arena 1 (keys stochastic rounding)
     double* d_rec = nullptr;     // 8 (case record) + 8 (conservation)
     double* scratch = nullptr;   // 18 x largest case
@@ -962,6 +968,7 @@ static void batch_release(lbm_batch* b) {
                     b->d_status, b->d_rec, b->scratch, b->aux_partials, b->aux_counter, b->d_steps};
     for (void* q : ptrs)
         if (q) cudaFree(q);
+    if (b->h_status) cudaFreeHost(b->h_status);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
 
@@ -1134,6 +1141,7 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
               cudaMalloc(&b->d_items, (size_t)b->max_items * sizeof(BatchItem)) == cudaSuccess &&
               cudaMalloc(&b->d_partials, (size_t)b->max_items * 8 * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&b->d_status, sizeof(int)) == cudaSuccess &&
+              cudaMallocHost(&b->h_status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&b->d_rec, 16 * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&b->scratch, 18 * max_n * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&b->aux_partials, nb_aux * NQ * sizeof(double)) == cudaSuccess &&
@@ -1159,11 +1167,11 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
 }
 
 static int batch_check(lbm_batch* b) {
+    CK(cudaMemcpyAsync(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     CK(cudaStreamSynchronize(b->stream));
-    int st = 0;
-    CK(cudaMemcpy(&st, b->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    const int st = *b->h_status;
     if (st) {
-        CK(cudaMemset(b->d_status, 0, sizeof(int)));
+        CK(cudaMemsetAsync(b->d_status, 0, sizeof(int), b->stream));
         if (st & ST_TIMEOUT) return fail(LBM_ERR_TIMEOUT, "a device-side wait exceeded its bound");
         if (st & ST_NONFINITE) return fail(LBM_ERR_DIVERGED, "non-finite or non-positive density in a batch case");
     }
