@@ -140,25 +140,6 @@ __device__ __forceinline__ void NodeAt<S>::densities(const double* __restrict__ 
     }
 }
 
-// M^-1 m for m = (m0, m1, m2, jx, -jx, jy, -jy, m7, m8)
-template <class C>
-__device__ __forceinline__ void populations_jj(C m0, C m1, C m2, C jx, C jy, C m7, C m8, C l[9]) {
-    const C a0 = ninth(m0);
-    const C axis = a0 - m1 * C(1.0 / 36.0) - m2 * C(1.0 / 18.0);
-    const C diag = a0 + m1 * C(1.0 / 18.0) + m2 * C(1.0 / 36.0);
-    l[0] = a0 + (m2 - m1) * C(1.0 / 9.0);
-    const C ap = axis + m7 * C(0.25), am = axis - m7 * C(0.25);
-    l[1] = ap + jx * C(1.0 / 3.0);
-    l[3] = ap - jx * C(1.0 / 3.0);
-    l[2] = am + jy * C(1.0 / 3.0);
-    l[4] = am - jy * C(1.0 / 3.0);
-    const C dp = diag + m8 * C(0.25), dm = diag - m8 * C(0.25), js = jx + jy, jd = jx - jy;
-    l[5] = dp + js * C(1.0 / 12.0);
-    l[7] = dp - js * C(1.0 / 12.0);
-    l[8] = dm + jd * C(1.0 / 12.0);
-    l[6] = dm - jd * C(1.0 / 12.0);
-}
-
 // Populations of the state (rho, u, T). In FP64 bound by the FP64 arithmetic
 // (1/64 of the FP32 rate): no division but the equation of state's, the
 // rest populations of shifted storage come off as three moments, and the
