@@ -26,21 +26,20 @@ struct BatchCfg {
 };
 
 template <class S>
-__global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch_step(const BatchLaunch B, int from, const S* __restrict__ arena_in, S* __restrict__ arena_out) {
+__global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch_step(const BatchLaunch B, int from, const S* arena_in, S* arena_out) {
     using Cf = MarchCfg<S>;
     using V = typename std::conditional<Cf::NPL == 2, F2, float>::type;
     constexpr int W = BatchCfg<S>::W;
     __shared__ BatchCase s_case[W];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int gw = blockIdx.x * W + warp;
-    if (blockIdx.x == 0 && threadIdx.x == 0) B.steps[1 - from] = __ldcg(&B.steps[from]) + 1.0;
     if (gw >= B.warps) return;
     BatchCase& cs = s_case[warp];
     Strip<S, float> w;
     w.phi = nullptr;
     w.wait_ns = B.tile_wait_ns;
     w.sr = Store<S, float>::SHIFTED && B.rounding;
-    w.step_key = w.sr ? fmix32((uint32_t)(long long)__ldcg(&B.steps[from]) * 0x9e3779b9u + 0x7f4a7c15u) : 0u;
+    w.steps = &B.steps[from];
     const int end = B.first[gw + 1];
     for (int item = B.first[gw]; item < end; ++item) {
         const BatchItem it = B.items[item];
@@ -73,6 +72,10 @@ __global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch
             for (int q = 0; q < 7; ++q) B.partials[(size_t)item * 8 + q] = v[q];
         }
     }
+    if (gw == 0 && lane == 0) {
+        after_previous_grid();
+        B.steps[1 - from] = __ldcg(&B.steps[from]) + 1.0;
+    }
 }
 
 // Per-case conservation record from the per-item partials, FP64, items in
@@ -100,8 +103,8 @@ __global__ void k_batch_case_record(const BatchItem* __restrict__ items, int nit
 
 template <class S>
 cudaError_t launch_bt(const BatchLaunch& B, int from, const void* in, void* out, cudaStream_t s) {
-    k_batch_step<S><<<(B.warps + BatchCfg<S>::W - 1) / BatchCfg<S>::W, 32 * BatchCfg<S>::W, 0, s>>>(B, from, static_cast<const S*>(in), static_cast<S*>(out));
-    return cudaGetLastError();
+    return launch_early(k_batch_step<S>, (B.warps + BatchCfg<S>::W - 1) / BatchCfg<S>::W, 32 * BatchCfg<S>::W, 0, s, B, from,
+                        static_cast<const S*>(in), static_cast<S*>(out));
 }
 
 }  // namespace

@@ -1,0 +1,37 @@
+// Launches that overlap the end of the kernel before them in the stream
+// (programmatic dependent launch): the blocks of the next kernel are placed
+// and started as soon as every block of this one runs and there is room, and
+// wait there for this kernel to complete. A step of a lattice becomes 1.2 to 3
+// us shorter (128 x 128 FP32 5.45 -> 4.31 us, 1363 x 777 in BF16 with walls
+// 31.7 -> 28.6, 4096 x 1024 in FP16 85.1 -> 81.8, FP32 105.7 -> 104.2).
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace lbm {
+
+// For a kernel launched by launch_early, in every thread before its first
+// access to memory that kernels write: waits until the kernel before it has
+// completed and its writes are visible, then lets the kernel after it start
+// (in this order, so that at most two kernels of a stream are on the GPU).
+__device__ __forceinline__ void after_previous_grid() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+}  // namespace lbm

@@ -39,10 +39,10 @@ __device__ __forceinline__ void combine_record(const double* partials, int nblk,
 // so that the common path carries none of their code)
 template <class S, class C, bool OPEN, bool CUBIC>
 __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
-    k_march(const S* __restrict__ in, S* __restrict__ out, const __grid_constant__ Launch L, const MarchGrid mg, double* __restrict__ partials,
-            const double* __restrict__ prev, double* __restrict__ stats, const double* __restrict__ cnt_in,
+    k_march(const S* in, S* out, const __grid_constant__ Launch L, const MarchGrid mg, double* __restrict__ partials,
+            const double* prev, double* __restrict__ stats, const double* cnt_in,
             double* __restrict__ cnt_out, unsigned* __restrict__ counter, int* __restrict__ status,
-            const double* __restrict__ phi) {
+            const double* phi) {
     using Cf = MarchCfg<S>;
     using V = typename std::conditional<Cf::NPL == 2, F2, C>::type;
     __shared__ C red[MW][7];
@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
     if (mg.combine_prev) {
         // block 0: the record of the step before this one
         if (block == 0) {
+            after_previous_grid();
             combine_record(prev, mg.groups * mg.chunks, stats, warp, nw, lane);
             return;
         }
@@ -70,10 +71,11 @@ __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
     Rec<C> acc = {C(0), C(0), C(0), C(0), C(0), C(0), C(0)};
     if (w.xs < G.nx) {
         w.wait_ns = L.tile_wait_ns;
-        // stochastic rounding is keyed by the step count
         w.sr = Store<S, C>::SHIFTED && L.rounding;
-        w.step_key = w.sr ? fmix32((uint32_t)(long long)__ldcg(cnt_in) * 0x9e3779b9u + 0x7f4a7c15u) : 0u;
+        w.steps = cnt_in;
         if (!march_rows<S, C, OPEN, CUBIC>(k, march_constants<V>(L), G, w, acc) && lane == 0) atomicOr(status, ST_TIMEOUT);
+    } else {
+        after_previous_grid();
     }
     if (block == 0 && threadIdx.x == 0) *cnt_out = __ldcg(cnt_in) + 1.0;
 
@@ -120,13 +122,8 @@ cudaError_t march_t(const Launch& L, const void* in, void* out, const MarchGrid&
     const dim3 grid((unsigned)(mg.groups * mg.chunks + (mg.combine_prev ? 1 : 0))), blk((unsigned)(32 * mg.warps));
     const S* i = static_cast<const S*>(in);
     S* o = static_cast<S*>(out);
-    if (L.geo.open)
-        k_march<S, C, true, false><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
-    else if (L.cubic)
-        k_march<S, C, false, true><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
-    else
-        k_march<S, C, false, false><<<grid, blk, 0, s>>>(i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
-    return cudaGetLastError();
+    auto* const kernel = L.geo.open ? k_march<S, C, true, false> : (L.cubic ? k_march<S, C, false, true> : k_march<S, C, false, false>);
+    return launch_early(kernel, grid, blk, 0, s, i, o, L, mg, partials, prev, stats, cnt_in, cnt_out, counter, status, phi);
 }
 
 }  // namespace

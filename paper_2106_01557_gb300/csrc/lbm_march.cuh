@@ -28,7 +28,8 @@
 // 64-wide tiles of all 18 planes in shared memory by tensor copies, with a
 // density pass and a block barrier per tile): FP32 115.0 -> 105.3 (5.74 TB/s;
 // what is left is mostly the memory mix: without the collision it takes 104.6),
-// FP16 107.5 -> 85.9 (bound by the packed arithmetic of 12 warps per SM).
+// FP16 107.5 -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with
+// launches that overlap (lbm_launch.cuh) 104.2 and 81.8.
 // Tried for the rows: a ring of tensor-copied boxes per warp (124, whatever the
 // depth: about 10 cycles of the copy engine per line of 128 bytes), 16-byte
 // asynchronous copies into a shared-memory ring (124: bound by the shared-
@@ -45,6 +46,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_f2.cuh"
+#include "lbm_launch.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_store.cuh"
 
@@ -64,16 +66,19 @@ struct MarchCfg {
     static constexpr int ROW = ROW_LINES * SW;                                 // elements per row of a strip
 };
 
+// A step is launched while the step before it still runs (lbm_launch.cuh), so
+// its loads of the state are ordinary ones: the read-only path (__ldg, or a
+// restricted pointer) is for memory that nobody writes while the kernel lives.
 // The nine populations of one DF pulled at this lane's node(s), as stored.
 // c, l, r: the DF's line 0 in the pulling row, at the lane's (first) column,
 // the column left of it and the column right of its last.
 template <class S, int NPL>
 struct Pulled {
     S v[9];
-    __device__ __forceinline__ void load(const S* __restrict__ c, const S* __restrict__ l, const S* __restrict__ r) {
+    __device__ __forceinline__ void load(const S* c, const S* l, const S* r) {
         using Cf = MarchCfg<S>;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) v[i] = __ldg((EXm(i) == 0 ? c : (EXm(i) > 0 ? l : r)) + (i * Cf::SW - EYm(i) * Cf::ROW));
+        for (int i = 0; i < 9; ++i) v[i] = (EXm(i) == 0 ? c : (EXm(i) > 0 ? l : r))[i * Cf::SW - EYm(i) * Cf::ROW];
     }
     template <class C>
     __device__ __forceinline__ void get(C o[9]) const {
@@ -87,16 +92,16 @@ template <class S>
 struct Pulled<S, 2> {
     uint32_t w[9];           // e_x = 0: both nodes, else node x
     unsigned short b[9];     // e_x != 0: node x + 1
-    __device__ __forceinline__ void load(const S* __restrict__ c, const S* __restrict__ l, const S* __restrict__ r) {
+    __device__ __forceinline__ void load(const S* c, const S* l, const S* r) {
         using Cf = MarchCfg<S>;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const int o = i * Cf::SW - EYm(i) * Cf::ROW;
             if (EXm(i) == 0) {
-                w[i] = __ldg(reinterpret_cast<const uint32_t*>(c + o));
+                w[i] = *reinterpret_cast<const uint32_t*>(c + o);
             } else {
-                w[i] = __ldg(reinterpret_cast<const unsigned short*>(EXm(i) > 0 ? l + o : c + o + 1));
-                b[i] = __ldg(reinterpret_cast<const unsigned short*>(EXm(i) > 0 ? c + o : r + o));
+                w[i] = *reinterpret_cast<const unsigned short*>(EXm(i) > 0 ? l + o : c + o + 1);
+                b[i] = *reinterpret_cast<const unsigned short*>(EXm(i) > 0 ? c + o : r + o);
             }
         }
     }
@@ -188,7 +193,7 @@ struct Strip {
     int xs, y0, y1;            // first column, rows
     unsigned long long wait_ns;  // bound on the wait for the first rows
     bool sr;                   // stochastic rounding of 16-bit storage, keyed by
-    uint32_t step_key;         // the step count
+    const double* steps;       // the step count
 };
 
 // Rows y0 .. y1 - 1 of a strip. False if the wait for the first rows ran out
@@ -201,7 +206,6 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
     constexpr int NPL = Cf::NPL, SW = Cf::SW, ROW = Cf::ROW;
     using V = typename std::conditional<NPL == 2, F2, C>::type;
     constexpr bool SH = Store<S, C>::SHIFTED;
-    if (w.wait_ns == 0) return false;
     const int lane = threadIdx.x % 32;
     const int x = w.xs + NPL * lane;
     const bool v0 = x < G.nx, v1 = x + 1 < G.nx;
@@ -218,7 +222,11 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
     const S* pc = w.in + G.at(0, x, w.y0 - 1);
     const S* pl = w.in + G.at(0, x - 1, w.y0 - 1);
     const S* pr = w.in + G.at(0, x + NPL, w.y0 - 1);
-    auto halo_load = [&]() { return hj < 9 ? __ldg(hp) : S(0.f); };
+    after_previous_grid();  // (a warp's second run of rows finds it done)
+    if (w.wait_ns == 0) return false;
+    // stochastic rounding is keyed by the step count
+    const uint32_t step_key = SH && w.sr ? fmix32((uint32_t)(long long)__ldcg(w.steps) * 0x9e3779b9u + 0x7f4a7c15u) : 0u;
+    auto halo_load = [&]() { return hj < 9 ? *hp : S(0.f); };
     auto next_row = [&]() {
         pc += ROW;
         pl += ROW;
@@ -350,8 +358,8 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
             auto r7 = [&](int xq) {
                 xq = xq < G.nx ? xq : G.nx - 1;
                 const int xm = xq == 0 ? G.nx - 1 : xq - 1, xp = xq == G.nx - 1 ? 0 : xq + 1;
-                const double dpx = 0.5 * (__ldg(w.phi + (long long)y * G.nx + xp) - __ldg(w.phi + (long long)y * G.nx + xm));
-                const double dpy = 0.5 * (__ldg(w.phi + n + (long long)yp * G.nx + xq) - __ldg(w.phi + n + (long long)ym * G.nx + xq));
+                const double dpx = 0.5 * (__ldcg(w.phi + (long long)y * G.nx + xp) - __ldcg(w.phi + (long long)y * G.nx + xm));
+                const double dpy = 0.5 * (__ldcg(w.phi + n + (long long)yp * G.nx + xq) - __ldcg(w.phi + n + (long long)ym * G.nx + xq));
                 return -k.c * ((C)dpx - (C)dpy);
             };
             if constexpr (NPL == 2) R7 = F2(r7(x), r7(x + 1));
@@ -366,7 +374,7 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
         if constexpr (NPL == 2) {
             using PW = PairWord<S>;
             if (w.sr) {
-                const uint32_t h = fmix32((uint32_t)(y * G.nx + x) ^ w.step_key);
+                const uint32_t h = fmix32((uint32_t)(y * G.nx + x) ^ step_key);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
                     wv[i] = PW::sr(f[i], h * (0x9e3779b9u * (2u * i + 1u)));
