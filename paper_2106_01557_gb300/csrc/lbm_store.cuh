@@ -18,31 +18,39 @@ namespace lbm {
 template <class S, class C, bool OPEN>
 __device__ __noinline__ void wall_store(S* __restrict__ out, const Geometry& G, const KC<C>& k, int x, int y,
                                         S fo0, S fo1, S fo2, S go0, S go1, S go2, C rho) {
+    constexpr int SW = sizeof(S) == 2 ? 64 : 32;  // a line's elements
     const bool bottom = (y == 0);
     const int yg = bottom ? -1 : G.ny;
     const C Tw = bottom ? k.T_bottom : k.T_top;
+    // n^eq of the wall at rest is linear in its temperature
+    C ga1, gd1;
+    g_rest_wall(k, rho, C(1), ga1, gd1);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const int opp = bottom ? (j == 0 ? 2 : (j == 1 ? 5 : 6)) : (j == 0 ? 4 : (j == 1 ? 7 : 8));
         // x step of the leaving direction: 0 for 4/2; 7 and 6 go left, 8 and 5 right
         const int ex = j == 0 ? 0 : (bottom ? (j == 1 ? -1 : 1) : (j == 1 ? 1 : -1));
+        const S fv = j == 0 ? fo0 : (j == 1 ? fo1 : fo2);
         S gv = j == 0 ? go0 : (j == 1 ? go1 : go2);
         int xg = x + ex;
         xg = xg < 0 ? xg + G.nx : (xg >= G.nx ? xg - G.nx : xg);
         C T_link = Tw;
         if (bottom && G.hot_len > 0) {
-            int dxh = (xg - G.hot_x0) % G.nx;
-            if (dxh < 0) dxh += G.nx;
-            if (dxh < G.hot_len) T_link = k.T_hot;
+            const int dxh = xg - G.hot_x0;  // (hot_x0 lies in the lattice)
+            if ((dxh < 0 ? dxh + G.nx : dxh) < G.hot_len) T_link = k.T_hot;
         }
         if (T_link > C(0)) {
-            C ga, gd;
-            g_rest_wall(k, rho, T_link, ga, gd);
             const C rest = Store<S, C>::SHIFTED ? k.rest[9 + opp] : C(0);
-            gv = Store<S, C>::st(C(2) * (j == 0 ? ga : gd) - Store<S, C>::ld(gv, rest), rest);
+            gv = Store<S, C>::st(C(2) * T_link * (j == 0 ? ga1 : gd1) - Store<S, C>::ld(gv, rest), rest);
         }
-        put<S, OPEN>(out, G, opp, xg, yg, j == 0 ? fo0 : (j == 1 ? fo1 : fo2));
-        put<S, OPEN>(out, G, 9 + opp, xg, yg, gv);
+        S* const q = out + G.at(opp, xg, yg);
+        q[0] = fv;
+        q[9 * SW] = gv;
+        if (!(OPEN && (G.open & 12)) && (xg < GHOST_COLS || xg >= G.nx - GHOST_COLS)) {  // the periodic copy
+            S* const c = out + G.at(opp, xg < GHOST_COLS ? xg + G.nx : xg - G.nx, yg);
+            c[0] = fv;
+            c[9 * SW] = gv;
+        }
     }
 }
 
