@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include "lbm_conv.h"
+#include "lbm_launch.cuh"
 
 namespace lbm {
 namespace {
@@ -199,8 +200,9 @@ struct WgCfg {
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(WT)
-    k_wgrad(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ dout, int N, int H, int W,
+    k_wgrad(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
             int in_relu, float* __restrict__ part) {
+    after_previous_grid();
     using Cf = WgCfg<CIN, COUT>;
     extern __shared__ __align__(16) unsigned char wg_smem[];
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
@@ -309,8 +311,9 @@ __global__ void __launch_bounds__(WT)
 // that order, then the eight rows are added in order (a fixed order).
 // The last block, where there is a bias gradient, adds its partials [nblk][64]
 // the same way: row j of four adds blocks j, j + 4, ...
-__global__ void __launch_bounds__(256) k_wgrad_sum(const float4* __restrict__ part, int nblk, int n4, float4* __restrict__ dw,
-                                                   const float* __restrict__ bpart, float* __restrict__ db) {
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float4* part, int nblk, int n4, float4* __restrict__ dw,
+                                                   const float* bpart, float* __restrict__ db) {
+    after_previous_grid();
     __shared__ float4 s[8][32];
     if (db && blockIdx.x == gridDim.x - 1) {
         float* t = reinterpret_cast<float*>(s);
@@ -354,7 +357,8 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float4* __restrict__ pa
 // Bias gradient db[c] = sum_p dOut[p][c] (C a multiple of 8, C <= 256):
 // thread = one 8-channel group of a pixel (16-byte loads, coalesced across
 // the block), per-thread sums reduced per channel group in shared memory.
-__global__ void k_bgrad(const __nv_bfloat16* __restrict__ dout, long long P, int C, float* __restrict__ part) {
+__global__ void k_bgrad(const __nv_bfloat16* dout, long long P, int C, float* __restrict__ part) {
+    after_previous_grid();
     __shared__ float s[256][9];
     const int G8 = C / 8;
     const int per = blockDim.x / G8;  // pixels per block sweep
@@ -416,7 +420,8 @@ __global__ void __launch_bounds__(128) k_bgrad64(const __nv_bfloat16* __restrict
 // One warp per channel: lane l adds the partials of blocks l, l + 32, ...
 // in that order, then a butterfly over the lanes; lane 0's result is the
 // same on every run (a fixed order, not a sequential one)
-__global__ void k_bgrad_sum(const float* __restrict__ part, int nblk, int C, float* __restrict__ db) {
+__global__ void k_bgrad_sum(const float* part, int nblk, int C, float* __restrict__ db) {
+    after_previous_grid();
     const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32), lane = threadIdx.x % 32;
     if (c >= C) return;
     float t = 0.f;
@@ -428,7 +433,8 @@ __global__ void k_bgrad_sum(const float* __restrict__ part, int nblk, int C, flo
 
 // *out = sum over i = 0 .. n-1 of part[i], by one warp in a fixed order
 // (lane l: i = l, l + 32, ...; then a butterfly)
-__global__ void k_sum_in_order(const double* __restrict__ part, int n, double* __restrict__ out) {
+__global__ void k_sum_in_order(const double* part, int n, double* __restrict__ out) {
+    after_previous_grid();
     const int lane = threadIdx.x;
     if (blockIdx.x != 0 || lane >= 32) return;
     double t = 0.0;
@@ -445,8 +451,9 @@ __global__ void k_sum_in_order(const double* __restrict__ part, int n, double* _
 // (4 P); sums[N + n] = sum over image n of (x_rho - target_rho), HW pixels per
 // image. Grid y: images. Bound by memory (P x 64 bytes); with 64-bit divisions
 // and 2-byte stores per pixel it took 47 us on 8 x 256 x 256.
-__global__ void k_mse(const float4* __restrict__ out, const float4* __restrict__ target, int N, long long HW,
-                      uint4* __restrict__ dout, double* __restrict__ part, const double* __restrict__ sums) {
+__global__ void k_mse(const float4* out, const float4* target, int N, long long HW,
+                      uint4* __restrict__ dout, double* __restrict__ part, const double* sums) {
+    after_previous_grid();
     __shared__ double s[256];
     double acc = 0.0;
     const long long P = HW * N;
@@ -488,9 +495,10 @@ __global__ void k_mse(const float4* __restrict__ out, const float4* __restrict__
 // for the input gradient: wf[8 - tap][ci][co] = w[tap][co][ci]. Without
 // `update` only the copies. (42 launches of one layer's update or copy took 95 + 69 us.)
 __global__ void k_adam_refresh(const LayerDesc* __restrict__ layers, float* __restrict__ w, float* __restrict__ m,
-                               float* __restrict__ v, const float* __restrict__ g, __nv_bfloat16* __restrict__ w16,
+                               float* __restrict__ v, const float* g, __nv_bfloat16* __restrict__ w16,
                                __nv_bfloat16* __restrict__ wflip, int update, float lr, float b1, float b2, float eps,
                                float c1, float c2) {
+    after_previous_grid();
     const LayerDesc d = layers[blockIdx.y];
     const int nw = 9 * d.cout * d.cin;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + d.cout; i += gridDim.x * blockDim.x) {
@@ -518,9 +526,10 @@ __global__ void k_adam_refresh(const LayerDesc* __restrict__ layers, float* __re
 // fields -> normalised network input: 16 BF16 channels (4 used; x16 may be
 // null) and an FP32 copy of the 4 channels. One pixel per thread, 16-byte
 // stores (with 2-byte stores: 100 us at 1024 x 1024, four times its memory time).
-__global__ void k_pack(const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
-                       const double* __restrict__ T, long long P, NormConsts nc, uint4* __restrict__ x16,
+__global__ void k_pack(const double* rho, const double* ux, const double* uy,
+                       const double* T, long long P, NormConsts nc, uint4* __restrict__ x16,
                        float4* __restrict__ x32) {
+    after_previous_grid();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
         const float4 v = make_float4((float)((rho[p] - nc.off[0]) * nc.inv_scale[0]), (float)((ux[p] - nc.off[1]) * nc.inv_scale[1]),
                                      (float)((uy[p] - nc.off[2]) * nc.inv_scale[2]), (float)((T[p] - nc.off[3]) * nc.inv_scale[3]));
@@ -538,9 +547,10 @@ __global__ void k_pack(const double* __restrict__ rho, const double* __restrict_
 
 // network output [P][4] -> fields, the density of image n (HW pixels; grid y =
 // images) first shifted by -sums[n] / HW (sums not null)
-__global__ void k_unpack(const float4* __restrict__ y, long long HW, const double* __restrict__ sums, NormConsts nc,
+__global__ void k_unpack(const float4* y, long long HW, const double* sums, NormConsts nc,
                          int N, double* __restrict__ rho, double* __restrict__ ux, double* __restrict__ uy,
                          double* __restrict__ T) {
+    after_previous_grid();
     __shared__ double s_mean;
     for (int n = blockIdx.y; n < N; n += gridDim.y) {
     __syncthreads();
@@ -564,8 +574,9 @@ __global__ void k_unpack(const float4* __restrict__ y, long long HW, const doubl
 // its readers shift y_rho by -sums[n] / HW. y, x, t: [P][4]; grid y = images.
 // Each block writes its two partial sums to part[n][block][2];
 // k_mass_sums adds them in block order.
-__global__ void k_mass_stats(const float4* __restrict__ y, const float4* __restrict__ x, const float4* __restrict__ t,
+__global__ void k_mass_stats(const float4* y, const float4* x, const float4* t,
                              int N, long long HW, double* __restrict__ part) {
+    after_previous_grid();
     __shared__ double s[2][256];
     const int n = blockIdx.y;
     double a = 0.0, b = 0.0;
@@ -594,7 +605,8 @@ __global__ void k_mass_stats(const float4* __restrict__ y, const float4* __restr
 
 // one warp per image: lane l adds blocks l, l + 32, ..., then a butterfly
 // (a fixed order)
-__global__ void k_mass_sums(const double* __restrict__ part, int N, int nblk, int with_t, double* __restrict__ sums) {
+__global__ void k_mass_sums(const double* part, int N, int nblk, int with_t, double* __restrict__ sums) {
+    after_previous_grid();
     const int n = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32), lane = threadIdx.x % 32;
     if (n >= N) return;
     double a = 0.0, b = 0.0;
@@ -708,8 +720,7 @@ cudaError_t wgrad_t(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, i
     long long gx = CIN == 64 && COUT == 64 ? wgrad64_blocks(N, H, W, sms) : (2 * sms) / 3;
     if (gx > chunks) gx = chunks;
     if (gx < 1) gx = 1;
-    k_wgrad<CIN, COUT><<<dim3((unsigned)gx, 3), WT, 2 * Cf::STAGE, s>>>(in, dout, N, H, W, in_relu, part);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_early(k_wgrad<CIN, COUT>, dim3((unsigned)gx, 3), WT, 2 * Cf::STAGE, s, in, dout, N, H, W, in_relu, part);
     return e != cudaSuccess ? e : launch_wgrad_sum(part, (int)gx, COUT * CIN, dw, nullptr, nullptr, s);
 }
 
@@ -741,11 +752,9 @@ cudaError_t launch_mass_layer(const float* y, const float* x, const float* t, in
     if (N < 1 || HW < 1) return cudaErrorInvalidValue;
     long long gx = (HW + 255) / 256;
     if (gx > MASS_BLOCKS) gx = MASS_BLOCKS;
-    k_mass_stats<<<dim3((unsigned)gx, (unsigned)N), 256, 0, s>>>(reinterpret_cast<const float4*>(y),
-                                                                 reinterpret_cast<const float4*>(x),
-                                                                 reinterpret_cast<const float4*>(t), N, HW, part);
-    k_mass_sums<<<(32 * N + 127) / 128, 128, 0, s>>>(part, N, (int)gx, t != nullptr, sums);
-    return cudaGetLastError();
+    const cudaError_t e = launch_early(k_mass_stats, dim3((unsigned)gx, (unsigned)N), 256, 0, s, reinterpret_cast<const float4*>(y),
+                                       reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(t), N, HW, part);
+    return e != cudaSuccess ? e : launch_early(k_mass_sums, (32 * N + 127) / 128, 128, 0, s, part, N, (int)gx, (int)(t != nullptr), sums);
 }
 
 size_t conv_smem_bytes(int cin, int cout) {
@@ -779,9 +788,8 @@ cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_
 cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, cudaStream_t s) {
     if (nblk < 1 || cc < 0 || cc % 4 != 0 || (cc == 0 && !db)) return cudaErrorInvalidValue;
     const int n4 = 9 * cc / 4;
-    k_wgrad_sum<<<(n4 + 31) / 32 + (db ? 1 : 0), 256, 0, s>>>(reinterpret_cast<const float4*>(part), nblk, n4,
-                                                             reinterpret_cast<float4*>(dw), bpart, db);
-    return cudaGetLastError();
+    return launch_early(k_wgrad_sum, (n4 + 31) / 32 + (db ? 1 : 0), 256, 0, s, reinterpret_cast<const float4*>(part), nblk, n4,
+                        reinterpret_cast<float4*>(dw), bpart, db);
 }
 
 int wgrad64_blocks(int N, int H, int W, int sms) {
@@ -801,9 +809,8 @@ cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* d
     const int per = 256 / (C / 8);
     long long g = (P + per - 1) / per;
     if (g > 608) g = 608;
-    k_bgrad<<<(unsigned)g, 256, 0, s>>>(dout, P, C, part);
-    k_bgrad_sum<<<(C * 32 + 255) / 256, 256, 0, s>>>(part, (int)g, C, db);
-    return cudaGetLastError();
+    const cudaError_t e = launch_early(k_bgrad, (unsigned)g, 256, 0, s, dout, P, C, part);
+    return e != cudaSuccess ? e : launch_early(k_bgrad_sum, (C * 32 + 255) / 256, 256, 0, s, part, (int)g, C, db);
 }
 
 cudaError_t launch_mse(const float* out, const float* target, int N, long long HW, __nv_bfloat16* dout, double* loss,
@@ -812,27 +819,23 @@ cudaError_t launch_mse(const float* out, const float* target, int N, long long H
     const int ny = N < MSE_BLOCKS ? N : MSE_BLOCKS;
     long long g = (HW + 255) / 256;
     if (g > MSE_BLOCKS / ny) g = MSE_BLOCKS / ny;
-    k_mse<<<dim3((unsigned)g, (unsigned)ny), 256, 0, s>>>(reinterpret_cast<const float4*>(out),
-                                                        reinterpret_cast<const float4*>(target), N, HW,
-                                                        reinterpret_cast<uint4*>(dout), part, sums);
-    k_sum_in_order<<<1, 32, 0, s>>>(part, (int)g * ny, loss);
-    return cudaGetLastError();
+    const cudaError_t e = launch_early(k_mse, dim3((unsigned)g, (unsigned)ny), 256, 0, s, reinterpret_cast<const float4*>(out),
+                                       reinterpret_cast<const float4*>(target), N, HW, reinterpret_cast<uint4*>(dout), part, sums);
+    return e != cudaSuccess ? e : launch_early(k_sum_in_order, 1, 32, 0, s, part, (int)g * ny, loss);
 }
 
 cudaError_t launch_adam_refresh(const LayerDesc* layers, int nlayers, float* w, float* m, float* v, const float* g,
                                 __nv_bfloat16* w16, __nv_bfloat16* wflip, int update, float lr, float b1, float b2, float eps,
                                 float c1, float c2, cudaStream_t s) {
     if (nlayers < 1) return cudaErrorInvalidValue;
-    k_adam_refresh<<<dim3(36, (unsigned)nlayers), 256, 0, s>>>(layers, w, m, v, g, w16, wflip, update, lr, b1, b2, eps, c1, c2);
-    return cudaGetLastError();
+    return launch_early(k_adam_refresh, dim3(36, (unsigned)nlayers), 256, 0, s, layers, w, m, v, g, w16, wflip, update, lr, b1, b2, eps, c1, c2);
 }
 
 cudaError_t launch_pack(const double* rho, const double* ux, const double* uy, const double* T, long long P,
                         const NormConsts& nc, __nv_bfloat16* x16, float* x32, cudaStream_t s) {
     long long g = (P + 255) / 256;
     if (g > 4096) g = 4096;
-    k_pack<<<(unsigned)g, 256, 0, s>>>(rho, ux, uy, T, P, nc, reinterpret_cast<uint4*>(x16), reinterpret_cast<float4*>(x32));
-    return cudaGetLastError();
+    return launch_early(k_pack, (unsigned)g, 256, 0, s, rho, ux, uy, T, P, nc, reinterpret_cast<uint4*>(x16), reinterpret_cast<float4*>(x32));
 }
 
 cudaError_t launch_unpack(const float* y, int N, long long HW, const double* sums, const NormConsts& nc, double* rho,
@@ -841,8 +844,7 @@ cudaError_t launch_unpack(const float* y, int N, long long HW, const double* sum
     const int ny = N < 1024 ? N : 1024;
     long long g = (HW + 255) / 256;
     if (g > 1216) g = 1216;
-    k_unpack<<<dim3((unsigned)g, (unsigned)ny), 256, 0, s>>>(reinterpret_cast<const float4*>(y), HW, sums, nc, N, rho, ux, uy, T);
-    return cudaGetLastError();
+    return launch_early(k_unpack, dim3((unsigned)g, (unsigned)ny), 256, 0, s, reinterpret_cast<const float4*>(y), HW, sums, nc, N, rho, ux, uy, T);
 }
 
 }  // namespace lbm

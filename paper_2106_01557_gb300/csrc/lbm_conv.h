@@ -13,6 +13,9 @@ struct NormConsts {
     double inv_scale[4];
 };
 
+// The tcgen05 kernels fetch weights and biases before they wait for the kernel
+// before them in the stream (lbm_launch.cuh): that kernel may not be the one
+// that writes them.
 struct ConvArgs {
     const __nv_bfloat16* in;      // [N][H][W][cin]
     const __nv_bfloat16* w;       // [9][cout][cin]

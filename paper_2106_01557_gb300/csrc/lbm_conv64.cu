@@ -45,6 +45,7 @@
 
 #include "lbm_conv.h"
 #include "lbm_conv64.cuh"
+#include "lbm_launch.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_tc.cuh"
 
@@ -65,8 +66,8 @@ struct C6Maps {
 };
 
 __global__ void __launch_bounds__(C6_THREADS, 1)
-    k_conv64(const __grid_constant__ C6Maps tm, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
-             int N, int H, int W, int in_relu, int out_relu, int with_res, const uint2* __restrict__ mbits,
+    k_conv64(const __grid_constant__ C6Maps tm, const __nv_bfloat16* w, const float* bias,
+             int N, int H, int W, int in_relu, int out_relu, int with_res, const uint2* mbits,
              uint2* __restrict__ obits, int* __restrict__ status) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[C6_SLOTS], ready[C6_SLOTS], empty[C6_SLOTS], acc_full[C6_BLK], acc_empty[C6_BLK],
@@ -99,14 +100,14 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
         fence_mbar_init();
         dead_flag = 0;
     }
-    if (tid < 64) s_bias[tid] = bias ? bias[tid] : 0.f;
+    if (tid < 64) s_bias[tid] = bias ? __ldcg(bias + tid) : 0.f;
     // weights [9 taps (dy, dx)][co][ci] -> [3 dx][n = block (dy = +1, 0, -1) * 64 + co][64 ci], 16-byte
     // chunks swizzled by the row
     for (int e = tid; e < 9 * 64 * 8; e += C6_THREADS) {
         const int kg = e % 8, co = (e / 8) % 64, tap = e / 512;
         const int n = (2 - tap / 3) * 64 + co;
         *reinterpret_cast<uint4*>(smem + (tap % 3) * C6_WDX + n * 128 + ((kg ^ (n & 7)) * 16)) =
-            *reinterpret_cast<const uint4*>(w + ((size_t)tap * 64 + co) * 64 + kg * 8);
+            __ldcg(reinterpret_cast<const uint4*>(w + ((size_t)tap * 64 + co) * 64 + kg * 8));
     }
     fence_proxy_async();
     tc_fence_before();
@@ -121,6 +122,8 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+
+    after_previous_grid();  // (the weights and biases are older: see ConvArgs)
 
     const StripRuns R(N, H, W);
     const long long r_begin = R.rows * blockIdx.x / gridDim.x, r_end = R.rows * (blockIdx.x + 1) / gridDim.x;
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
             const unsigned tt = c.t0 + c.t;
             const size_t pix = ((size_t)c.u.n * H + c.u.y0 + c.t) * W + c.u.x0 + px;
             uint2 mw = make_uint2(0xffffffffu, 0xffffffffu);
-            if (mbits && px < c.u.nv) mw = __ldg(mbits + pix);
+            if (mbits && px < c.u.nv) mw = mbits[pix];
             if (!role_wait(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
             __syncwarp();
             tc_fence_after();
@@ -400,12 +403,13 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
 
 // The sign bits of an activation no layer of this kernel has written (the
 // lift layer's): one 32-channel word per thread.
-__global__ void k_sign_bits(const uint4* __restrict__ x, long long words, uint32_t* __restrict__ bits) {
+__global__ void k_sign_bits(const uint4* x, long long words, uint32_t* __restrict__ bits) {
+    after_previous_grid();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < words; i += (long long)gridDim.x * blockDim.x) {
         uint32_t b = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const uint4 v = __ldg(x + 4 * i + q);
+            const uint4 v = x[4 * i + q];
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
             for (int j = 0; j < 4; ++j) b |= __hgt2_mask(h[j], __floats2bfloat162_rn(0.f, 0.f)) & (0x10001u << (4 * q + j));
@@ -449,8 +453,7 @@ cudaError_t encode_rows64(const void* base, long long rows, int W, int px, CUten
 cudaError_t launch_sign_bits(const __nv_bfloat16* x, long long P, unsigned long long* bits, cudaStream_t s) {
     long long g = (2 * P + 255) / 256;
     if (g > 8192) g = 8192;
-    k_sign_bits<<<(unsigned)g, 256, 0, s>>>(reinterpret_cast<const uint4*>(x), 2 * P, reinterpret_cast<uint32_t*>(bits));
-    return cudaGetLastError();
+    return launch_early(k_sign_bits, (unsigned)g, 256, 0, s, reinterpret_cast<const uint4*>(x), 2 * P, reinterpret_cast<uint32_t*>(bits));
 }
 
 cudaError_t launch_conv64(const ConvArgs& a, cudaStream_t s, int sms, int* status) {
@@ -471,10 +474,8 @@ cudaError_t launch_conv64(const ConvArgs& a, cudaStream_t s, int sms, int* statu
     const cudaError_t e = cudaFuncSetAttribute(k_conv64, cudaFuncAttributeMaxDynamicSharedMemorySize, C6_BYTES);
     if (e != cudaSuccess) return e;
     const int grid = tiles < sms ? (int)tiles : sms;
-    k_conv64<<<grid, C6_THREADS, C6_BYTES, s>>>(m, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.out_relu, a.res16 != nullptr,
-                                               reinterpret_cast<const uint2*>(a.mbits), reinterpret_cast<uint2*>(a.obits),
-                                               status);
-    return cudaGetLastError();
+    return launch_early(k_conv64, grid, C6_THREADS, C6_BYTES, s, m, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.out_relu,
+                        (int)(a.res16 != nullptr), reinterpret_cast<const uint2*>(a.mbits), reinterpret_cast<uint2*>(a.obits), status);
 }
 
 }  // namespace lbm

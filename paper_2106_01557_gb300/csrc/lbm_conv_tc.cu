@@ -59,6 +59,7 @@
 #include <stdint.h>
 
 #include "lbm_conv.h"
+#include "lbm_launch.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_tc.cuh"
 
@@ -132,9 +133,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
-              int N, int H, int W, int in_relu, const __nv_bfloat16* __restrict__ mask,
-              const __nv_bfloat16* __restrict__ res16, const float* __restrict__ res32,
+    k_conv_tc(const __nv_bfloat16* in, const __nv_bfloat16* w, const float* bias,
+              int N, int H, int W, int in_relu, const __nv_bfloat16* mask,
+              const __nv_bfloat16* res16, const float* res32,
               __nv_bfloat16* __restrict__ out16, float* __restrict__ out32, int* __restrict__ status) {
     using Cf = TcCfg<CIN, COUT>;
     extern __shared__ unsigned char smem_raw[];
@@ -159,14 +160,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         mbar_init(&bar[1], 1);
         fence_mbar_init();
     }
-    for (int c = tid; c < COUT; c += TC_THREADS) s_bias[c] = bias ? bias[c] : 0.f;
+    for (int c = tid; c < COUT; c += TC_THREADS) s_bias[c] = bias ? __ldcg(bias + c) : 0.f;
     // weights [9 taps (dy, dx)][COUT][CIN] -> per dx, N rows n = block (dy = +1,
     // 0, -1) * COUT + co: [3 dx][n][64 channels, chunk kg at kg ^ (n % 8)]
     // (CIN = 64) or [3 dx][CIN/8][n][8 channels]
     for (int e = tid; e < 9 * COUT * Cf::KG; e += TC_THREADS) {
         const int kg = e % Cf::KG, co = (e / Cf::KG) % COUT, tap = e / (Cf::KG * COUT);
         const int dyi = tap / 3, dxi = tap % 3, n = (2 - dyi) * COUT + co;
-        const uint4 v = *reinterpret_cast<const uint4*>(w + ((size_t)tap * COUT + co) * CIN + kg * 8);
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(w + ((size_t)tap * COUT + co) * CIN + kg * 8));
         const int off = Cf::WSW ? dxi * Cf::WDX + n * 128 + ((kg ^ (n & 7)) * 16)
                                 : (dxi * Cf::KG + kg) * Cf::WGS + n * 16;
         *reinterpret_cast<uint4*>(s_w + off) = v;
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base;
+    after_previous_grid();  // (the weights and biases are older: see ConvArgs)
     // instruction descriptor: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9,
     // 10-12 = 1), both K-major (bits 15, 16 = 0), M >> 4 (bits 24-28); N >> 3
     // (bits 17-22) is added per MMA
@@ -483,9 +485,8 @@ cudaError_t conv_tc_t(const ConvArgs& a, cudaStream_t s, int sms, int* status) {
     }
     const long long rows = (long long)a.N * a.H * ((a.W + TC_TW - 1) / TC_TW);
     const int grid = rows < sms ? (int)rows : sms;
-    k_conv_tc<CIN, COUT><<<grid, TC_THREADS, Cf::BYTES, s>>>(a.in, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.mask,
-                                                             a.res16, a.res32, a.out16, a.out32, status);
-    return cudaGetLastError();
+    return launch_early(k_conv_tc<CIN, COUT>, grid, TC_THREADS, Cf::BYTES, s, a.in, a.w, a.bias, a.N, a.H, a.W, a.in_relu, a.mask,
+                        a.res16, a.res32, a.out16, a.out32, status);
 }
 
 }  // namespace

@@ -3,7 +3,9 @@
 // and started as soon as every block of this one runs and there is room, and
 // wait there for this kernel to complete. A step of a lattice becomes 1.2 to 3
 // us shorter (128 x 128 FP32 5.45 -> 4.31 us, 1363 x 777 in BF16 with walls
-// 31.7 -> 28.6, 4096 x 1024 in FP16 85.1 -> 81.8, FP32 105.7 -> 104.2).
+// 31.7 -> 28.6, 4096 x 1024 in FP16 85.1 -> 81.8, FP32 105.7 -> 104.2), a
+// forward pass of the surrogate on 1024 x 1024 1163 -> 1103 us, a training step
+// on 8 x 256 x 256 2175 -> 1963 and on 3 x 100 x 208 897 -> 692.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -31,6 +31,7 @@
 
 #include "lbm_conv.h"
 #include "lbm_conv64.cuh"
+#include "lbm_launch.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_tc.cuh"
 
@@ -93,6 +94,8 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+
+    after_previous_grid();
 
     const StripRuns R(N, H, W);
     const long long r_begin = R.rows * blockIdx.x / gridDim.x, r_end = R.rows * (blockIdx.x + 1) / gridDim.x;
@@ -308,8 +311,7 @@ cudaError_t launch_wgrad64(const __nv_bfloat16* in, const __nv_bfloat16* dout, i
     if (e != cudaSuccess) return e;
     const int grid = wgrad64_blocks(N, H, W, sms);
     float* bpart = part + (size_t)grid * 9 * 64 * 64;
-    k_wgrad64<<<grid, W6_THREADS, W6_BYTES, s>>>(tx, tx8, td, N, H, W, in_relu, part, bpart, status);
-    e = cudaGetLastError();
+    e = launch_early(k_wgrad64, grid, W6_THREADS, W6_BYTES, s, tx, tx8, td, N, H, W, in_relu, part, bpart, status);
     return e != cudaSuccess ? e : launch_wgrad_sum(part, grid, 64 * 64, dw, bpart, db, s);
 }
 
