@@ -27,7 +27,7 @@ struct ConvArgs {
     const float* res32;           // [P][4] added to out32 (or null)
     __nv_bfloat16* out16;         // [P][cout] BF16 output, or
     float* out32;                 // [P][4] FP32 output of the first four channels
-    // launch_conv64 only:
+    // launch_conv_tc only (and mask launch_conv only):
     int out_relu;                 // max(0, .) of the BF16 output
     const unsigned long long* mbits;  // [P]: the mask as bits (or null), as an earlier layer's obits
     unsigned long long* obits;    // [P]: set to the sign bits (> 0) of the BF16 output before its ReLU (or null)
@@ -35,15 +35,12 @@ struct ConvArgs {
 
 size_t conv_smem_bytes(int cin, int cout);
 cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms);
-// The same convolution on tcgen05 MMAs with tensor-memory accumulators
-// (lbm_conv_tc.cu); bit 0 of the device int *status is set if a wait for
-// the tensor cores ran out of time (the output is then incomplete).
+// The same convolution on tcgen05 MMAs with tensor-memory accumulators,
+// warp-specialised (lbm_conv_tc.cu): 64 -> 64 and 16 -> 64 (without in_relu) to
+// BF16, masked by bits, 64 -> 16 to FP32. Bit 0 of the device int *status is
+// set if a wait for the tensor cores ran out of time (the output is then
+// incomplete).
 cudaError_t launch_conv_tc(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms, int* status);
-// The 64 -> 64 layers, warp-specialised (lbm_conv64.cu); outputs and status
-// as launch_conv_tc's.
-cudaError_t launch_conv64(const ConvArgs& a, cudaStream_t s, int sms, int* status);
-// the sign bits of a [P][64] activation, as launch_conv64's obits
-cudaError_t launch_sign_bits(const __nv_bfloat16* x, long long P, unsigned long long* bits, cudaStream_t s);
 // The gradient reductions write per-block partial sums to `part` and add
 // them in block order (no atomics, so results are reproducible bit for
 // bit); grad_scratch_floats(sms) floats serve both.

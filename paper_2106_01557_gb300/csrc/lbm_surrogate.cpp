@@ -131,7 +131,7 @@ static int ensure_acts(lbm_surrogate* s, long long P, bool train) {
     if (ok && train)
         ok = cudaMalloc(&s->g0, a) == cudaSuccess && cudaMalloc(&s->g1, a) == cudaSuccess &&
              cudaMalloc(&s->g2, a) == cudaSuccess &&
-             cudaMalloc(&s->hbits, (size_t)P * s->cfg.blocks * 8) == cudaSuccess &&
+             cudaMalloc(&s->hbits, (size_t)P * (s->cfg.blocks + 1) * 8) == cudaSuccess &&
              cudaMalloc(&s->zbits, (size_t)P * s->cfg.blocks * 8) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -157,9 +157,7 @@ static ConvArgs cargs(const __nv_bfloat16* in, const __nv_bfloat16* w, const flo
 
 // 3x3 convolution on the configured path
 static int conv(lbm_surrogate* s, int cin, int cout, const ConvArgs& a) {
-    if (s->cfg.conv_path == 0 && cin == 64 && cout == 64) {
-        SCK(launch_conv64(a, s->stream, s->sms, s->d_status));
-    } else if (s->cfg.conv_path == 0) {
+    if (s->cfg.conv_path == 0) {
         SCK(launch_conv_tc(cin, cout, a, s->stream, s->sms, s->d_status));
     } else {
         SCK(launch_conv(cin, cout, a, s->stream, s->sms));
@@ -214,8 +212,8 @@ static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
     const Layer& lift = s->layers[0];
     ConvArgs a = cargs(s->x16, lift.w16, lift.b, N, H, W, 0);
     a.out16 = s->h[0];
+    if (train && s->cfg.conv_path == 0) a.obits = s->hbits;
     CONV(16, C, a);
-    if (train && s->cfg.conv_path == 0) SCK(launch_sign_bits(s->h[0], P, s->hbits, s->stream));
     for (int b = 0; b < B; ++b) {
         const Layer& L1 = s->layers[1 + 2 * b];
         const Layer& L2 = s->layers[2 + 2 * b];
@@ -233,7 +231,7 @@ static int run_forward(lbm_surrogate* s, int N, int H, int W, bool train) {
         a = cargs(z, L2.w16, L2.b, N, H, W, !tc);
         a.res16 = hin;
         a.out16 = hout;
-        if (tc && train && b + 1 < B) a.obits = s->hbits + (b + 1) * P;
+        if (tc && train) a.obits = s->hbits + (b + 1) * P;
         CONV(C, C, a);
     }
     const Layer& proj = s->layers.back();
@@ -252,7 +250,8 @@ static int run_backward(lbm_surrogate* s, int N, int H, int W) {
     Layer& proj = s->layers.back();
     WGRAD(proj, s->h[B], s->dy16, 1);
     ConvArgs a = cargs(s->dy16, proj.wflip, nullptr, N, H, W, 0);
-    a.mask = s->h[B];
+    if (tc) a.mbits = s->hbits + B * P;
+    else a.mask = s->h[B];
     a.out16 = s->g0;  // d h_B
     CONV(16, C, a);
     __nv_bfloat16* dh = s->g0;
