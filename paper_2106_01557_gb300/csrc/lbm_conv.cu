@@ -6,16 +6,17 @@
 //                sit in shared memory; fused epilogue: bias, ReLU mask of
 //                another tensor, residual add (BF16 or FP32), BF16 or FP32
 //                output. Also serves the input gradient (flipped weights).
-//   k_wgrad      weight gradient: per (tap, 16 output channels) a GEMM over
-//                pixels, warps splitting the pixels; each block writes its
-//                partial sums, which k_wgrad_sum adds in block order (the
-//                64 -> 64 layers have a tcgen05 version in lbm_conv_tc.cu).
-//   k_bgrad      bias gradient (per-block partials, summed in block order).
+//   k_wgrad      weight gradient: per filter row a GEMM over pixels; each
+//                block writes its partial sums, which k_wgrad_sum adds in a
+//                fixed order
+//   k_bgrad      bias gradient (per-block partials, summed in a fixed order).
+// (These three on mma.sync; conv_path 0 takes the tcgen05 kernels of
+// lbm_conv_tc.cu and lbm_wgrad64.cu, which sum in the same order.)
 // No reduction uses atomics: the order of every sum is fixed, so training
 // is bit-for-bit reproducible.
 //   k_mse        loss and its gradient.
-//   k_adam       optimiser step on FP32 master weights, refreshing the BF16
-//                forward and flipped copies.
+//   k_adam_refresh  optimiser step on FP32 master weights of all layers, and
+//                the BF16 forward and flipped copies.
 //   k_pack / k_unpack  fields <-> normalised network tensors.
 // The MMA is mma.sync m16n8k16 (BF16 in, FP32 accumulate).
 #include <cuda_bf16.h>
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(CT, 1)
 // tiles: A = dOut^T (co x pixels), B = input (pixels x ci, shifted by dx).
 // One A fragment serves the three taps. Warp w owns the 16-channel output
 // block w % (COUT/16) and a contiguous group of 8-channel input blocks; its
-// FP32 sums are added to dw once at the end (atomics).
+// FP32 sums are the block's partial, added by k_wgrad_sum in a fixed order.
 constexpr int WT = 256;      // threads (8 warps)
 constexpr int WCH = 128;     // pixels per chunk
 
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(WT)
 // The last block, where there is a bias gradient, adds its partials [nblk][64]
 // the same way: row j of four adds blocks j, j + 4, ...
 __global__ void __launch_bounds__(256) k_wgrad_sum(const float4* part, int nblk, int n4, float4* __restrict__ dw,
-                                                   const float* bpart, float* __restrict__ db) {
+                                                   const float* bpart, float* __restrict__ db, int nb) {
     after_previous_grid();
     __shared__ float4 s[8][32];
     if (db && blockIdx.x == gridDim.x - 1) {
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float4* part, int nblk,
         for (int b = j; b < nblk; b += 4) a += __ldcg(bpart + (size_t)b * 64 + c);
         t[threadIdx.x] = a;
         __syncthreads();
-        if (j == 0) db[c] = ((a + t[64 + c]) + t[128 + c]) + t[192 + c];
+        if (j == 0 && c < nb) db[c] = ((a + t[64 + c]) + t[128 + c]) + t[192 + c];
         return;
     }
     const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
@@ -354,38 +355,11 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float4* part, int nblk,
     }
 }
 
-// Bias gradient db[c] = sum_p dOut[p][c] (C a multiple of 8, C <= 256):
-// thread = one 8-channel group of a pixel (16-byte loads, coalesced across
-// the block), per-thread sums reduced per channel group in shared memory.
-__global__ void k_bgrad(const __nv_bfloat16* dout, long long P, int C, float* __restrict__ part) {
-    after_previous_grid();
-    __shared__ float s[256][9];
-    const int G8 = C / 8;
-    const int per = blockDim.x / G8;  // pixels per block sweep
-    const int c8 = threadIdx.x % G8, sub = threadIdx.x / G8;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (sub < per) {
-        for (long long p = (long long)blockIdx.x * per + sub; p < P; p += (long long)gridDim.x * per) {
-            const uint4 v = *reinterpret_cast<const uint4*>(dout + p * C + c8 * 8);
-            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc[q] += __bfloat162float(h[q]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[threadIdx.x][q] = acc[q];
-    __syncthreads();
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        const int g8 = c / 8, q = c % 8;
-        float t = 0.f;
-        for (int k = 0; k < per; ++k) t += s[k * G8 + g8][q];
-        part[(size_t)blockIdx.x * C + c] = t;
-    }
-}
-
-// The same of 64 channels, over the blocks' runs of rows and in the order in
-// which k_wgrad64 sums it (128 threads: 8 channels of pixels sub, sub + 16, ...).
-__global__ void __launch_bounds__(128) k_bgrad64(const __nv_bfloat16* __restrict__ dout, int N, int H, int W, float* __restrict__ part) {
+// Bias gradient db[c] = sum_p dOut[p][c]: the block's partial sums over the
+// blocks' runs of rows, in the order in which k_wgrad_tc sums them (128 threads:
+// 8 channels of pixels sub, sub + 16, ...; [64] per block, zeros past C).
+template <int C>
+__global__ void __launch_bounds__(128) k_bgrad(const __nv_bfloat16* __restrict__ dout, int N, int H, int W, float* __restrict__ part) {
     __shared__ float s[16][64];
     const int c8 = threadIdx.x % 8, sub = threadIdx.x / 8;
     const int tiles_x = (W + WCH - 1) / WCH;
@@ -395,12 +369,12 @@ __global__ void __launch_bounds__(128) k_bgrad64(const __nv_bfloat16* __restrict
     for (long long r = rows * blockIdx.x / gridDim.x; r < r_end; ++r) {
         const long long strip = r / H;
         const int x0 = (int)(strip % tiles_x) * WCH;
-        const __nv_bfloat16* row = dout + ((strip / tiles_x * H + r % H) * W + x0) * 64 + c8 * 8;
+        const __nv_bfloat16* row = dout + ((strip / tiles_x * H + r % H) * W + x0) * C + c8 * 8;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int px = sub + 16 * i;
-            if (x0 + px >= W) break;
-            const uint4 v = *reinterpret_cast<const uint4*>(row + (size_t)px * 64);
+            if (x0 + px >= W || c8 * 8 >= C) break;
+            const uint4 v = *reinterpret_cast<const uint4*>(row + (size_t)px * C);
             const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v);
 #pragma unroll
             for (int c = 0; c < 8; ++c) acc[c] += __bfloat162float(h[c]);
@@ -414,21 +388,6 @@ __global__ void __launch_bounds__(128) k_bgrad64(const __nv_bfloat16* __restrict
         for (int j = 0; j < 16; ++j) t += s[j][threadIdx.x];
         part[(size_t)blockIdx.x * 64 + threadIdx.x] = t;
     }
-}
-
-// db[c] = sum over blocks b = 0, 1, ... of part[b][c]
-// One warp per channel: lane l adds the partials of blocks l, l + 32, ...
-// in that order, then a butterfly over the lanes; lane 0's result is the
-// same on every run (a fixed order, not a sequential one)
-__global__ void k_bgrad_sum(const float* part, int nblk, int C, float* __restrict__ db) {
-    after_previous_grid();
-    const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32), lane = threadIdx.x % 32;
-    if (c >= C) return;
-    float t = 0.f;
-    for (int b = lane; b < nblk; b += 32) t += part[(size_t)b * C + c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) db[c] = t;
 }
 
 // *out = sum over i = 0 .. n-1 of part[i], by one warp in a fixed order
@@ -714,14 +673,9 @@ cudaError_t wgrad_t(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, i
         if (e != cudaSuccess) return e;
         set = true;
     }
-    const long long chunks = (long long)N * H * ((W + WCH - 1) / WCH);
-    // with the three filter rows two CTAs per SM; the 64 -> 64 layers' rows are
-    // split as the tcgen05 path splits them
-    long long gx = CIN == 64 && COUT == 64 ? wgrad64_blocks(N, H, W, sms) : (2 * sms) / 3;
-    if (gx > chunks) gx = chunks;
-    if (gx < 1) gx = 1;
+    const int gx = wgrad_blocks(N, H, W, sms);  // the rows are split as the tcgen05 path splits them
     const cudaError_t e = launch_early(k_wgrad<CIN, COUT>, dim3((unsigned)gx, 3), WT, 2 * Cf::STAGE, s, in, dout, N, H, W, in_relu, part);
-    return e != cudaSuccess ? e : launch_wgrad_sum(part, (int)gx, COUT * CIN, dw, nullptr, nullptr, s);
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, gx, COUT * CIN, dw, nullptr, nullptr, 0, s);
 }
 
 }  // namespace
@@ -773,8 +727,7 @@ cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, in
 }
 
 size_t grad_scratch_floats(int sms) {
-    const size_t w = (size_t)sms * (9 * 64 * 64 + 64), b = (size_t)608 * 256;
-    return w > b ? w : b;
+    return (size_t)sms * (9 * 64 * 64 + 64);
 }
 
 cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
@@ -785,32 +738,25 @@ cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, cudaStream_t s) {
+cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, int nb, cudaStream_t s) {
     if (nblk < 1 || cc < 0 || cc % 4 != 0 || (cc == 0 && !db)) return cudaErrorInvalidValue;
     const int n4 = 9 * cc / 4;
     return launch_early(k_wgrad_sum, (n4 + 31) / 32 + (db ? 1 : 0), 256, 0, s, reinterpret_cast<const float4*>(part), nblk, n4,
-                        reinterpret_cast<float4*>(dw), bpart, db);
+                        reinterpret_cast<float4*>(dw), bpart, db, nb);
 }
 
-int wgrad64_blocks(int N, int H, int W, int sms) {
+int wgrad_blocks(int N, int H, int W, int sms) {
     const long long rows = (long long)N * H * ((W + WCH - 1) / WCH);
     return rows < sms ? (int)rows : sms;
 }
 
-cudaError_t launch_bgrad64(const __nv_bfloat16* dout, int N, int H, int W, float* db, float* part, cudaStream_t s, int sms) {
-    const int g = wgrad64_blocks(N, H, W, sms);
-    k_bgrad64<<<g, 128, 0, s>>>(dout, N, H, W, part);
+cudaError_t launch_bgrad(const __nv_bfloat16* dout, int N, int H, int W, int C, float* db, float* part, cudaStream_t s, int sms) {
+    const int g = wgrad_blocks(N, H, W, sms);
+    if (C == 64) k_bgrad<64><<<g, 128, 0, s>>>(dout, N, H, W, part);
+    else if (C == 16) k_bgrad<16><<<g, 128, 0, s>>>(dout, N, H, W, part);
+    else return cudaErrorInvalidValue;
     const cudaError_t e = cudaGetLastError();
-    return e != cudaSuccess ? e : launch_wgrad_sum(part, g, 0, nullptr, part, db, s);
-}
-
-cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* db, float* part, cudaStream_t s) {
-    if (C < 8 || C % 8 != 0 || C > 256) return cudaErrorInvalidValue;
-    const int per = 256 / (C / 8);
-    long long g = (P + per - 1) / per;
-    if (g > 608) g = 608;
-    const cudaError_t e = launch_early(k_bgrad, (unsigned)g, 256, 0, s, dout, P, C, part);
-    return e != cudaSuccess ? e : launch_early(k_bgrad_sum, (C * 32 + 255) / 256, 256, 0, s, part, (int)g, C, db);
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, g, 0, nullptr, part, db, C, s);
 }
 
 cudaError_t launch_mse(const float* out, const float* target, int N, long long HW, __nv_bfloat16* dout, double* loss,

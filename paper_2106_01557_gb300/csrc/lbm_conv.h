@@ -47,19 +47,18 @@ cudaError_t launch_conv_tc(int cin, int cout, const ConvArgs& a, cudaStream_t s,
 size_t grad_scratch_floats(int sms);
 cudaError_t launch_wgrad(int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
                          int in_relu, float* dw, float* part, cudaStream_t s, int sms);
-// Weight and bias gradients of a 64 -> 64 layer on tcgen05 MMAs (lbm_wgrad64.cu;
-// the rows split over wgrad64_blocks, as launch_wgrad and launch_bgrad64 split
-// them for these layers: the same partial sums in the same order); bit 0 of
-// *status as for launch_conv_tc.
-int wgrad64_blocks(int N, int H, int W, int sms);
-cudaError_t launch_wgrad64(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W, int in_relu, float* dw,
-                           float* db, float* part, cudaStream_t s, int sms, int* status);
-cudaError_t launch_bgrad64(const __nv_bfloat16* dout, int N, int H, int W, float* db, float* part, cudaStream_t s, int sms);
+// Weight and bias gradients on tcgen05 MMAs (lbm_wgrad64.cu; the rows split over
+// wgrad_blocks, as launch_wgrad and launch_bgrad split them: the same partial
+// sums in the same order); 16 -> 64 without in_relu; bit 0 of *status as for
+// launch_conv_tc.
+int wgrad_blocks(int N, int H, int W, int sms);
+cudaError_t launch_wgrad_tc(int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
+                            int in_relu, float* dw, float* db, float* part, cudaStream_t s, int sms, int* status);
+cudaError_t launch_bgrad(const __nv_bfloat16* dout, int N, int H, int W, int C, float* db, float* part, cudaStream_t s, int sms);
 // dw[9][cc] = the sum over blocks 0 .. nblk - 1 (in a fixed order) of the
-// partials part[nblk][3 dy][3 dx][cc]; db[64] (if not null) likewise of
+// partials part[nblk][3 dy][3 dx][cc]; db[nb] (if not null) likewise of
 // bpart[nblk][64]
-cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, cudaStream_t s);
-cudaError_t launch_bgrad(const __nv_bfloat16* dout, long long P, int C, float* db, float* part, cudaStream_t s);
+cudaError_t launch_wgrad_sum(const float* part, int nblk, int cc, float* dw, const float* bpart, float* db, int nb, cudaStream_t s);
 // blocks per image of the mass layer's sums: part holds 2 MASS_BLOCKS N doubles
 constexpr int MASS_BLOCKS = 256;
 // loss partials: part holds MSE_BLOCKS doubles

@@ -168,17 +168,12 @@ static int conv(lbm_surrogate* s, int cin, int cout, const ConvArgs& a) {
 // weight and bias gradients of a layer
 static int wgrad(lbm_surrogate* s, const Layer& L, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
                  int relu) {
-    if (L.cin == 64 && L.cout == 64) {
-        if (s->cfg.conv_path == 0) {
-            SCK(launch_wgrad64(in, dout, N, H, W, relu, L.gw, L.gb, s->gpart, s->stream, s->sms, s->d_status));
-            return LBM_OK;
-        }
-        SCK(launch_wgrad(64, 64, in, dout, N, H, W, relu, L.gw, s->gpart, s->stream, s->sms));
-        SCK(launch_bgrad64(dout, N, H, W, L.gb, s->gpart, s->stream, s->sms));
+    if (s->cfg.conv_path == 0) {
+        SCK(launch_wgrad_tc(L.cin, L.cout, in, dout, N, H, W, relu, L.gw, L.gb, s->gpart, s->stream, s->sms, s->d_status));
         return LBM_OK;
     }
     SCK(launch_wgrad(L.cin, L.cout, in, dout, N, H, W, relu, L.gw, s->gpart, s->stream, s->sms));
-    SCK(launch_bgrad(dout, (long long)N * H * W, L.cout, L.gb, s->gpart, s->stream));
+    SCK(launch_bgrad(dout, N, H, W, L.cout, L.gb, s->gpart, s->stream, s->sms));
     return LBM_OK;
 }
 

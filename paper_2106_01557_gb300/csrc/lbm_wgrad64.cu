@@ -1,5 +1,5 @@
-// Weight and bias gradients of a 64 -> 64 convolution on the tensor cores,
-// warp-specialised:
+// Weight and bias gradients of the surrogate's convolutions (64 -> 64, 16 -> 64,
+// 64 -> 16) on the tensor cores, warp-specialised:
 // dW[tap (dy, dx)][co][ci] = sum over pixels p of dOut[p][co] In[p + (dy, dx)][ci]
 // (In after the ReLU the forward applied) and db[co] = sum of dOut[p][co].
 //
@@ -18,12 +18,18 @@
 //   warp 1       issues the MMAs
 //   warps 4-7    ReLU of an input row in place, where the layer wants it
 //   warps 8-11   sum the dOut rows over the pixels for the bias gradient
+//   warps 12-15  (with a 16-channel operand) copy its rows, 16 bytes at a time,
+//                into the first two chunks of 128-byte rows whose other 48
+//                channels stay zero: the MMAs and layouts are the 64 -> 64
+//                layers', three quarters of one operand idle
 //
 // What bounds it (8 x 256 x 256, 38.7 GFLOP, 134 MB): 21 us of MMAs at the
 // tensor rate, a quarter of it spent on the repeated dx = 0, and 20 us at the
 // copy bandwidth; it takes 41 us (bias included) where the kernel before it, which
 // read every dOut row three times, took 79 and the bias sums another 23: it ran
-// a block per filter row with block barriers per 128 pixels.
+// a block per filter row with block barriers per 128 pixels. The lift and the
+// projection take 43 and 44 us where that kernel and separate bias sums took 81
+// and 102.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -40,15 +46,27 @@ namespace {
 
 constexpr int W6_XS = 4;                 // input-row ring
 constexpr int W6_DS = 6;                 // dOut-row ring
-constexpr int W6_THREADS = 384;
+template <int CIN, int COUT>
+constexpr int W6_THREADS = CIN == 64 && COUT == 64 ? 384 : 512;
+constexpr int W6_AHEAD = 3;              // 16-channel rows in flight
+// Row q is handed over once row q + W6_AHEAD is issued, for which row q +
+// W6_AHEAD - (ring) has to be free: an earlier step than the first that needs
+// row q (for dOut, step q - 2) frees it.
+static_assert(W6_AHEAD < W6_XS && W6_AHEAD + 2 < W6_DS, "rings");
 constexpr int W6_OFF_D = W6_XS * C6_SLOT;
 constexpr int W6_BYTES = W6_OFF_D + W6_DS * C6_ROW + 1024;
 static_assert(W6_BYTES <= 227 * 1024 && C6_SLOT % 1024 == 0, "shared memory");
 
-__global__ void __launch_bounds__(W6_THREADS, 1)
-    k_wgrad64(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tx8,
-              const __grid_constant__ CUtensorMap td, int N, int H, int W, int in_relu, float* __restrict__ part,
-              float* __restrict__ bpart, int* __restrict__ status) {
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, int src_bytes) {  // src_bytes 0: zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(W6_THREADS<CIN, COUT>, 1)
+    k_wgrad_tc(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tx8,
+               const __grid_constant__ CUtensorMap td, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
+               int in_relu, float* __restrict__ part, float* __restrict__ bpart, int* __restrict__ status) {
+    constexpr int THREADS = W6_THREADS<CIN, COUT>;
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t xfull[W6_XS], xready[W6_XS], xempty[W6_XS], dfull[W6_DS], dempty[W6_DS], done;
     __shared__ uint32_t tmem_base;
@@ -72,15 +90,16 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
             mbar_init(&xempty[s], 1);
         }
         for (int s = 0; s < W6_DS; ++s) {
-            mbar_init(&dfull[s], 1);
+            mbar_init(&dfull[s], COUT == 64 ? 1 : 4);
             mbar_init(&dempty[s], 5);  // the MMAs and the four bias warps
         }
         mbar_init(&done, 1);
         fence_mbar_init();
         dead_flag = 0;
     }
-    // pixels past a narrow strip meet dOut zeros, but have to be finite
-    for (int e = tid; e < W6_XS * C6_SLOT / 16; e += W6_THREADS) reinterpret_cast<uint4*>(smem)[e] = make_uint4(0, 0, 0, 0);
+    // pixels past a narrow strip meet dOut zeros, but have to be finite; 16-channel rows leave the other 48 channels zero
+    for (int e = tid; e < (COUT == 64 ? W6_OFF_D : W6_OFF_D + W6_DS * C6_ROW) / 16; e += THREADS)
+        reinterpret_cast<uint4*>(smem)[e] = make_uint4(0, 0, 0, 0);
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -109,7 +128,7 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
                 r += u.L;
                 const int xl = u.x0 == 0 ? W - 8 : u.x0 - 8, xr = u.x0 + u.nv == W ? 0 : u.x0 + u.nv;
                 for (int j = 0; j < u.L + 2; ++j) {
-                    {
+                    if constexpr (COUT == 64) {
                         const unsigned s = qd % W6_DS;
                         if (qd >= W6_DS && !role_wait(&dempty[s], (qd / W6_DS - 1) & 1u, dead)) {
                             ok = false;
@@ -119,7 +138,7 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
                         tma_load_rows(sbase + W6_OFF_D + s * C6_ROW, &td, u.x0, u.n * H + R.wrap(u.y0 - 1 + j), &dfull[s]);
                         ++qd;
                     }
-                    if (j < 2) continue;
+                    if (CIN == 16 || j < 2) continue;
                     const unsigned s = qx % W6_XS;
                     if (qx >= W6_XS && !role_wait(&xempty[s], (qx / W6_XS - 1) & 1u, dead)) {
                         ok = false;
@@ -159,7 +178,7 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
                     const unsigned d = qd + li + j;
                     ok = ok && role_wait_warp(&dfull[d % W6_DS], (d / W6_DS) & 1u, dead);
                 }
-                ok = ok && role_wait_warp(in_relu ? &xready[s] : &xfull[s], (qx / W6_XS) & 1u, dead);
+                ok = ok && role_wait_warp(CIN == 16 || in_relu ? &xready[s] : &xfull[s], (qx / W6_XS) & 1u, dead);
                 if (!ok) break;
                 tc_fence_after();
                 const unsigned d0 = (qd + li) % W6_DS;
@@ -194,7 +213,7 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
         if (elect_one()) tc_commit(&done);
         __syncwarp();
     } else if (warp >= 4 && warp < 8) {
-        if (in_relu) {
+        if (CIN == 64 && in_relu) {
             const int rt = tid - 4 * 32;
             unsigned q = 0;
             bool ok = true;
@@ -217,6 +236,56 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
                 }
             }
         }
+    } else if (warp >= 12) {
+        // the rows of the 16-channel operand, 16 bytes a copy
+        const int rt = tid - 12 * 32;
+        uint64_t *const given = COUT == 16 ? dfull : xready, *const taken = COUT == 16 ? dempty : xempty;
+        constexpr unsigned RING = COUT == 16 ? W6_DS : W6_XS;
+        unsigned q = 0;  // rows issued
+        bool ok = true;
+        auto hand_over = [&](unsigned j) {  // row j has landed
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&given[j % RING]);
+        };
+        for (long long r = r_begin; r < r_end && ok;) {
+            const StripRun u = R.at(r, r_end);
+            r += u.L;
+            for (int j = 0; j < (COUT == 16 ? u.L + 2 : u.L); ++j) {
+                const unsigned s = q % RING;
+                if (q >= RING && !role_wait_warp(&taken[s], (q / RING - 1) & 1u, dead)) {
+                    ok = false;
+                    break;
+                }
+                if constexpr (COUT == 16) {  // zeros past a narrow strip
+                    const __nv_bfloat16* row = dout + ((size_t)u.n * H + R.wrap(u.y0 - 1 + j)) * W * 16;
+                    const uint32_t dst = sbase + W6_OFF_D + s * C6_ROW;
+                    for (int e = rt; e < C6_W * 2; e += 128) {
+                        const int kg = e & 1, px = e >> 1;
+                        cp16(dst + px * 128 + ((kg ^ (px & 7)) * 16), row + (size_t)(u.x0 + (px < u.nv ? px : 0)) * 16 + kg * 8,
+                             px < u.nv ? 16 : 0);
+                    }
+                } else {  // pixels -1 .. nv
+                    const __nv_bfloat16* row = in + ((size_t)u.n * H + u.y0 + j) * W * 16;
+                    const uint32_t dst = sbase + s * C6_SLOT + 1024 - 128;
+                    for (int e = rt; e < (u.nv + 2) * 2; e += 128) {
+                        const int kg = e & 1, px = e >> 1;
+                        int gx = u.x0 - 1 + px;
+                        gx = gx < 0 ? gx + W : (gx >= W ? gx - W : gx);
+                        cp16(dst + px * 128 + ((kg ^ ((px + 7) & 7)) * 16), row + (size_t)gx * 16 + kg * 8, 16);
+                    }
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                ++q;
+                if (q > W6_AHEAD) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(W6_AHEAD) : "memory");
+                    hand_over(q - 1 - W6_AHEAD);
+                }
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (ok)
+            for (unsigned j = q > W6_AHEAD ? q - W6_AHEAD : 0; j < q; ++j) hand_over(j);
     } else if (warp >= 8) {
         // 8 channels of pixels sub, sub + 16, ... (those past a narrow strip are zero)
         const int bt = tid - 8 * 32, c8 = bt % 8, sub = bt / 8;
@@ -268,21 +337,23 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
     if (warp >= 4 && warp < 8) {
         const int m = 32 * (warp % 4) + lane, ci = m % 64;
         const uint32_t tl = tmem + ((uint32_t)(32 * (warp % 4)) << 16);
-        float* pb = part + (size_t)blockIdx.x * 9 * 64 * 64;
+        float* pb = part + (size_t)blockIdx.x * 9 * COUT * CIN;
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
             if (h == 1 && warp % 4 < 2) continue;
             const int dxi = m / 64 + h;  // 0, 1, 2 for dx = -1, 0, +1
 #pragma unroll 1
-            for (int c = 0; c < 192; c += 32) {
+            for (int c = 0; c < 192; c += COUT == 64 ? 32 : 64) {
                 float v[32];
                 __syncwarp();
                 tc_ld32(tl + h * 192 + c, v);
                 tc_wait_ld(v);
                 const int by = 2 - c / 64;
-                float* o = pb + ((size_t)(by * 3 + dxi) * 64 + c % 64) * 64 + ci;
+                float* o = pb + ((size_t)(by * 3 + dxi) * COUT + c % 64) * CIN + ci;
+                if (CIN == 64 || ci < CIN) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) o[j * 64] = ok ? v[j] : 0.f;
+                    for (int j = 0; j < (COUT < 32 ? COUT : 32); ++j) o[j * CIN] = ok ? v[j] : 0.f;
+                }
             }
         }
     }
@@ -298,21 +369,38 @@ __global__ void __launch_bounds__(W6_THREADS, 1)
 
 }  // namespace
 
-cudaError_t launch_wgrad64(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W, int in_relu, float* dw,
-                           float* db, float* part, cudaStream_t s, int sms, int* status) {
-    if (N < 1 || H < 1 || W < 16 || W % 16 != 0 || !status || sms < 1) return cudaErrorInvalidValue;
+namespace {
+
+template <int CIN, int COUT>
+cudaError_t wgrad_tc_t(const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W, int in_relu, float* dw, float* db,
+                       float* part, cudaStream_t s, int sms, int* status) {
     const long long rows = (long long)N * H;
     if (rows >= (1ll << 31)) return cudaErrorInvalidValue;
-    CUtensorMap tx, tx8, td;
-    cudaError_t e = encode_rows64(in, rows, W, C6_W, &tx);
-    if (e == cudaSuccess) e = encode_rows64(in, rows, W, 8, &tx8);
-    if (e == cudaSuccess) e = encode_rows64(dout, rows, W, C6_W, &td);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad64, cudaFuncAttributeMaxDynamicSharedMemorySize, W6_BYTES);
+    CUtensorMap tx{}, tx8{}, td{};
+    cudaError_t e = cudaSuccess;
+    if (CIN == 64) {
+        e = encode_rows64(in, rows, W, C6_W, &tx);
+        if (e == cudaSuccess) e = encode_rows64(in, rows, W, 8, &tx8);
+    }
+    if (e == cudaSuccess && COUT == 64) e = encode_rows64(dout, rows, W, C6_W, &td);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, W6_BYTES);
     if (e != cudaSuccess) return e;
-    const int grid = wgrad64_blocks(N, H, W, sms);
-    float* bpart = part + (size_t)grid * 9 * 64 * 64;
-    e = launch_early(k_wgrad64, grid, W6_THREADS, W6_BYTES, s, tx, tx8, td, N, H, W, in_relu, part, bpart, status);
-    return e != cudaSuccess ? e : launch_wgrad_sum(part, grid, 64 * 64, dw, bpart, db, s);
+    const int grid = wgrad_blocks(N, H, W, sms);
+    float* bpart = part + (size_t)grid * 9 * COUT * CIN;
+    e = launch_early(k_wgrad_tc<CIN, COUT>, grid, W6_THREADS<CIN, COUT>, W6_BYTES, s, tx, tx8, td, in, dout, N, H, W, in_relu, part,
+                     bpart, status);
+    return e != cudaSuccess ? e : launch_wgrad_sum(part, grid, COUT * CIN, dw, bpart, db, COUT, s);
+}
+
+}  // namespace
+
+cudaError_t launch_wgrad_tc(int cin, int cout, const __nv_bfloat16* in, const __nv_bfloat16* dout, int N, int H, int W,
+                            int in_relu, float* dw, float* db, float* part, cudaStream_t s, int sms, int* status) {
+    if (N < 1 || H < 1 || W < 16 || W % 16 != 0 || !status || sms < 1) return cudaErrorInvalidValue;
+    if (cin == 64 && cout == 64) return wgrad_tc_t<64, 64>(in, dout, N, H, W, in_relu, dw, db, part, s, sms, status);
+    if (cin == 16 && cout == 64 && !in_relu) return wgrad_tc_t<16, 64>(in, dout, N, H, W, in_relu, dw, db, part, s, sms, status);
+    if (cin == 64 && cout == 16) return wgrad_tc_t<64, 16>(in, dout, N, H, W, in_relu, dw, db, part, s, sms, status);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace lbm
