@@ -61,15 +61,13 @@ __global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch
             if (lane == 0) atomicOr(B.status, ST_TIMEOUT);
             break;
         }
-        float v[7];
-        reduce_record(acc, v);
-        if (lane == 0) {
-            v[1] *= cs.kf.c;
-            v[2] *= cs.kf.c;
-            v[5] *= cs.kf.c2;
-            if (v[6] > 0.f) atomicOr(B.status, ST_NONFINITE);
-#pragma unroll
-            for (int q = 0; q < 7; ++q) B.partials[(size_t)item * 8 + q] = v[q];
+        const int q = lane / 4;
+        float v = reduce_record(acc, lane);
+        if (q == 1 || q == 2) v *= cs.kf.c;
+        if (q == 5) v *= cs.kf.c2;
+        if (lane % 4 == 0 && q < 7) {
+            if (q == 6 && v > 0.f) atomicOr(B.status, ST_NONFINITE);
+            B.partials[(size_t)item * 8 + q] = v;
         }
     }
     if (gw == 0 && lane == 0) {

@@ -236,6 +236,14 @@ __device__ __forceinline__ void moments_of(const C l[9], const R* rest, C m[9]) 
     }
 }
 
+// moment 0 alone, the same bits
+template <bool SH, class C, class R>
+__device__ __forceinline__ C density_of(const C l[9], const R* rest) {
+    const C m0 = (((l[1] + l[3]) + (l[2] + l[4])) + ((l[5] + l[7]) + (l[6] + l[8]))) + l[0];
+    if constexpr (SH) return m0 + rest[0];
+    else return m0;
+}
+
 // The macroscopic state from the moments s.m and s.n and the density around
 // the node.
 template <class C, class K>
@@ -273,6 +281,14 @@ __device__ __forceinline__ void node_macro(const K& k, const C f[9], const C g[9
 template <class C>
 __device__ __forceinline__ bool bad_node(C rho, C T, C u2) {
     return !(rho > C(0) && rho < C(1e30) && T > C(0) && T < C(1e30) && u2 < C(1e30));
+}
+// (FP64 comparisons go through the FP64 unit; bit patterns order as the values
+// do, with the negative ones, infinity and NaN above all positive ones, and
+// zero wrapped around to the top)
+__device__ __forceinline__ bool bad_node(double rho, double T, double u2) {
+    const unsigned long long lim = 0x46293e5939a08ceaull;  // 1e30
+    const unsigned long long r = (unsigned long long)__double_as_longlong(rho) - 1, t = (unsigned long long)__double_as_longlong(T) - 1;
+    return !(r < lim - 1 && t < lim - 1 && (unsigned long long)__double_as_longlong(u2) < lim);
 }
 
 // p_BE = p_EOS + a rho^2 with Eq. 17

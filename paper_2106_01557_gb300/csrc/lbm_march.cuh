@@ -156,19 +156,33 @@ __device__ __forceinline__ void record(const K& k, const V rn[9], const NodeMacr
     acc.u2max = vmax(acc.u2max, u2);
 }
 
-// the lanes' sums of a record, reduced over the warp (lane 0 holds the result)
+// The lanes' sums of a record, reduced over the warp: lanes 4 q .. 4 q + 3 hold
+// quantity q (7: nothing). Each of the first three exchanges halves the
+// quantities a lane still carries, so 9 additions take the place of 35: a
+// twelfth of a one-row warp's FP64 operations.
 template <class C>
-__device__ __forceinline__ void reduce_record(const Rec<C>& acc, C v[7]) {
+__device__ __forceinline__ C reduce_record(const Rec<C>& acc, int lane) {
+    C v[8];
     const C* a = &acc.mass;
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        v[q] = a[q];
+    for (int q = 0; q < 7; ++q) v[q] = a[q];
+    v[7] = C(0);
+    auto join = [](C x, C y, bool largest) { return largest ? (y > x ? y : x) : x + y; };  // (quantity 5 is a maximum)
+    bool five = true;  // is place `at` quantity 5 if the lane keeps it?
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const C w = __shfl_down_sync(0xffffffffu, v[q], o);
-            v[q] = (q == 5) ? (w > v[q] ? w : v[q]) : v[q] + w;
+    for (int s = 16, n = 4; s >= 4; s >>= 1, n >>= 1) {
+        const bool up = lane & s;
+        five = five && up == ((5 & n) != 0);
+#pragma unroll
+        for (int j = 0; j < n; ++j) {
+            const C w = __shfl_xor_sync(0xffffffffu, up ? v[j] : v[n + j], s);
+            const C x = up ? v[n + j] : v[j];
+            v[j] = j == (5 & (n - 1)) ? join(x, w, five) : x + w;
         }
     }
+#pragma unroll
+    for (int s = 2; s >= 1; s >>= 1) v[0] = join(v[0], __shfl_xor_sync(0xffffffffu, v[0], s), five);
+    return v[0];
 }
 
 // the constants a step computes with
@@ -297,8 +311,7 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
         hn = halo_load();
         V l[9];
         rm.get(l);
-        moments_of<SH>(l, kv.mrest, mn);
-        dm = dens(mn[0], halo_sum(hm));
+        dm = dens(density_of<SH>(l, kv.mrest), halo_sum(hm));
         rc.get(l);
         moments_of<SH>(l, kv.mrest, mn);
         dc = dens(mn[0], halo_sum(hc));
@@ -321,7 +334,9 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
 #pragma unroll
             for (int i = 0; i < 9; ++i) s.m[i] = mn[i];
             rf.get(l);
-            moments_of<SH>(l, kv.mrest, mn);
+            // beyond the run only the density is wanted: worth a branch in FP64
+            if (sizeof(C) < 8 || y + 1 < w.y1) moments_of<SH>(l, kv.mrest, mn);
+            else mn[0] = density_of<SH>(l, kv.mrest);
             rg.get(l);
             moments_of<SH>(l, kv.nrest, s.n);
         }
