@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "lbm_device.cuh"
+#include "lbm_ptx.cuh"
 
 namespace lbm {
 
@@ -93,19 +94,8 @@ struct NodeAt {
         for (int i = 0; i < 9; ++i) {
             const S v = __ldg(buf + from(p, i));
             if constexpr (sizeof(S) == 8) l[i] = v;
-            else l[i] = widen<C>(Store<S, float>::raw(v));
-        }
-    }
-    // float to C. To FP64 by integer arithmetic, exact: the conversion unit
-    // takes a warp's worth every 16 cycles, as FP64 arithmetic does.
-    template <class C>
-    static __device__ __forceinline__ C widen(float v) {
-        if constexpr (sizeof(C) == 4) {
-            return v;
-        } else {
-            const uint32_t u = __float_as_uint(v), a = u << 1;
-            if (a - 0x01000000u >= 0xfe000000u) return (double)v;  // zero, subnormal, infinite or NaN
-            return __hiloint2double((int)((u & 0x80000000u) | ((a >> 4) + 0x38000000u)), (int)(u << 29));
+            else if constexpr (sizeof(C) == 8) l[i] = widen(Store<S, float>::raw(v));
+            else l[i] = Store<S, float>::raw(v);
         }
     }
 };

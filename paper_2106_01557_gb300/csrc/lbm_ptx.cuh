@@ -1,5 +1,6 @@
-// Inline-PTX helpers of the asynchronous pipelines: shared-memory addresses, the
-// global timer for bounded waits, mbarrier set-up / arrive / try-wait.
+// Helpers of several kernels: shared-memory addresses, the global timer for
+// bounded waits, mbarrier set-up / arrive / try-wait, and conversions between
+// FP32 and FP64.
 #pragma once
 
 #include <stdint.h>
@@ -46,6 +47,29 @@ static __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t par
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
+}
+
+// float <-> double by integer arithmetic, the same bits as the conversions: the
+// conversion unit takes a warp every 16 cycles, as FP64 arithmetic does, the
+// integer units eight operations in that time on each of the four schedulers.
+// (Values out of the normal FP32 range are left to the unit.)
+// (The unit's conversions are calls: as predicated instructions they would take
+// their cycles on the path that skips them too.)
+static __device__ __noinline__ double widen_unit(float v) { return (double)v; }
+static __device__ __noinline__ float narrow_unit(double v) { return (float)v; }
+static __device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), a = u << 1;
+    if (a - 0x01000000u >= 0xfe000000u) return widen_unit(v);  // zero, subnormal, infinite or NaN
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 4) + 0x38000000u)), (int)(u << 29));
+}
+static __device__ __forceinline__ float narrow(double v) {  // to nearest, ties to even
+    const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+    const uint32_t a = h & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x0fd00000u) return narrow_unit(v);  // below 2^-126, or 2^127 and more
+    // the exponent and the upper 23 bits of the fraction; the 29 below round
+    const uint32_t m = ((a - 0x38000000u) << 3) | (l >> 29), rest = l << 3;
+    const uint32_t up = (rest > 0x80000000u || (rest == 0x80000000u && (m & 1u))) ? 1u : 0u;
+    return __uint_as_float((h & 0x80000000u) | (m + up));
 }
 
 }  // namespace lbm
