@@ -15,7 +15,6 @@
 #include <type_traits>
 
 #include "lbm_device.cuh"
-#include "lbm_ptx.cuh"
 
 namespace lbm {
 
@@ -94,8 +93,7 @@ struct NodeAt {
         for (int i = 0; i < 9; ++i) {
             const S v = __ldg(buf + from(p, i));
             if constexpr (sizeof(S) == 8) l[i] = v;
-            else if constexpr (sizeof(C) == 8) l[i] = widen(Store<S, float>::raw(v));
-            else l[i] = Store<S, float>::raw(v);
+            else l[i] = (C)Store<S, float>::raw(v);
         }
     }
 };
