@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(32 * BatchCfg<S>::W, BatchCfg<S>::BPS) k_batch
         G.lsw = Cf::NPL == 2 ? 6 : 5;  // (known here, so that the compiler knows them too; a batch's cases are periodic)
         G.walls = G.open = 0;
         Rec<float> acc = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (!march_rows<S, float, false, false>(cs.kf, march_constants<V>(cs), G, w, acc)) {
+        if (!march_rows<S, float, false, false, true>(cs.kf, march_constants<V>(cs), G, w, acc)) {
             if (lane == 0) atomicOr(B.status, ST_TIMEOUT);
             break;
         }

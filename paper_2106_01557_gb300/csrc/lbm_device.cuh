@@ -89,16 +89,10 @@ __device__ __forceinline__ uint32_t fmix32(uint32_t h) {
     return h;
 }
 
-// The nine (f_i, g_i) pairs of a node converted with stochastic rounding
-// from the node's seed h (cvt_sr2: the upper 16 bits round f_i, the lower
-// 16 bits g_i).
-template <class S, class C>
-__device__ __forceinline__ void cvt_sr_node(const C f[9], const C g[9], uint32_t h, S sf[9], S sg[9]) {
-    constexpr uint32_t K[9] = {0x9e3779b1u, 0x85ebca77u, 0xc2b2ae3du, 0x27d4eb2fu, 0x165667b1u,
-                               0xd3a2646du, 0xfd7046c5u, 0xb55a4f09u, 0x61c88647u};
-#pragma unroll
-    for (int i = 0; i < 9; ++i) Store<S, C>::cvt_sr2(f[i], g[i], h * K[i], sf[i], sg[i]);
-}
+// The factors of the words that round a node's nine pairs (f_i, g_i), f_i by the
+// upper 16 bits.
+__device__ constexpr uint32_t NODE_DITHER_K[9] = {0x9e3779b1u, 0x85ebca77u, 0xc2b2ae3du, 0x27d4eb2fu, 0x165667b1u,
+                                                  0xd3a2646du, 0xfd7046c5u, 0xb55a4f09u, 0x61c88647u};
 
 // Reciprocal: IEEE in FP64; in FP32 the hardware approximation (relative
 // error ~1e-7, far below the FP32 path's 1e-5 parity bound).

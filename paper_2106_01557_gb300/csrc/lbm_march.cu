@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
         w.wait_ns = L.tile_wait_ns;
         w.sr = Store<S, C>::SHIFTED && L.rounding;
         w.steps = cnt_in;
-        if (!march_rows<S, C, OPEN, CUBIC>(k, march_constants<V>(L), G, w, acc) && lane == 0) atomicOr(status, ST_TIMEOUT);
+        if (!march_rows<S, C, OPEN, CUBIC, OPEN || CUBIC>(k, march_constants<V>(L), G, w, acc) && lane == 0) atomicOr(status, ST_TIMEOUT);
     } else {
         after_previous_grid();
     }

@@ -29,7 +29,7 @@
 // density pass and a block barrier per tile): FP32 115.0 -> 105.3 (5.74 TB/s;
 // what is left is mostly the memory mix: without the collision it takes 104.6),
 // FP16 107.5 -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with
-// launches that overlap (lbm_launch.cuh) 104.2 and 81.8.
+// launches that overlap (lbm_launch.cuh) and the later changes 103.9 and 81.2.
 // Tried for the rows: a ring of tensor-copied boxes per warp (124, whatever the
 // depth: about 10 cycles of the copy engine per line of 128 bytes), 16-byte
 // asynchronous copies into a shared-memory ring (124: bound by the shared-
@@ -69,6 +69,7 @@ struct MarchCfg {
 // A step is launched while the step before it still runs (lbm_launch.cuh), so
 // its loads of the state are ordinary ones: the read-only path (__ldg, or a
 // restricted pointer) is for memory that nobody writes while the kernel lives.
+
 // The nine populations of one DF pulled at this lane's node(s), as stored.
 // c, l, r: the DF's line 0 in the pulling row, at the lane's (first) column,
 // the column left of it and the column right of its last.
@@ -213,7 +214,8 @@ struct Strip {
 // Rows y0 .. y1 - 1 of a strip. False if the wait for the first rows ran out
 // (nothing is stored then).
 // kv: the constants in the arithmetic's type (k, or both lanes of k).
-template <class S, class C, bool OPEN, bool CUBIC, class K>
+// NODE_DITHER: stochastic rounding from every node's own seed, not the pair's.
+template <class S, class C, bool OPEN, bool CUBIC, bool NODE_DITHER, class K>
 __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Geometry& G, const Strip<S, C>& w,
                                            Rec<C>& acc) {
     using Cf = MarchCfg<S>;
@@ -388,7 +390,17 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
         W wv[18];
         if constexpr (NPL == 2) {
             using PW = PairWord<S>;
-            if (w.sr) {
+            if (NODE_DITHER && w.sr) {
+                // from each node's own seed: a word for the pair (f_i, g_i)
+                const uint32_t h0 = fmix32((uint32_t)(y * G.nx + x) ^ step_key), h1 = fmix32((uint32_t)(y * G.nx + x + 1) ^ step_key);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    const uint32_t r0 = h0 * NODE_DITHER_K[i], r1 = h1 * NODE_DITHER_K[i];
+                    wv[i] = PW::sr(f[i], __byte_perm(r0, r1, 0x7632));
+                    wv[9 + i] = PW::sr(g[i], __byte_perm(r0, r1, 0x5410));
+                }
+            } else if (w.sr) {
+                // from the pair's seed: a word for each population
                 const uint32_t h = fmix32((uint32_t)(y * G.nx + x) ^ step_key);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
