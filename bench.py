@@ -127,11 +127,11 @@ class ClockSampler:
 
 METRIC = "MLUPS of the fused f+g step (FP32 plain)"
 
-# DRAM bytes (read + write) of one k_step launch on this workload, from one
-# ncu capture (profiles/k_step_f32_4096x1024_full.md), valid only for the
+# DRAM bytes (read + write) of one k_march launch on this workload, from one
+# ncu capture (profiles/k_march.md), valid only for the
 # kernel sources it was taken on: any change to them makes it null.
-STEP_TRAFFIC = {"bytes_per_launch": (309391616 + 255389184 + 308886528 + 253282560) // 2,
-                "sources_sha256": "22adc04600794184e7f2dc0308ed44331d9bf8cfaa462689084fc037aff67e11"}
+STEP_TRAFFIC = {"bytes_per_launch": (310760000 + 257460000 + 310790000 + 255060000) // 2,
+                "sources_sha256": "d171edcbc0b1b939d2cd6b9ed556c9a31774b64470a0837d2e8b29f4187e1abb"}
 STEP_SOURCES = ["lbm_march.cu", "lbm_march.cuh", "lbm_store.cuh", "lbm_device.cuh", "lbm_internal.h"]
 
 

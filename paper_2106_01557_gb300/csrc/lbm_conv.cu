@@ -714,13 +714,6 @@ cudaError_t launch_mass_layer(const float* y, const float* x, const float* t, in
     return e != cudaSuccess ? e : launch_early(k_mass_sums, (32 * N + 127) / 128, 128, 0, s, part, N, (int)gx, (int)(t != nullptr), sums);
 }
 
-size_t conv_smem_bytes(int cin, int cout) {
-    if (cin == 16 && cout == 64) return ConvSmem<16, 64>::BYTES;
-    if (cin == 64 && cout == 64) return ConvSmem<64, 64>::BYTES;
-    if (cin == 64 && cout == 16) return ConvSmem<64, 16>::BYTES;
-    return 0;
-}
-
 cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms) {
     if (a.W % 16 != 0) return cudaErrorInvalidValue;
     if (cin == 16 && cout == 64) return conv_t<16, 64>(a, s, sms);

@@ -33,7 +33,6 @@ struct ConvArgs {
     unsigned long long* obits;    // [P]: set to the sign bits (> 0) of the BF16 output before its ReLU (or null)
 };
 
-size_t conv_smem_bytes(int cin, int cout);
 cudaError_t launch_conv(int cin, int cout, const ConvArgs& a, cudaStream_t s, int sms);
 // The same convolution on tcgen05 MMAs with tensor-memory accumulators,
 // warp-specialised (lbm_conv_tc.cu): 64 -> 64 and 16 -> 64 (without in_relu) to

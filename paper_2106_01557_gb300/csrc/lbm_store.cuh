@@ -54,18 +54,11 @@ __device__ __noinline__ void wall_store(S* __restrict__ out, const Geometry& G, 
     }
 }
 
-// One population of a node pair (x even, x + 1) as stored: a 64-bit word of
-// two FP32 values, or a 32-bit word of two 16-bit values with node x in the
-// low half; nearest rounding (rn) or stochastic (sr, 32 random bits: the
+// One population of a node pair (x even, x + 1) as stored: a 32-bit word of two
+// 16-bit values with node x in the low half; nearest rounding (rn) or stochastic (sr, 32 random bits: the
 // upper 16 drive node x + 1, the lower 16 node x).
 template <class S>
 struct PairWord;
-template <>
-struct PairWord<float> {
-    using W = float2;
-    static __device__ __forceinline__ W rn(F2 v) { return v.v; }
-    static __device__ __forceinline__ W sr(F2 v, uint32_t) { return v.v; }
-};
 template <>
 struct PairWord<__half> {
     using W = uint32_t;
