@@ -677,7 +677,7 @@ static cudaError_t step_once(lbm_handle* h, int from, bool first, bool last) {
         phi = h->scratch + n;
     }
     MarchGrid mg = h->grid;
-    mg.combine_prev = first ? 0 : 1;
+    if (first) mg.combine_prev = 0;
     mg.combine_here = last ? 1 : 0;
     return launch_march(h->storage, h->L, h->buf[from], h->buf[1 - from], mg, h->partials + from * h->part_stride, h->partials + (1 - from) * h->part_stride, h->stats,
                         h->count(from), h->count(1 - from), h->counter, h->status, h->stream, phi);

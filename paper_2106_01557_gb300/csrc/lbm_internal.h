@@ -106,11 +106,11 @@ cudaError_t launch_cubic_phi(int storage, const Launch& L, const void* buf, doub
 // strips each across x, `chunks` chunks of rows.
 struct MarchGrid {
     int groups, warps, chunks;
-    int combine_prev;  // an extra block combines the record of the step before (prev)
+    int combine_prev;  // that many extra blocks combine the record of the step before (prev)
     int combine_here;  // the last block to finish combines this step's record
 };
 int march_strip(int storage);  // width of a warp's strip
-MarchGrid march_grid(int storage, const Geometry& g);
+MarchGrid march_grid(int storage, const Geometry& g);  // with combine_prev as a step after another takes it
 // partials: [groups * chunks][NQ]; cnt_in, cnt_out: the step count before and
 // after the step (two places, so that every block can read it); phi: with
 // L.cubic, [2][ny][nx] rho u_x^3 and rho u_y^3 (u over c) of the state

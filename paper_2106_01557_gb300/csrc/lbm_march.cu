@@ -6,7 +6,7 @@
 // sectors two strips share are in the L2 cache when the second one asks.
 //
 // The conservation record of a step (per-block FP64 partial sums) is combined
-// by an extra block of the next step's launch, off the critical path, or,
+// by extra blocks of the next step's launch, off the critical path, or,
 // where no step follows in the call, by the last block to finish.
 #include "lbm_march.cuh"
 
@@ -21,9 +21,13 @@ namespace {
 __device__ __forceinline__ void combine_record(const double* partials, int nblk, double* stats, int warp, int nw, int lane) {
     for (int q = warp; q < 7; q += nw) {
         double t = 0.0;
-        for (int b = lane; b < nblk; b += 32) {
-            const double pv = __ldcg(partials + (size_t)b * NQ + q);
-            t = (q == 5) ? fmax(t, pv) : t + pv;
+        for (int b = lane; b < nblk; b += 32 * 8) {
+            double pv[8];  // eight loads in flight
+#pragma unroll
+            for (int j = 0; j < 8; ++j) pv[j] = b + 32 * j < nblk ? __ldcg(partials + (size_t)(b + 32 * j) * NQ + q) : 0.0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (b + 32 * j < nblk) t = (q == 5) ? fmax(t, pv[j]) : t + pv[j];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -56,13 +60,13 @@ __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nw = blockDim.x / 32;
     int block = blockIdx.x;
     if (mg.combine_prev) {
-        // block 0: the record of the step before this one
-        if (block == 0) {
+        // the first blocks: the record of the step before this one
+        if (block < mg.combine_prev) {
             after_previous_grid();
-            combine_record(prev, mg.groups * mg.chunks, stats, warp, nw, lane);
+            combine_record(prev, mg.groups * mg.chunks, stats, warp + block * nw, nw * mg.combine_prev, lane);
             return;
         }
-        block -= 1;
+        block -= mg.combine_prev;
     }
     const int group = block % mg.groups, chunk = block / mg.groups;
     Strip<S, C> w;
@@ -119,7 +123,7 @@ template <class S, class C>
 cudaError_t march_t(const Launch& L, const void* in, void* out, const MarchGrid& mg,
                     double* partials, const double* prev, double* stats, const double* cnt_in, double* cnt_out,
                     unsigned* counter, int* status, cudaStream_t s, const double* phi) {
-    const dim3 grid((unsigned)(mg.groups * mg.chunks + (mg.combine_prev ? 1 : 0))), blk((unsigned)(32 * mg.warps));
+    const dim3 grid((unsigned)(mg.groups * mg.chunks + mg.combine_prev)), blk((unsigned)(32 * mg.warps));
     const S* i = static_cast<const S*>(in);
     S* o = static_cast<S*>(out);
     auto* const kernel = L.geo.open ? k_march<S, C, true, false> : (L.cubic ? k_march<S, C, false, true> : k_march<S, C, false, false>);
@@ -132,29 +136,45 @@ int march_strip(int storage) {
     return storage == S_F64 ? MarchCfg<double>::SW : (storage == S_F32 ? MarchCfg<float>::SW : MarchCfg<__half>::SW);
 }
 
+// Blocks of w warps that combine a record, a warp per quantity: with one block, and
+// one load at a time, they ran longer than the step of a lattice of up to about
+// 300 x 300 (FP32: 300 x 300 9.1 -> 6.5 us per step, 224 x 224 8.4 -> 4.8, 128 x
+// 128 4.23 -> 3.92, 40 x 40 7.3 -> 3.6, 96 x 500 17.3 -> 5.4).
+static int combine_blocks(int w) { return (7 + w - 1) / w; }
+
 MarchGrid march_grid(int storage, const Geometry& g) {
     const int sw = march_strip(storage);
     const int bps = storage == S_F64 ? MarchCfg<double>::BPS : (storage == S_F32 ? MarchCfg<float>::BPS : MarchCfg<__half>::BPS);
     const int strips = (g.nx + sw - 1) / sw;
-    MarchGrid m;
-    m.groups = (strips + MW - 1) / MW;
-    m.warps = (strips + m.groups - 1) / m.groups;
-    // as many chunks of rows as fill one wave of resident blocks, which the
-    // block that combines the last record is part of
-    int chunks = (bps * g.sms - 1) / m.groups;
-    if (chunks > g.ny) chunks = g.ny;
-    if (chunks < 1) chunks = 1;
+    // Blocks of w adjacent strips, and as many chunks of rows as fill one wave of
+    // resident blocks, which the blocks that combine the last record are part of.
+    // w is the largest for which the longest chunk is shortest: with 4 warps, 22
+    // strips leave 2 of 24 idle, and 5 strips a quarter of every SM's, as blocks
+    // of 3 count as blocks of 4 (1363 x 777 in BF16 27.4 -> 25.8 us per step, 900 x
+    // 2000 43.2 -> 41.1, 160 x 900 in FP32 13.3 -> 7.7, 40 x 3000 in FP16 24.6 ->
+    // 11.0).
+    MarchGrid m{};
+    int chunks = 0, rows = 0;
+    for (int w = MW; w >= 2; --w) {
+        const int groups = (strips + w - 1) / w, warps = (strips + groups - 1) / groups;
+        int n = (bps * MW / w * g.sms - combine_blocks(warps)) / groups;
+        n = n > g.ny ? g.ny : (n < 1 ? 1 : n);
+        const int longest = (g.ny + n - 1) / n;
+        if (rows == 0 || longest < rows) {
+            rows = longest;
+            chunks = n;
+            m.groups = groups;
+            m.warps = warps;
+        }
+    }
     // In FP32, which waits for memory, as few chunks as keep the longest as it
     // is: fewer rows read twice (512 x 512: 10.5 us per step with 151 chunks of 3
     // or 4 rows, 9.6 with 128 of 4). In 16-bit storage and FP64 the warps of the
     // shorter chunks leave the arithmetic to the others (512 x 512 in FP16 10.45
     // and 10.8 us, 1363 x 777 in BF16 27.5 and 28.0).
-    if (storage == S_F32) {
-        const int rows = (g.ny + chunks - 1) / chunks;
-        chunks = (g.ny + rows - 1) / rows;
-    }
+    if (storage == S_F32) chunks = (g.ny + rows - 1) / rows;
     m.chunks = chunks;
-    m.combine_prev = m.combine_here = 0;
+    m.combine_prev = combine_blocks(m.warps);
     return m;
 }
 

@@ -172,3 +172,27 @@ def test_fields_in_and_out_match_oracle(gpu_lib, nx, ny, opts, prec):
         assert max(abs(got[1] - want[1]), abs(got[2] - want[2])) < tol * want[0] * o.p.c
         if "open_sides" not in opts:  # (the oracle's total energy takes the density beyond an open side for a wall's)
             assert abs(got[4] - want[4]) < tol * abs(want[3])
+
+
+# 1, 2, 3, 5 and 6 strips, in blocks of 1 to 4 warps: the blocks that combine the
+# record of the step before, and the last block, take its quantities in shares
+@pytest.mark.parametrize("prec,tol", [("f64", 1e-12), ("f32", 1e-5), ("f16s", 1e-3)])
+@pytest.mark.parametrize("nx,ny", [(20, 400), (64, 33), (96, 500), (160, 90), (320, 40)])
+def test_record_of_narrow_lattices(gpu_lib, nx, ny, prec, tol):
+    from paper_2106_01557_gb300 import lbm
+    o = oracle_case(nx, ny)
+    fields = slab_fields(o, seed=31, eps=0.01, uamp=0.005)
+    for n in (1, 2, 21, 40):
+        g, h = (lbm.Lattice.create(nx, ny, precision=prec) for _ in range(2))
+        for lat in (g, h):
+            lat.set_fields(*fields)
+        g.step(n)
+        for _ in range(n):
+            h.step(1)
+        got = g.step_stats()
+        # the record of a step is that of the state it began with, whichever block adds it up
+        assert np.array_equal(got, h.step_stats()) and got[7] == n
+        f = g.get_populations()[0]
+        assert abs(got[0] / f.sum() - 1) < tol
+        g.close()
+        h.close()
