@@ -1,4 +1,4 @@
-// What the warp-specialised 64 -> 64 kernels share: the cut of an image into
+// What the surrogate's warp-specialised kernels share: the cut of an image into
 // strips of rows, tensor copies of pixel rows, and the bounded waits of roles.
 #pragma once
 

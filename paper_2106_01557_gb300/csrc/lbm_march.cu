@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(32 * MW, MarchCfg<S>::BPS)
     __shared__ C red[MW][7];
     __shared__ bool last;
     // 16-bit storage, which is short of issue slots, gains from a strip width
-    // that the compiler knows (4096 x 1024 in FP16 82.2 -> 81.1 us); FP32 loses
+    // that the compiler knows (4096 x 1024 in FP16 82.2 -> 81.1 us when it came in); FP32 loses
     // (103.8 -> 104.2) by the copy that the calls for the edges then take
     typename std::conditional<Cf::NPL == 2, Geometry, const Geometry&>::type G = L.geo;
     if constexpr (Cf::NPL == 2) G.lsw = 6;

@@ -29,7 +29,7 @@
 // density pass and a block barrier per tile): FP32 115.0 -> 105.3 (5.74 TB/s;
 // what is left is mostly the memory mix: without the collision it takes 104.6),
 // FP16 107.5 -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with
-// launches that overlap (lbm_launch.cuh) and the later changes 103.9 and 81.2.
+// launches that overlap (lbm_launch.cuh) and the later changes 103.6 and 79.6.
 // Tried for the rows: a ring of tensor-copied boxes per warp (124, whatever the
 // depth: about 10 cycles of the copy engine per line of 128 bytes), 16-byte
 // asynchronous copies into a shared-memory ring (124: bound by the shared-
