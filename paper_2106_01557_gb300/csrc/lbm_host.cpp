@@ -664,9 +664,7 @@ int lbm_get_populations(lbm_handle* h, double* f, double* g) {
     return check_status(h);
 }
 
-// One step from buffer `from`. last: no step follows it in this call, so the
-// step combines its own record; otherwise the next step does. first: the
-// record of the step before is combined already.
+// One step from buffer `from`; first, last: of step_grid.
 static cudaError_t step_once(lbm_handle* h, int from, bool first, bool last) {
     const double* phi = nullptr;
     if (h->L.cubic) {
@@ -676,10 +674,7 @@ static cudaError_t step_once(lbm_handle* h, int from, bool first, bool last) {
         if (e != cudaSuccess) return e;
         phi = h->scratch + n;
     }
-    MarchGrid mg = h->grid;
-    if (first) mg.combine_prev = 0;
-    mg.combine_here = last ? 1 : 0;
-    return launch_march(h->storage, h->L, h->buf[from], h->buf[1 - from], mg, h->partials + from * h->part_stride, h->partials + (1 - from) * h->part_stride, h->stats,
+    return launch_march(h->storage, h->L, h->buf[from], h->buf[1 - from], step_grid(h->grid, first, last), h->partials + from * h->part_stride, h->partials + (1 - from) * h->part_stride, h->stats,
                         h->count(from), h->count(1 - from), h->counter, h->status, h->stream, phi);
 }
 

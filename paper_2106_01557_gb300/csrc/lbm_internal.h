@@ -111,6 +111,16 @@ struct MarchGrid {
 };
 int march_strip(int storage);  // width of a warp's strip
 MarchGrid march_grid(int storage, const Geometry& g);  // with combine_prev as a step after another takes it
+// The grid of one step of a call. first: the record of the step before is
+// combined already; last: no step follows in the call, so this one combines its
+// own record. A launch has one writer of the record: the blocks that combine the
+// record before run unordered beside the block that combines this one, and what
+// they would write is replaced by it.
+inline MarchGrid step_grid(MarchGrid m, bool first, bool last) {
+    if (first || last) m.combine_prev = 0;
+    m.combine_here = last ? 1 : 0;
+    return m;
+}
 // partials: [groups * chunks][NQ]; cnt_in, cnt_out: the step count before and
 // after the step (two places, so that every block can read it); phi: with
 // L.cubic, [2][ny][nx] rho u_x^3 and rho u_y^3 (u over c) of the state
