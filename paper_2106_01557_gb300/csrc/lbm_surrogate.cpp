@@ -85,6 +85,7 @@ struct lbm_surrogate {
     double* pred = nullptr;
     double* ver = nullptr;           // the verified state's fields
     unsigned long long* d_chg = nullptr;  // field change of a verification (4 maxima)
+    long long field_cap = 0;         // pixels these hold
     void* snapshot = nullptr;
     size_t snapshot_bytes = 0;
     long long step_count = 0;        // Adam steps
@@ -528,9 +529,13 @@ int lbm_surrogate_rollout(lbm_surrogate* s, lbm_handle* h, int32_t njumps, int32
     rc = ensure_acts(s, P, false);
     if (rc) return rc;
     const size_t sb = lbm_internal_state_bytes(h);
-    if (!s->fields || s->snapshot_bytes < sb) {
+    // (the bytes of a state are not in proportion to its nodes: strips, ghosts and
+    // storage differ from handle to handle)
+    if (s->field_cap < P || s->snapshot_bytes < sb) {
         s_free(s->fields); s_free(s->pred); s_free(s->ver); s_free(s->snapshot); s_free(s->d_chg);
         s->fields = s->pred = s->ver = nullptr; s->snapshot = nullptr; s->d_chg = nullptr;
+        s->field_cap = 0;
+        s->snapshot_bytes = 0;
         if (cudaMalloc(&s->fields, 4 * P * 8) != cudaSuccess || cudaMalloc(&s->pred, 4 * P * 8) != cudaSuccess ||
             cudaMalloc(&s->ver, 4 * P * 8) != cudaSuccess ||
             cudaMalloc(&s->d_chg, 4 * sizeof(unsigned long long)) != cudaSuccess ||
@@ -538,6 +543,7 @@ int lbm_surrogate_rollout(lbm_surrogate* s, lbm_handle* h, int32_t njumps, int32
             cudaGetLastError();
             return sfail(LBM_ERR_OOM, "rollout buffers");
         }
+        s->field_cap = P;
         s->snapshot_bytes = sb;
     }
     double acc = 0, fb = 0, t_sur = 0, t_lb = 0, max_dm = 0, max_de = 0;
