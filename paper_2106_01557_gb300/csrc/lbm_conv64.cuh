@@ -57,7 +57,9 @@ __device__ __forceinline__ void tma_store_rows(const CUtensorMap* tm, int x, int
 }
 
 // Wait for a phase of bar, bounded; false after the bound, or once another
-// role has given up (dead is set for all).
+// role has given up (dead is set for all). For a single lane: lanes of a warp
+// that wait each for itself can part when the bound is near, and the ones that go
+// on would wait without a bound at the next instruction of the whole warp.
 __device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
@@ -69,7 +71,9 @@ __device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, volati
     }
     return true;
 }
-// the same for a converged warp: one outcome for all lanes
+// the same for a converged warp: one outcome for all lanes. (Warps of a group
+// that meet at a barrier in between can still differ: the ones that give up go
+// on to the barrier, group_any.)
 __device__ __forceinline__ bool role_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
     return __all_sync(0xffffffffu, role_wait(bar, parity, dead));
 }

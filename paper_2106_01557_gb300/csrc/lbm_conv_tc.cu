@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
                 const int nvec = (u.nv + 2) * 8;
                 for (int li = 0; li < u.L + 2; ++li, ++q) {
                     const unsigned s = q % C6_SLOTS;
-                    if (!role_wait(&full[s], (q / C6_SLOTS) & 1u, dead)) {
+                    if (!role_wait_warp(&full[s], (q / C6_SLOTS) & 1u, dead)) {
                         ok = false;
                         break;
                     }
@@ -383,8 +383,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
             if constexpr (COUT == 16) {  // the first four channels in FP32, a pixel per thread
                 float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (res32 && px < c.u.nv) o = res32[pix];
-                if (!role_wait(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
-                __syncwarp();
+                if (!role_wait_warp(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
                 tc_fence_after();
                 float v[16];
                 tc_ld<16>(t_lane + (tt % C6_BLK) * 16u, v);
@@ -404,66 +403,71 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
             } else {
                 uint2 mw = make_uint2(0xffffffffu, 0xffffffffu);
                 if (mbits && px < c.u.nv) mw = mbits[pix];
-                if (!role_wait(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
-                __syncwarp();
-                tc_fence_after();
-                float v[64];
-                tc_ld32(t_lane + (tt % C6_BLK) * 64u, v);
-                tc_ld32(t_lane + (tt % C6_BLK) * 64u + 32u, v + 32);
-                tc_wait_ld(v);
-                tc_st_zero32(t_lane + (tt % C6_BLK) * 64u);
-                tc_st_zero32(t_lane + (tt % C6_BLK) * 64u + 32u);
-                tc_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty[tt % C6_BLK]);
-                if (with_res && !role_wait(&side[grp][k & 1u], (k >> 1) & 1u, dead)) break;
-                unsigned char* orow = smem + stage(k) + px * 128;
-                uint32_t bits[2] = {0u, 0u};
-    #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    float* x = v + 8 * q;
-                    const int at = (q ^ (px & 7)) * 16;
-    #pragma unroll
-                    for (int j = 0; j < 8; j += 4) {
-                        const float4 b = *reinterpret_cast<const float4*>(s_bias + 8 * q + j);
-                        x[j] += b.x;
-                        x[j + 1] += b.y;
-                        x[j + 2] += b.z;
-                        x[j + 3] += b.w;
-                    }
-                    if (mbits) {
-                        // bit j of a word: channel 2 j of its 32, bit 16 + j: channel 2 j + 1
-                        const uint32_t m = q < 4 ? mw.x : mw.y;
-    #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (!(m & (1u << (4 * (q & 3) + j)))) x[2 * j] = 0.f;
-                            if (!(m & (0x10000u << (4 * (q & 3) + j)))) x[2 * j + 1] = 0.f;
+                // A warp whose wait runs out skips the row, but not the barrier that
+                // ends it: the group leaves together.
+                bool failed = true;
+                do {
+                    if (!role_wait_warp(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
+                    tc_fence_after();
+                    float v[64];
+                    tc_ld32(t_lane + (tt % C6_BLK) * 64u, v);
+                    tc_ld32(t_lane + (tt % C6_BLK) * 64u + 32u, v + 32);
+                    tc_wait_ld(v);
+                    tc_st_zero32(t_lane + (tt % C6_BLK) * 64u);
+                    tc_st_zero32(t_lane + (tt % C6_BLK) * 64u + 32u);
+                    tc_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[tt % C6_BLK]);
+                    if (with_res && !role_wait_warp(&side[grp][k & 1u], (k >> 1) & 1u, dead)) break;
+                    unsigned char* orow = smem + stage(k) + px * 128;
+                    uint32_t bits[2] = {0u, 0u};
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        float* x = v + 8 * q;
+                        const int at = (q ^ (px & 7)) * 16;
+#pragma unroll
+                        for (int j = 0; j < 8; j += 4) {
+                            const float4 b = *reinterpret_cast<const float4*>(s_bias + 8 * q + j);
+                            x[j] += b.x;
+                            x[j + 1] += b.y;
+                            x[j + 2] += b.z;
+                            x[j + 3] += b.w;
                         }
+                        if (mbits) {
+                            // bit j of a word: channel 2 j of its 32, bit 16 + j: channel 2 j + 1
+                            const uint32_t m = q < 4 ? mw.x : mw.y;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                if (!(m & (1u << (4 * (q & 3) + j)))) x[2 * j] = 0.f;
+                                if (!(m & (0x10000u << (4 * (q & 3) + j)))) x[2 * j + 1] = 0.f;
+                            }
+                        }
+                        if (with_res) {
+                            const uint4 m = *reinterpret_cast<const uint4*>(orow + at);
+                            const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(&m);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) x[j] += __bfloat162float(mh[j]);
+                        }
+                        uint4 o;
+                        __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+                        if (obits) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                bits[q / 4] |= __hgt2_mask(oh[j], __floats2bfloat162_rn(0.f, 0.f)) & (0x10001u << (4 * (q & 3) + j));
+                        }
+                        if (out_relu) o = relu8(o);
+                        *reinterpret_cast<uint4*>(orow + at) = o;
                     }
-                    if (with_res) {
-                        const uint4 m = *reinterpret_cast<const uint4*>(orow + at);
-                        const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(&m);
-    #pragma unroll
-                        for (int j = 0; j < 8; ++j) x[j] += __bfloat162float(mh[j]);
-                    }
-                    uint4 o;
-                    __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
-    #pragma unroll
-                    for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-                    if (obits) {
-    #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            bits[q / 4] |= __hgt2_mask(oh[j], __floats2bfloat162_rn(0.f, 0.f)) & (0x10001u << (4 * (q & 3) + j));
-                    }
-                    if (out_relu) o = relu8(o);
-                    *reinterpret_cast<uint4*>(orow + at) = o;
-                }
-                if (obits && px < c.u.nv) obits[pix] = make_uint2(bits[0], bits[1]);
+                    if (obits && px < c.u.nv) obits[pix] = make_uint2(bits[0], bits[1]);
+                    failed = false;
+                } while (false);
                 Rows d = c;  // the row after this one
                 d.t += 2;
                 settle(d);
-                if (leader) {
+                if (leader && !failed) {
                     // the other staging row is free once the store before has been read
                     bulk_wait_read0();
                     if (with_res && d.more) {
@@ -472,7 +476,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
                     }
                 }
                 fence_proxy_async();
-                group_sync(grp);
+                if (group_any(grp, failed)) break;
                 if (leader) {
                     const int row = c.u.n * H + c.u.y0 + c.t;
                     const uint32_t src = sbase + stage(k);

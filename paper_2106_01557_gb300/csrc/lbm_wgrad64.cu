@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(W6_THREADS<CIN, COUT>, 1)
                 const int nvec = (u.nv + 2) * 8;  // pixels -1 .. nv of the strip, 8 vectors each
                 for (int li = 0; li < u.L; ++li, ++q) {
                     const unsigned s = q % W6_XS;
-                    if (!role_wait(&xfull[s], (q / W6_XS) & 1u, dead)) {
+                    if (!role_wait_warp(&xfull[s], (q / W6_XS) & 1u, dead)) {
                         ok = false;
                         break;
                     }
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(W6_THREADS<CIN, COUT>, 1)
             r += u.L;
             for (int j = 0; j < u.L + 2; ++j, ++q) {
                 const unsigned s = q % W6_DS;
-                if (!role_wait(&dfull[s], (q / W6_DS) & 1u, dead)) {
+                if (!role_wait_warp(&dfull[s], (q / W6_DS) & 1u, dead)) {
                     ok = false;
                     break;
                 }
@@ -329,9 +329,9 @@ __global__ void __launch_bounds__(W6_THREADS<CIN, COUT>, 1)
     __syncwarp();
     bool ok = true;
     if (warp >= 4 && warp < 8) {
-        ok = role_wait(&done, 0u, dead);
+        ok = role_wait_warp(&done, 0u, dead);
         if (!ok) land(&done, 0u);
-        ok = __all_sync(0xffffffffu, ok);
+        __syncwarp();
     }
     tc_fence_after();
     if (warp >= 4 && warp < 8) {
