@@ -11,13 +11,14 @@ namespace lbm {
 // Wall ghost-row stores of a node next to a wall: the populations leaving
 // through the wall come back reversed at the next pull (half-way bounce-back
 // of f; of g adiabatic, or anti-bounce-back on a fixed-temperature segment).
-// fo0.., go0..: the post-collision populations, as stored, of the three
-// directions that leave through the wall: (4, 7, 8) at the bottom, (2, 5, 6) at
-// the top. Opposite directions have equal rest populations, so for shifted
-// formats too a reversed population is stored as it is.
+// fo0.., go0..: the post-collision populations (for shifted formats, their
+// deviations from the rest populations) of the three directions that leave
+// through the wall: (4, 7, 8) at the bottom, (2, 5, 6) at the top. They come in
+// the arithmetic's precision and are rounded once, to nearest. Opposite
+// directions have equal rest populations.
 template <class S, class C, bool OPEN>
 __device__ __noinline__ void wall_store(S* __restrict__ out, const Geometry& G, const KC<C>& k, int x, int y,
-                                        S fo0, S fo1, S fo2, S go0, S go1, S go2, C rho) {
+                                        C fo0, C fo1, C fo2, C go0, C go1, C go2, C rho) {
     constexpr int SW = sizeof(S) == 2 ? 64 : 32;  // a line's elements
     const bool bottom = (y == 0);
     const int yg = bottom ? -1 : G.ny;
@@ -30,8 +31,8 @@ __device__ __noinline__ void wall_store(S* __restrict__ out, const Geometry& G, 
         const int opp = bottom ? (j == 0 ? 2 : (j == 1 ? 5 : 6)) : (j == 0 ? 4 : (j == 1 ? 7 : 8));
         // x step of the leaving direction: 0 for 4/2; 7 and 6 go left, 8 and 5 right
         const int ex = j == 0 ? 0 : (bottom ? (j == 1 ? -1 : 1) : (j == 1 ? 1 : -1));
-        const S fv = j == 0 ? fo0 : (j == 1 ? fo1 : fo2);
-        S gv = j == 0 ? go0 : (j == 1 ? go1 : go2);
+        const S fv = Store<S, C>::cvt(j == 0 ? fo0 : (j == 1 ? fo1 : fo2));
+        C go = j == 0 ? go0 : (j == 1 ? go1 : go2);
         int xg = x + ex;
         xg = xg < 0 ? xg + G.nx : (xg >= G.nx ? xg - G.nx : xg);
         C T_link = Tw;
@@ -41,8 +42,9 @@ __device__ __noinline__ void wall_store(S* __restrict__ out, const Geometry& G, 
         }
         if (T_link > C(0)) {
             const C rest = Store<S, C>::SHIFTED ? k.rest[9 + opp] : C(0);
-            gv = Store<S, C>::st(C(2) * T_link * (j == 0 ? ga1 : gd1) - Store<S, C>::ld(gv, rest), rest);
+            go = (C(2) * T_link * (j == 0 ? ga1 : gd1) - (go + rest)) - rest;
         }
+        const S gv = Store<S, C>::cvt(go);
         S* const q = out + G.at(opp, xg, yg);
         q[0] = fv;
         q[9 * SW] = gv;
