@@ -26,7 +26,7 @@ struct BatchLaunch {
     const int* first;
     int nitems, warps;
     const BatchCase* cases;
-    float* partials;          // [nitems][8]
+    double* partials;         // [nitems][8]
     int* status;
     double* steps;            // [2] by buffer: steps executed (keys stochastic rounding)
     int rounding;             // 16-bit storage: 0 nearest, 1 stochastic

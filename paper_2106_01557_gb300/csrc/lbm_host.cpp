@@ -924,7 +924,7 @@ struct lbm_batch {
     int max_items = 0, warps = 0;
     std::vector<BatchItem> items[2][3];  // [shape][order], the warps' lists one after another
     std::vector<int> first[2][3];        // where each warp's list begins (and where the last ends)
-    float* d_partials = nullptr;
+    double* d_partials = nullptr;
     int* d_status = nullptr;
     int* h_status = nullptr;  // pinned: its copy after a call
     double* d_steps = nullptr;   // step count as of arena 0 and of arena 1 (keys stochastic rounding)
@@ -1134,7 +1134,7 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
               cudaMalloc(&b->d_cases, ncases * sizeof(BatchCase)) == cudaSuccess &&
               cudaMalloc(&b->d_first, ((size_t)b->warps + 1) * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&b->d_items, (size_t)b->max_items * sizeof(BatchItem)) == cudaSuccess &&
-              cudaMalloc(&b->d_partials, (size_t)b->max_items * 8 * sizeof(float)) == cudaSuccess &&
+              cudaMalloc(&b->d_partials, (size_t)b->max_items * 8 * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&b->d_status, sizeof(int)) == cudaSuccess &&
               cudaMallocHost(&b->h_status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&b->d_rec, 16 * sizeof(double)) == cudaSuccess &&
@@ -1151,7 +1151,7 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
     ok = cudaMemcpy(b->d_cases, hc.data(), ncases * sizeof(BatchCase), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(b->arena[0], 0, abytes) == cudaSuccess && cudaMemset(b->arena[1], 0, abytes) == cudaSuccess &&
          cudaMemset(b->d_status, 0, sizeof(int)) == cudaSuccess &&
-         cudaMemset(b->d_partials, 0, (size_t)b->max_items * 8 * sizeof(float)) == cudaSuccess &&
+         cudaMemset(b->d_partials, 0, (size_t)b->max_items * 8 * sizeof(double)) == cudaSuccess &&
          cudaMemset(b->aux_counter, 0, sizeof(unsigned)) == cudaSuccess &&
          cudaMemset(b->d_steps, 0, 2 * sizeof(double)) == cudaSuccess;
     if (!ok) { batch_release(b); delete b; return fail(LBM_ERR_CUDA, "device initialisation failed"); }

@@ -215,9 +215,13 @@ struct Strip {
 // (nothing is stored then).
 // kv: the constants in the arithmetic's type (k, or both lanes of k).
 // NODE_DITHER: stochastic rounding from every node's own seed, not the pair's.
-template <class S, class C, bool OPEN, bool CUBIC, bool NODE_DITHER, class K>
+// flush(acc): called after every 16 rows and after the last, where runs can be
+// long, to carry the lanes' sums on in more bits. (Between two loops over rows: as
+// a branch of the loop it costs twice the time.)
+struct NoFlush {};
+template <class S, class C, bool OPEN, bool CUBIC, bool NODE_DITHER, class K, class Flush = NoFlush>
 __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Geometry& G, const Strip<S, C>& w,
-                                           Rec<C>& acc) {
+                                           Rec<C>& acc, Flush flush = Flush()) {
     using Cf = MarchCfg<S>;
     constexpr int NPL = Cf::NPL, SW = Cf::SW, ROW = Cf::ROW;
     using V = typename std::conditional<NPL == 2, F2, C>::type;
@@ -328,187 +332,193 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
     // nodes with copies in the ghost columns
     const bool xg = v0 && xper && (x < GHOST_COLS || x + NPL > G.nx - GHOST_COLS);
 
+    int y = w.y0;
 #pragma unroll 1
-    for (int y = w.y0; y < w.y1; ++y) {
-        V rn[9];
-        {
-            V l[9];
+    do {
+        const int ye = std::is_same<Flush, NoFlush>::value || w.y1 - y <= 16 ? w.y1 : y + 16;
+#pragma unroll 1
+        for (; y < ye; ++y) {
+            V rn[9];
+            {
+                V l[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) s.m[i] = mn[i];
-            rf.get(l);
-            // beyond the run only the density is wanted: worth a branch in FP64
-            if (sizeof(C) < 8 || y + 1 < w.y1) moments_of<SH>(l, kv.mrest, mn);
-            else mn[0] = density_of<SH>(l, kv.mrest);
-            rg.get(l);
-            moments_of<SH>(l, kv.nrest, s.n);
-        }
-        const S hcur = hn;
-        if (y + 1 < w.y1) {
-            rg.load(pc + 9 * SW, pl + 9 * SW, pr + 9 * SW);
-            next_row();
-            rf.load(pc, pl, pr);
-            hn = halo_load();
-        }
-        Dens dp = dens(mn[0], halo_sum(hcur));
-        if (y == G.ny - 1 && G.walls) {
-            if (OPEN && (G.open & 2)) dp = dopen;
-            else dp = dc;
-        }
-        rn[0] = dc.at();
-        rn[1] = dc.r;
-        rn[2] = dp.at();
-        rn[3] = dc.l;
-        rn[4] = dm.at();
-        rn[5] = dp.r;
-        rn[6] = dp.l;
-        rn[7] = dm.l;
-        rn[8] = dm.r;
-        dm = dc;
-        dc = dp;
-        macro_of(kv, rn, s);
-        if (v0) record(kv, rn, s, v1, acc);
-        V R7 = V(0);
-        if constexpr (CUBIC) {
-            // -c (d_x(rho u_x^3) - d_y(rho u_y^3)), periodic central differences
-            const long long n = (long long)G.nx * G.ny;
-            const int ym = y == 0 ? G.ny - 1 : y - 1, yp = y == G.ny - 1 ? 0 : y + 1;
-            auto r7 = [&](int xq) {
-                xq = xq < G.nx ? xq : G.nx - 1;
-                const int xm = xq == 0 ? G.nx - 1 : xq - 1, xp = xq == G.nx - 1 ? 0 : xq + 1;
-                const double dpx = 0.5 * (__ldcg(w.phi + (long long)y * G.nx + xp) - __ldcg(w.phi + (long long)y * G.nx + xm));
-                const double dpy = 0.5 * (__ldcg(w.phi + n + (long long)yp * G.nx + xq) - __ldcg(w.phi + n + (long long)ym * G.nx + xq));
-                return -k.c * ((C)dpx - (C)dpy);
-            };
-            if constexpr (NPL == 2) R7 = F2(r7(x), r7(x + 1));
-            else R7 = r7(x);
-        }
-        V f[9], g[9];
-        collide<SH, CUBIC>(kv, f, g, s, R7);
-
-        // ---- next to a wall: the reflections this node owns -----------------
-        // From the values of the collision, so before the row is rounded, where
-        // the values are no longer needed; not with open sides, whose ghosts need
-        // them to the end (512 x 512 in FP32: 2 - 3% slower there).
-        auto reflect = [&]() {
-            if (!(G.walls && (y == 0 || y == G.ny - 1) && v0)) return;
-#pragma unroll
-            for (int q = 0; q < NPL; ++q) {
-                if (q == 1 && !v1) break;
-                auto of = [&](V v) -> C {
-                    if constexpr (NPL == 2) return q ? v.v.y : v.v.x;
-                    else return v;
-                };
-                // (a side that is open has its own ghosts instead)
-                if (y == 0 && !(OPEN && (G.open & 1)))
-                    wall_store<S, C, OPEN>(w.out, G, k, x + q, y, of(f[4]), of(f[7]), of(f[8]), of(g[4]), of(g[7]), of(g[8]), of(s.rho));
-                if (y == G.ny - 1 && !(OPEN && (G.open & 2)))
-                    wall_store<S, C, OPEN>(w.out, G, k, x + q, y, of(f[2]), of(f[5]), of(f[6]), of(g[2]), of(g[5]), of(g[6]), of(s.rho));
+                for (int i = 0; i < 9; ++i) s.m[i] = mn[i];
+                rf.get(l);
+                // beyond the run only the density is wanted: worth a branch in FP64
+                if (sizeof(C) < 8 || y + 1 < w.y1) moments_of<SH>(l, kv.mrest, mn);
+                else mn[0] = density_of<SH>(l, kv.mrest);
+                rg.get(l);
+                moments_of<SH>(l, kv.nrest, s.n);
             }
-        };
-        if constexpr (!OPEN) reflect();
-        // ---- the row as stored ----------------------------------------------
-        using W = typename std::conditional<NPL == 2, uint32_t, S>::type;  // a lane's share of a line
-        W wv[18];
-        if constexpr (NPL == 2) {
-            using PW = PairWord<S>;
-            if (NODE_DITHER && w.sr) {
-                // from each node's own seed: a word for the pair (f_i, g_i)
-                const uint32_t h0 = fmix32((uint32_t)(y * G.nx + x) ^ step_key), h1 = fmix32((uint32_t)(y * G.nx + x + 1) ^ step_key);
+            const S hcur = hn;
+            if (y + 1 < w.y1) {
+                rg.load(pc + 9 * SW, pl + 9 * SW, pr + 9 * SW);
+                next_row();
+                rf.load(pc, pl, pr);
+                hn = halo_load();
+            }
+            Dens dp = dens(mn[0], halo_sum(hcur));
+            if (y == G.ny - 1 && G.walls) {
+                if (OPEN && (G.open & 2)) dp = dopen;
+                else dp = dc;
+            }
+            rn[0] = dc.at();
+            rn[1] = dc.r;
+            rn[2] = dp.at();
+            rn[3] = dc.l;
+            rn[4] = dm.at();
+            rn[5] = dp.r;
+            rn[6] = dp.l;
+            rn[7] = dm.l;
+            rn[8] = dm.r;
+            dm = dc;
+            dc = dp;
+            macro_of(kv, rn, s);
+            if (v0) record(kv, rn, s, v1, acc);
+            V R7 = V(0);
+            if constexpr (CUBIC) {
+                // -c (d_x(rho u_x^3) - d_y(rho u_y^3)), periodic central differences
+                const long long n = (long long)G.nx * G.ny;
+                const int ym = y == 0 ? G.ny - 1 : y - 1, yp = y == G.ny - 1 ? 0 : y + 1;
+                auto r7 = [&](int xq) {
+                    xq = xq < G.nx ? xq : G.nx - 1;
+                    const int xm = xq == 0 ? G.nx - 1 : xq - 1, xp = xq == G.nx - 1 ? 0 : xq + 1;
+                    const double dpx = 0.5 * (__ldcg(w.phi + (long long)y * G.nx + xp) - __ldcg(w.phi + (long long)y * G.nx + xm));
+                    const double dpy = 0.5 * (__ldcg(w.phi + n + (long long)yp * G.nx + xq) - __ldcg(w.phi + n + (long long)ym * G.nx + xq));
+                    return -k.c * ((C)dpx - (C)dpy);
+                };
+                if constexpr (NPL == 2) R7 = F2(r7(x), r7(x + 1));
+                else R7 = r7(x);
+            }
+            V f[9], g[9];
+            collide<SH, CUBIC>(kv, f, g, s, R7);
+
+            // ---- next to a wall: the reflections this node owns -----------------
+            // From the values of the collision, so before the row is rounded, where
+            // the values are no longer needed; not with open sides, whose ghosts need
+            // them to the end (512 x 512 in FP32: 2 - 3% slower there).
+            auto reflect = [&]() {
+                if (!(G.walls && (y == 0 || y == G.ny - 1) && v0)) return;
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    const uint32_t r0 = h0 * NODE_DITHER_K[i], r1 = h1 * NODE_DITHER_K[i];
-                    wv[i] = PW::sr(f[i], __byte_perm(r0, r1, 0x7632));
-                    wv[9 + i] = PW::sr(g[i], __byte_perm(r0, r1, 0x5410));
+                for (int q = 0; q < NPL; ++q) {
+                    if (q == 1 && !v1) break;
+                    auto of = [&](V v) -> C {
+                        if constexpr (NPL == 2) return q ? v.v.y : v.v.x;
+                        else return v;
+                    };
+                    // (a side that is open has its own ghosts instead)
+                    if (y == 0 && !(OPEN && (G.open & 1)))
+                        wall_store<S, C, OPEN>(w.out, G, k, x + q, y, of(f[4]), of(f[7]), of(f[8]), of(g[4]), of(g[7]), of(g[8]), of(s.rho));
+                    if (y == G.ny - 1 && !(OPEN && (G.open & 2)))
+                        wall_store<S, C, OPEN>(w.out, G, k, x + q, y, of(f[2]), of(f[5]), of(f[6]), of(g[2]), of(g[5]), of(g[6]), of(s.rho));
                 }
-            } else if (w.sr) {
-                // from the pair's seed: a word for each population
-                const uint32_t h = fmix32((uint32_t)(y * G.nx + x) ^ step_key);
+            };
+            if constexpr (!OPEN) reflect();
+            // ---- the row as stored ----------------------------------------------
+            using W = typename std::conditional<NPL == 2, uint32_t, S>::type;  // a lane's share of a line
+            W wv[18];
+            if constexpr (NPL == 2) {
+                using PW = PairWord<S>;
+                if (NODE_DITHER && w.sr) {
+                    // from each node's own seed: a word for the pair (f_i, g_i)
+                    const uint32_t h0 = fmix32((uint32_t)(y * G.nx + x) ^ step_key), h1 = fmix32((uint32_t)(y * G.nx + x + 1) ^ step_key);
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    wv[i] = PW::sr(f[i], h * (0x9e3779b9u * (2u * i + 1u)));
-                    wv[9 + i] = PW::sr(g[i], h * (0x9e3779b9u * (2u * i + 19u)));
+                    for (int i = 0; i < 9; ++i) {
+                        const uint32_t r0 = h0 * NODE_DITHER_K[i], r1 = h1 * NODE_DITHER_K[i];
+                        wv[i] = PW::sr(f[i], __byte_perm(r0, r1, 0x7632));
+                        wv[9 + i] = PW::sr(g[i], __byte_perm(r0, r1, 0x5410));
+                    }
+                } else if (w.sr) {
+                    // from the pair's seed: a word for each population
+                    const uint32_t h = fmix32((uint32_t)(y * G.nx + x) ^ step_key);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        wv[i] = PW::sr(f[i], h * (0x9e3779b9u * (2u * i + 1u)));
+                        wv[9 + i] = PW::sr(g[i], h * (0x9e3779b9u * (2u * i + 19u)));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        wv[i] = PW::rn(f[i]);
+                        wv[9 + i] = PW::rn(g[i]);
+                    }
                 }
             } else {
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    wv[i] = PW::rn(f[i]);
-                    wv[9 + i] = PW::rn(g[i]);
+                    wv[i] = Store<S, C>::cvt(f[i]);
+                    wv[9 + i] = Store<S, C>::cvt(g[i]);
                 }
             }
-        } else {
+            S* const o = po;
+            po += ROW;
+            if (NPL == 1 ? v0 : v1) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                wv[i] = Store<S, C>::cvt(f[i]);
-                wv[9 + i] = Store<S, C>::cvt(g[i]);
+                for (int i = 0; i < 18; ++i) *reinterpret_cast<W*>(o + i * SW) = wv[i];
             }
-        }
-        S* const o = po;
-        po += ROW;
-        if (NPL == 1 ? v0 : v1) {
-#pragma unroll
-            for (int i = 0; i < 18; ++i) *reinterpret_cast<W*>(o + i * SW) = wv[i];
-        }
-        // rows next to the periodic seam also have a copy beyond it
-        int dup = 0;
-        if (!G.walls) dup = y < 2 ? G.ny : (y >= G.ny - 2 ? -G.ny : 0);
-        if (v0 && (xg || dup || (NPL == 2 && !v1))) {
+            // rows next to the periodic seam also have a copy beyond it
+            int dup = 0;
+            if (!G.walls) dup = y < 2 ? G.ny : (y >= G.ny - 2 ? -G.ny : 0);
+            if (v0 && (xg || dup || (NPL == 2 && !v1))) {
 #pragma unroll 1
-            for (int r = 0; r < 2; ++r) {
-                if (r == 1 && !dup) break;
-                const int yr = y + (r ? dup : 0);
-                S* q = w.out + G.at(0, x, yr);
-                S* ql = w.out + G.at(0, x < GHOST_COLS ? x + G.nx : x - G.nx, yr);                   // copy of node x
-                S* qr = w.out + G.at(0, x + 1 < GHOST_COLS ? x + 1 + G.nx : x + 1 - G.nx, yr);       // of node x + 1
-                const bool cl = xper && (x < GHOST_COLS || x >= G.nx - GHOST_COLS);
-                const bool cr = NPL == 2 && xper && v1 && (x + 1 < GHOST_COLS || x + 1 >= G.nx - GHOST_COLS);
+                for (int r = 0; r < 2; ++r) {
+                    if (r == 1 && !dup) break;
+                    const int yr = y + (r ? dup : 0);
+                    S* q = w.out + G.at(0, x, yr);
+                    S* ql = w.out + G.at(0, x < GHOST_COLS ? x + G.nx : x - G.nx, yr);                   // copy of node x
+                    S* qr = w.out + G.at(0, x + 1 < GHOST_COLS ? x + 1 + G.nx : x + 1 - G.nx, yr);       // of node x + 1
+                    const bool cl = xper && (x < GHOST_COLS || x >= G.nx - GHOST_COLS);
+                    const bool cr = NPL == 2 && xper && v1 && (x + 1 < GHOST_COLS || x + 1 >= G.nx - GHOST_COLS);
 #pragma unroll
-                for (int i = 0; i < 18; ++i) {
-                    if constexpr (NPL == 2) {
-                        const unsigned short lo = (unsigned short)(wv[i] & 0xffffu), hi = (unsigned short)(wv[i] >> 16);
-                        unsigned short* h = reinterpret_cast<unsigned short*>(q + i * SW);
-                        h[0] = lo;
-                        if (v1) h[1] = hi;
-                        if (cl) *reinterpret_cast<unsigned short*>(ql + i * SW) = lo;
-                        if (cr) *reinterpret_cast<unsigned short*>(qr + i * SW) = hi;
-                    } else {
-                        if (r) q[i * SW] = wv[i];
-                        if (cl) ql[i * SW] = wv[i];
+                    for (int i = 0; i < 18; ++i) {
+                        if constexpr (NPL == 2) {
+                            const unsigned short lo = (unsigned short)(wv[i] & 0xffffu), hi = (unsigned short)(wv[i] >> 16);
+                            unsigned short* h = reinterpret_cast<unsigned short*>(q + i * SW);
+                            h[0] = lo;
+                            if (v1) h[1] = hi;
+                            if (cl) *reinterpret_cast<unsigned short*>(ql + i * SW) = lo;
+                            if (cr) *reinterpret_cast<unsigned short*>(qr + i * SW) = hi;
+                        } else {
+                            if (r) q[i * SW] = wv[i];
+                            if (cl) ql[i * SW] = wv[i];
+                        }
+                    }
+                }
+            }
+            // ---- next to an open side: the ghosts this node owns ----------------
+            if constexpr (OPEN) {
+                reflect();
+                if (v0 && (((G.open & 1) && y == 0) || ((G.open & 2) && y == G.ny - 1) || ((G.open & 4) && x == 0) ||
+                           ((G.open & 8) && x + NPL >= G.nx))) {
+#pragma unroll
+                    for (int q = 0; q < NPL; ++q) {
+                        const int xq = x + q;
+                        if (!(((G.open & 1) && y == 0) || ((G.open & 2) && y == G.ny - 1) || ((G.open & 4) && xq == 0) ||
+                              ((G.open & 8) && xq == G.nx - 1)) || xq >= G.nx)
+                            continue;
+                        Pops9<C> pf, pg;
+                        if constexpr (NPL == 2) {
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) {
+                                pf.v[i] = q ? f[i].v.y : f[i].v.x;
+                                pg.v[i] = q ? g[i].v.y : g[i].v.x;
+                            }
+                            if (q == 0) open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho.v.x, s.uhx.v.x, s.uhy.v.x, s.T.v.x);
+                            else open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho.v.y, s.uhx.v.y, s.uhy.v.y, s.T.v.y);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) {
+                                pf.v[i] = f[i];
+                                pg.v[i] = g[i];
+                            }
+                            open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho, s.uhx, s.uhy, s.T);
+                        }
                     }
                 }
             }
         }
-        // ---- next to an open side: the ghosts this node owns ----------------
-        if constexpr (OPEN) {
-            reflect();
-            if (v0 && (((G.open & 1) && y == 0) || ((G.open & 2) && y == G.ny - 1) || ((G.open & 4) && x == 0) ||
-                       ((G.open & 8) && x + NPL >= G.nx))) {
-#pragma unroll
-                for (int q = 0; q < NPL; ++q) {
-                    const int xq = x + q;
-                    if (!(((G.open & 1) && y == 0) || ((G.open & 2) && y == G.ny - 1) || ((G.open & 4) && xq == 0) ||
-                          ((G.open & 8) && xq == G.nx - 1)) || xq >= G.nx)
-                        continue;
-                    Pops9<C> pf, pg;
-                    if constexpr (NPL == 2) {
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) {
-                            pf.v[i] = q ? f[i].v.y : f[i].v.x;
-                            pg.v[i] = q ? g[i].v.y : g[i].v.x;
-                        }
-                        if (q == 0) open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho.v.x, s.uhx.v.x, s.uhy.v.x, s.T.v.x);
-                        else open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho.v.y, s.uhx.v.y, s.uhy.v.y, s.T.v.y);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) {
-                            pf.v[i] = f[i];
-                            pg.v[i] = g[i];
-                        }
-                        open_store<S, C>(w.out, G, k, xq, y, pf, pg, s.rho, s.uhx, s.uhy, s.T);
-                    }
-                }
-            }
-        }
-    }
+        if constexpr (!std::is_same<Flush, NoFlush>::value) flush(acc);
+    } while (!std::is_same<Flush, NoFlush>::value && y < w.y1);
     return true;
 }
 
