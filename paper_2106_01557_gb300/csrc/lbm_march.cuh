@@ -124,13 +124,14 @@ struct Rec {
     C mass, mx, my, ek, et, u2max, bad;
 };
 
-// a value of a node, or of a node pair: the sum, the larger and the lane's own
+// a value of a node, or of a node pair: the sum, and the larger of a and it (a
+// where it is NaN: the record's largest speed is that of the nodes that have one)
 __device__ __forceinline__ float vsum(float a) { return a; }
 __device__ __forceinline__ double vsum(double a) { return a; }
 __device__ __forceinline__ float vsum(F2 a) { return a.v.x + a.v.y; }
-__device__ __forceinline__ float vmax(float a, float b) { return a > b ? a : b; }
-__device__ __forceinline__ double vmax(double a, double b) { return a > b ? a : b; }
-__device__ __forceinline__ float vmax(float a, F2 b) { return vmax(a, vmax(b.v.x, b.v.y)); }
+__device__ __forceinline__ float vmax(float a, float b) { return b > a ? b : a; }
+__device__ __forceinline__ double vmax(double a, double b) { return b > a ? b : a; }
+__device__ __forceinline__ float vmax(float a, F2 b) { return vmax(vmax(a, b.v.x), b.v.y); }
 // Conservation record of the entering state at a node, or a node pair whose
 // second node lies in the lattice if v1. The total energy rho e_k - a rho^2 -
 // kappa / 2 rho lap(rho), lap = 2 (axes / 3 + diagonals / 12 - 5 rho / 3).
