@@ -20,6 +20,16 @@ static __device__ __forceinline__ uint64_t globaltimer_ns() {
     return t;
 }
 
+// The timer once x is there: the read is predicated on x, so that it waits for
+// the loads x was formed from. (t where x is -1e30, which no density is.)
+static __device__ __forceinline__ uint64_t globaltimer_ns_after(float x, uint64_t t) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.neu.f32 p, %1, 0fF149F2CA;\n\t@p mov.u64 %0, %%globaltimer;\n\t}" : "+l"(t) : "f"(x));
+    return t;
+}
+static __device__ __forceinline__ uint64_t globaltimer_ns_after(double x, uint64_t t) {
+    return globaltimer_ns_after(__int_as_float(__double2hiint(x)), t);
+}
+
 static __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
