@@ -371,6 +371,35 @@ __global__ void __launch_bounds__(RECORD ? AUX_NT : FIELD_NT)
     }
 }
 
+// Elements of a checkpoint file's planes from and into the strips, a thread per
+// element of the file. Bound by the copy to or from the host (4096 x 1024 in FP32:
+// save 118 -> 65 ms, load 140 -> 36 ms against rows copied by the host).
+template <class E, bool SAVE>
+__global__ void __launch_bounds__(AUX_NT) k_file(const Geometry G, const FilePlanes F, E* __restrict__ state, long long e, long long n,
+                                                 E* __restrict__ file) {
+    for (long long i = blockIdx.x * (long long)AUX_NT + threadIdx.x; i < n; i += (long long)gridDim.x * AUX_NT) {
+        const long long row = (e + i) / F.pitch;
+        const int x = (int)((e + i) - row * F.pitch) - F.px, p = (int)(row / F.nyp), y = (int)(row - (long long)p * F.nyp) - 2;
+        const bool read = x >= -GHOST_COLS && x < G.nx + GHOST_COLS && y < G.ny + 2;
+        if constexpr (SAVE) file[i] = read ? state[G.at(p, x, y)] : E(0);
+        else if (read) state[G.at(p, x, y)] = file[i];
+    }
+}
+
+template <bool SAVE>
+cudaError_t launch_file(int esize, const Geometry& g, const FilePlanes& F, void* state, long long e, long long n, void* file,
+                        cudaStream_t s) {
+    const long long b = (n + AUX_NT - 1) / AUX_NT;
+    const unsigned grid = (unsigned)(b < 65536 ? b : 65536);
+    switch (esize) {
+        case 2: k_file<uint16_t, SAVE><<<grid, AUX_NT, 0, s>>>(g, F, static_cast<uint16_t*>(state), e, n, static_cast<uint16_t*>(file)); break;
+        case 4: k_file<uint32_t, SAVE><<<grid, AUX_NT, 0, s>>>(g, F, static_cast<uint32_t*>(state), e, n, static_cast<uint32_t*>(file)); break;
+        case 8: k_file<uint64_t, SAVE><<<grid, AUX_NT, 0, s>>>(g, F, static_cast<uint64_t*>(state), e, n, static_cast<uint64_t*>(file)); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 int aux_blocks(const Geometry& g) {
     const long long n = (long long)g.nx * g.ny;
     long long b = (n + AUX_NT - 1) / AUX_NT;
@@ -432,6 +461,15 @@ struct AuxT {
 }  // namespace
 
 int moments_blocks(const Geometry& g) { return aux_blocks(g); }
+
+cudaError_t launch_state_to_file(int esize, const Geometry& g, const FilePlanes& F, const void* buf, long long e, long long n,
+                                 void* out, cudaStream_t s) {
+    return launch_file<true>(esize, g, F, const_cast<void*>(buf), e, n, out, s);
+}
+cudaError_t launch_file_to_state(int esize, const Geometry& g, const FilePlanes& F, const void* in, long long e, long long n,
+                                 void* buf, cudaStream_t s) {
+    return launch_file<false>(esize, g, F, buf, e, n, const_cast<void*>(in), s);
+}
 
 #define LBM_DISPATCH(storage, call)                                  \
     switch (storage) {                                               \

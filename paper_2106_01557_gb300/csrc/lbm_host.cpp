@@ -8,7 +8,7 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
-#include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -807,67 +807,54 @@ static uint64_t config_hash(const lbm_config& c) {
     return h;
 }
 
-// The file holds the state as 18 planes (f_0 .. f_8, g_0 .. g_8) of node rows
-// -2 .. ny + 1 (and on to `nyp` rows), each row from 128 bytes before its
-// column 0 to a whole number of 128 bytes that takes the 16 bytes of ghost
-// columns beyond the last.
-struct FilePlanes {
-    size_t px, pitch, nyp, plane;
-    explicit FilePlanes(const lbm_handle* h) {
-        const size_t line = 128 / h->esize;
-        const int min_x = h->storage == S_F64 ? 32 : 64, min_y = h->storage == S_F64 || h->storage == S_F32 ? 16 : 32;
-        px = line;
-        pitch = (px + std::max(h->cfg.nx, min_x) + 16 / h->esize + line - 1) / line * line;
-        nyp = std::max(h->cfg.ny, min_y) + 4;
-        plane = pitch * nyp;
-    }
-};
-// stored strips <-> the file's planes, both on the host: the rows and columns
-// that a step reads
-static void copy_planes(const lbm_handle* h, unsigned char* file, unsigned char* state, bool save) {
-    const Geometry& G = h->L.geo;
-    const FilePlanes F(h);
-    const size_t es = h->esize;
-    const int sw = 1 << G.lsw;
-    for (int p = 0; p < 18; ++p)
-        for (int y = -2; y < G.ny + 2; ++y)
-            for (int x = -GHOST_COLS; x < G.nx + GHOST_COLS;) {
-                const int n = std::min(sw - ((x + sw) & (sw - 1)), G.nx + GHOST_COLS - x);  // up to the strip's end
-                unsigned char* a = file + (p * F.plane + (size_t)(y + 2) * F.pitch + F.px + x) * es;
-                unsigned char* b = state + (size_t)G.at(p, x, y) * es;
-                std::memcpy(save ? a : b, save ? b : a, n * es);
-                x += n;
-            }
+static FilePlanes file_planes(const lbm_handle* h) {
+    const size_t es = h->esize, line = 128 / es;
+    const int min_x = h->storage == S_F64 ? 32 : 64, min_y = h->storage == S_F64 || h->storage == S_F32 ? 16 : 32;
+    FilePlanes F;
+    F.px = (int)line;
+    F.pitch = (long long)((line + std::max(h->cfg.nx, min_x) + 16 / es + line - 1) / line * line);
+    F.nyp = std::max(h->cfg.ny, min_y) + 4;
+    return F;
 }
+// the elements of the file that the scratch area takes at a time
+static long long file_chunk(const lbm_handle* h) { return (long long)(h->scratch_elems * sizeof(double) / h->esize); }
 
-int lbm_save(lbm_handle* h, const char* path) {
+int lbm_save(lbm_handle* h, const char* path) try {
     if (!h || !path) return fail(LBM_ERR_ARG, "null argument");
     int rc = check_status(h);
     if (rc) return rc;
-    const size_t bytes = 18 * FilePlanes(h).plane * h->esize;
-    std::vector<unsigned char> host(bytes), state((size_t)h->L.geo.elems() * h->esize);
-    CK(cudaMemcpy(state.data(), h->buf[h->cur], state.size(), cudaMemcpyDeviceToHost));
-    copy_planes(h, host.data(), state.data(), true);
+    const FilePlanes F = file_planes(h);
+    const long long n = F.elems(), part = file_chunk(h);
+    std::vector<unsigned char> host((size_t)n * h->esize);
+    for (long long e = 0; e < n; e += part) {
+        const long long m = std::min(part, n - e);
+        CK(launch_state_to_file((int)h->esize, h->L.geo, F, h->buf[h->cur], e, m, h->scratch, h->stream));
+        CK(cudaMemcpyAsync(host.data() + (size_t)e * h->esize, h->scratch, (size_t)m * h->esize, cudaMemcpyDeviceToHost, h->stream));
+    }
+    CK(cudaStreamSynchronize(h->stream));
     FILE* fp = std::fopen(path, "wb");
     if (!fp) return fail(LBM_ERR_IO, std::string("cannot open ") + path);
     int32_t hdr[4] = {h->cfg.nx, h->cfg.ny, h->cfg.precision, h->cfg.walls};
     const uint64_t ch = config_hash(h->cfg);
     bool ok = std::fwrite(&CK_MAGIC, 8, 1, fp) == 1 && std::fwrite(hdr, sizeof hdr, 1, fp) == 1 &&
               std::fwrite(&ch, 8, 1, fp) == 1 && std::fwrite(&h->steps, 8, 1, fp) == 1 &&
-              std::fwrite(host.data(), 1, bytes, fp) == bytes;
+              std::fwrite(host.data(), 1, host.size(), fp) == host.size();
     ok = (std::fclose(fp) == 0) && ok;
     return ok ? LBM_OK : fail(LBM_ERR_IO, std::string("write failed: ") + path);
+} catch (const std::bad_alloc&) {
+    return fail(LBM_ERR_OOM, "host allocation failed");
 }
 
-int lbm_load(lbm_handle* h, const char* path) {
+int lbm_load(lbm_handle* h, const char* path) try {
     if (!h || !path) return fail(LBM_ERR_ARG, "null argument");
+    const FilePlanes F = file_planes(h);
+    const long long n = F.elems(), part = file_chunk(h);
+    std::vector<unsigned char> host((size_t)n * h->esize);
     FILE* fp = std::fopen(path, "rb");
     if (!fp) return fail(LBM_ERR_IO, std::string("cannot open ") + path);
     uint64_t magic = 0, ch = 0;
     int32_t hdr[4];
     int64_t steps = 0;
-    const size_t bytes = 18 * FilePlanes(h).plane * h->esize;
-    std::vector<unsigned char> host(bytes), state((size_t)h->L.geo.elems() * h->esize);
     bool ok = std::fread(&magic, 8, 1, fp) == 1 && std::fread(hdr, sizeof hdr, 1, fp) == 1 &&
               std::fread(&ch, 8, 1, fp) == 1 && std::fread(&steps, 8, 1, fp) == 1;
     if (ok && (magic != CK_MAGIC || hdr[0] != h->cfg.nx || hdr[1] != h->cfg.ny || hdr[2] != h->cfg.precision ||
@@ -880,19 +867,25 @@ int lbm_load(lbm_handle* h, const char* path) {
         return fail(LBM_ERR_ARG, "checkpoint was written under another configuration (EOS, rates, forces, "
                                  "walls or rounding differ)");
     }
-    ok = ok && std::fread(host.data(), 1, bytes, fp) == bytes;
+    ok = ok && std::fread(host.data(), 1, host.size(), fp) == host.size();
     std::fclose(fp);
     if (!ok) return fail(LBM_ERR_IO, std::string("read failed: ") + path);
-    CK(cudaStreamSynchronize(h->stream));
-    copy_planes(h, host.data(), state.data(), false);
-    CK(cudaMemcpy(h->buf[0], state.data(), state.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemsetAsync(h->buf[0], 0, (size_t)h->L.geo.elems() * h->esize, h->stream));
+    for (long long e = 0; e < n; e += part) {
+        const long long m = std::min(part, n - e);
+        CK(cudaMemcpyAsync(h->scratch, host.data() + (size_t)e * h->esize, (size_t)m * h->esize, cudaMemcpyHostToDevice, h->stream));
+        CK(launch_file_to_state((int)h->esize, h->L.geo, F, h->scratch, e, m, h->buf[0], h->stream));
+    }
     // the device copy of the step count keys the stochastic rounding of
     // 16-bit storage: a resumed run continues with the same dither
     const double st = (double)steps;
     h->cur = 0;
-    CK(cudaMemcpy(h->count(0), &st, sizeof st, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(h->count(0), &st, sizeof st, cudaMemcpyHostToDevice, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
     h->steps = steps;
     return LBM_OK;
+} catch (const std::bad_alloc&) {
+    return fail(LBM_ERR_OOM, "host allocation failed");
 }
 
 int lbm_destroy(lbm_handle* h) {

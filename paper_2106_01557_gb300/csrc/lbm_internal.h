@@ -144,6 +144,22 @@ cudaError_t launch_moments(int storage, const Launch& L, const void* buf, double
                            double* stats, unsigned* counter, cudaStream_t s, bool fast = false);
 int moments_blocks(const Geometry& g);
 
+// A checkpoint file holds the state as 18 planes (f_0 .. f_8, g_0 .. g_8) of node
+// rows -2 .. ny + 1 (and on to `nyp` rows), each row from 128 bytes before its
+// column 0 (px elements) to a whole number of 128 bytes that takes the 16 bytes of
+// ghost columns beyond the last.
+struct FilePlanes {
+    int px, nyp;
+    long long pitch;
+    __host__ __device__ __forceinline__ long long elems() const { return 18 * pitch * nyp; }
+};
+// elements e .. e + n - 1 of the file from the stored state (zero where a step
+// reads nothing), and into it; esize: bytes of a stored value
+cudaError_t launch_state_to_file(int esize, const Geometry& g, const FilePlanes& F, const void* buf, long long e, long long n,
+                                 void* out, cudaStream_t s);
+cudaError_t launch_file_to_state(int esize, const Geometry& g, const FilePlanes& F, const void* in, long long e, long long n,
+                                 void* buf, cudaStream_t s);
+
 // Conservation record of caller-owned [9][ny][nx] FP64 populations with all
 // scratch in a fixed device array (lbm_noalloc.cu); allocates nothing.
 long long noalloc_max_nodes();
