@@ -173,6 +173,7 @@ struct lbm_handle {
     unsigned* counter = nullptr; // 2 counters
     int* status = nullptr;
     int* h_status = nullptr;  // pinned: its copy after a call
+    double* h_stats = nullptr;  // pinned: a copy of stats
     double* scratch = nullptr;   // 9 * 2 * n doubles (populations / fields)
     size_t scratch_elems = 0;
     cudaStream_t stream = nullptr;
@@ -182,6 +183,7 @@ struct lbm_handle {
     MarchGrid grid;        // of the row-marching step
     bool pending = false;  // the last step's record is not combined yet
     static constexpr int GRAPH_STEPS = 20;  // even: the graph returns to buffer 0
+    static constexpr int STATS = 2 * NQ + 2;
     double* count(int b) const { return stats + 2 * NQ + b; }
 };
 
@@ -446,7 +448,7 @@ static void release(lbm_handle* h) {
     if (h->stats) cudaFree(h->stats);
     if (h->counter) cudaFree(h->counter);
     if (h->status) cudaFree(h->status);
-    if (h->h_status) cudaFreeHost(h->h_status);
+    if (h->h_stats) cudaFreeHost(h->h_stats);  // (h_status lies behind it)
     if (h->scratch) cudaFree(h->scratch);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
@@ -483,10 +485,10 @@ int lbm_init(const lbm_config* cfg, lbm_handle** out) {
     h->scratch_elems = 18 * n;
     bool ok = cudaMalloc(&h->buf[0], bytes) == cudaSuccess && cudaMalloc(&h->buf[1], bytes) == cudaSuccess &&
               cudaMalloc(&h->partials, 2 * h->part_stride * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&h->stats, (2 * NQ + 2) * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&h->stats, lbm_handle::STATS * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&h->counter, 2 * sizeof(unsigned)) == cudaSuccess &&
               cudaMalloc(&h->status, sizeof(int)) == cudaSuccess &&
-              cudaMallocHost(&h->h_status, sizeof(int)) == cudaSuccess &&
+              cudaMallocHost(&h->h_stats, (lbm_handle::STATS + 1) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&h->scratch, h->scratch_elems * sizeof(double)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -494,9 +496,10 @@ int lbm_init(const lbm_config* cfg, lbm_handle** out) {
         delete h;
         return fail(LBM_ERR_OOM, "device allocation failed");
     }
+    h->h_status = reinterpret_cast<int*>(h->h_stats + lbm_handle::STATS);
     ok = cudaMemsetAsync(h->buf[0], 0, bytes, h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->buf[1], 0, bytes, h->stream) == cudaSuccess &&
-         cudaMemsetAsync(h->stats, 0, (2 * NQ + 2) * sizeof(double), h->stream) == cudaSuccess &&
+         cudaMemsetAsync(h->stats, 0, lbm_handle::STATS * sizeof(double), h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->partials, 0, 2 * h->part_stride * sizeof(double), h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->counter, 0, 2 * sizeof(unsigned), h->stream) == cudaSuccess &&
          cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) == cudaSuccess &&
@@ -750,11 +753,11 @@ int lbm_conservation(lbm_handle* h, double out[6]) {
 
 int lbm_step_stats(lbm_handle* h, double out[8]) {
     if (!h || !out) return fail(LBM_ERR_ARG, "null argument");
-    double s[NQ];
-    CK(cudaMemcpyAsync(s, h->stats, (NQ - 1) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(s + 7, h->count(h->cur), sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    // the record and both step counts in one copy (two took 4.5 us more)
+    CK(cudaMemcpyAsync(h->h_stats, h->stats, lbm_handle::STATS * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     int rc = check_status(h);
-    for (int k = 0; k < 8; ++k) out[k] = s[k];
+    for (int k = 0; k < 7; ++k) out[k] = h->h_stats[k];
+    out[7] = h->h_stats[2 * NQ + h->cur];
     return rc;
 }
 
