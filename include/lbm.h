@@ -314,8 +314,9 @@ int lbm_batch_set_tile_wait(lbm_batch* b, int64_t ns);
 /* Autotuner: times every candidate (work split x work-list order) for
  * trial_steps steps on the current state and keeps the fastest; the trial
  * steps are real steps of every case (the state advances). choice[0] =
- * work split index (0 an equal run of rows per warp, 1 items of 32 rows), choice[1] = order index (0 case-major, 1 largest case
- * first, 2 round-robin over cases); ms[k] (may be NULL, >= 6 entries) =
+ * work split index (0 an equal run of rows per warp, 1 items of at most 32
+ * rows), choice[1] = order index (0 case-major, 1 largest case first, 2
+ * round-robin over cases); ms[k] (may be NULL, >= 6 entries) =
  * the time per step of candidate k = 3 * shape + order. Synchronous. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, int32_t choice[2], double* ms);
 /* Select a candidate directly (work split, order). */

@@ -1024,7 +1024,7 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
     // Work lists: strips of the cases in one of three orders (case after case,
     // the largest case first, or strip 0 of every case, then strip 1, ...),
     // their rows dealt to the warps of one wave. Shape 0: every warp an equal
-    // run of rows. Shape 1: items of at most 32 rows in turn.
+    // run of rows. Shape 1: items of at most 32 rows (batch_item_rows) in turn.
     // The strips of a case read each other's edge columns, so in the first two
     // orders they are cut at the same rows and given to neighbouring warps,
     // which find these columns in L1 and L2: for shape 0 the cases with s
@@ -1046,12 +1046,13 @@ int lbm_batch_init(const lbm_config* cfgs, int32_t ncases, lbm_batch** out) {
         rows += (long long)strips_of(i) * cfgs[i].ny;
     }
     b->warps = (int)std::min<long long>(batch_warps(b->storage, b->sms), rows);
+    const int item_rows = batch_item_rows(rows, b->warps);
     for (int o = 0; o < 3; ++o) {
         std::vector<std::vector<BatchItem>> even(b->warps), dealt(b->warps);
-        std::vector<BatchItem> rest, cut;  // items left for single warps; items of at most 32 rows
+        std::vector<BatchItem> rest, cut;  // items left for single warps; items of at most item_rows rows
         int w = 0;                         // warps that have their rows
         auto pieces = [&](int i, int s0, int s1) {
-            const int ny = cfgs[i].ny, n = (ny + 31) / 32;
+            const int ny = cfgs[i].ny, n = (ny + item_rows - 1) / item_rows;
             for (int j = 0; j < n; ++j)
                 for (int s = s0; s < s1; ++s)
                     cut.push_back({i, s * sw, (int)((long long)ny * j / n), (int)((long long)ny * (j + 1) / n)});
