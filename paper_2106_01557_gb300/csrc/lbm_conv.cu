@@ -367,16 +367,23 @@ __global__ void __launch_bounds__(128) k_bgrad(const __nv_bfloat16* __restrict__
     const long long rows = (long long)N * H * tiles_x;
     const long long r_end = rows * (blockIdx.x + 1) / gridDim.x;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    // A row's loads are issued before any is used, two rows at a time: one after
+    // another they cost the gradients of 8 x 256 x 256 0.6 ms of 8.3.
+#pragma unroll 2
     for (long long r = rows * blockIdx.x / gridDim.x; r < r_end; ++r) {
         const long long strip = r / H;
         const int x0 = (int)(strip % tiles_x) * WCH;
         const __nv_bfloat16* row = dout + ((strip / tiles_x * H + r % H) * W + x0) * C + c8 * 8;
+        uint4 v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int px = sub + 16 * i;
-            if (x0 + px >= W || c8 * 8 >= C) break;
-            const uint4 v = *reinterpret_cast<const uint4*>(row + (size_t)px * C);
-            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v);
+            v[i] = make_uint4(0, 0, 0, 0);
+            if (x0 + px < W && c8 * 8 < C) v[i] = *reinterpret_cast<const uint4*>(row + (size_t)px * C);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v[i]);
 #pragma unroll
             for (int c = 0; c < 8; ++c) acc[c] += __bfloat162float(h[c]);
         }
