@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(C6_THREADS, 1)
                 if (!role_wait_warp(&acc_full[tt % C6_BLK], (tt / C6_BLK) & 1u, dead)) break;
                 tc_fence_after();
                 float v[16];
-                tc_ld<16>(t_lane + (tt % C6_BLK) * 16u, v);
+                tc_ld16(t_lane + (tt % C6_BLK) * 16u, v);
                 tc_st_zero16(t_lane + (tt % C6_BLK) * 16u);
                 tc_wait_st();
                 tc_fence_before();
