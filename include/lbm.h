@@ -256,13 +256,13 @@ int64_t lbm_step_count(const lbm_handle* h);
 #define LBM_TILE_WAIT_DEFAULT_NS 2000000000LL
 
 /* Bound, in nanoseconds, on the time a warp of the step kernel waits for the
- * loads of its first rows (later rows load while earlier ones are computed;
- * failure detection, not a parameter of the paper's method). A warp whose
- * wait was longer stores nothing and sets the handle's status, and the next
- * synchronising call returns LBM_ERR_TIMEOUT; the state is then undefined
- * until the next lbm_set_fields, lbm_set_populations or lbm_load. 0 means no
- * waiting, which every warp runs out of. ns < 0: LBM_ERR_ARG. Takes effect
- * from the next lbm_step. */
+ * loads of its first rows (later rows load while earlier ones are computed
+ * and are not timed; failure detection, not a parameter of the paper's
+ * method). A warp whose wait was longer stores nothing and sets the handle's
+ * status, and the next synchronising call returns LBM_ERR_TIMEOUT; the state
+ * is then undefined until the next lbm_set_fields, lbm_set_populations or
+ * lbm_load. 0 means no waiting, which every warp runs out of. ns < 0:
+ * LBM_ERR_ARG. Takes effect from the next lbm_step. */
 int lbm_set_tile_wait(lbm_handle* h, int64_t ns);
 
 /* Bytes of population traffic one time step moves at the algorithmic
@@ -279,9 +279,11 @@ int lbm_destroy(lbm_handle* h);
  * batch gives the same populations as that case on its own handle with the
  * same precision, up to floating-point rounding (the two kernels are
  * compiled separately). With 16-bit storage the batch rounds its stores
- * as lbm_config.rounding says, stochastically by default, with the dither
- * of a single handle keyed by (node, batch step count), which the device
- * keeps. Extension of the paper's method for parameter sweeps (the paper
+ * as lbm_config.rounding says, stochastically by default, keyed by (node,
+ * batch step count), which the device keeps; the bits it draws are not those
+ * of a single handle (which takes a seed per pair of nodes, a batch, open
+ * sides and the cubic-term elimination one per node), so with rounding = 1
+ * the two agree statistically only. Extension of the paper's method for parameter sweeps (the paper
  * runs single cases). Requirements: every cfgs[i] periodic (walls = 0, no
  * open sides), one precision for all (LBM_F32, LBM_F16S or LBM_BF16S), one
  * rounding for all; the stream and device of cfgs[0] are used. */
@@ -299,7 +301,7 @@ int lbm_batch_moments(lbm_batch* b, int32_t i, double* rho, double* ux, double* 
 int lbm_batch_conservation(lbm_batch* b, int32_t i, double out[6]);
 int lbm_batch_get_populations(lbm_batch* b, int32_t i, double* f, double* g);
 /* Case i's conservation record as reduced inside the most recent step
- * (FP32 partial sums per work item, summed per case in FP64): layout of
+ * (FP32 sums over 16 rows of a strip, FP64 from there): layout of
  * lbm_step_stats out[0..6]; out[7] = the steps the batch has executed, as
  * counted on the device (the count that keys stochastic rounding).
  * Synchronous. */

@@ -69,7 +69,7 @@ struct Geometry {
     }
     __host__ __device__ __forceinline__ long long elems() const { return ((long long)strips * nyp * ROW_LINES) << lsw; }
     int hot_x0, hot_len;
-    int sms;         // persistent grid size (one CTA per SM)
+    int sms;         // multiprocessors of the device: a step's grid is one wave of resident blocks
     int open;        // open sides: 1 bottom, 2 top, 4 left, 8 right (left and right only together with all)
 };
 

@@ -26,10 +26,10 @@
 //
 // Measured on 4096 x 1024 with walls (us per step; before, the step staged
 // 64-wide tiles of all 18 planes in shared memory by tensor copies, with a
-// density pass and a block barrier per tile): FP32 115.0 -> 105.3 (5.74 TB/s;
-// what is left is mostly the memory mix: without the collision it takes 104.6),
-// FP16 107.5 -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with
-// launches that overlap (lbm_launch.cuh) and the later changes 103.6 and 79.6.
+// density pass and a block barrier per tile): FP32 115.0 -> 105.3 (a copy without
+// the collision took 104.6 then: what is left is mostly the memory mix), FP16 107.5
+// -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with launches that
+// overlap (lbm_launch.cuh) and the later changes 103.4 (5.84 TB/s) and 79.5.
 // Tried for the rows: a ring of tensor-copied boxes per warp (124, whatever the
 // depth: about 10 cycles of the copy engine per line of 128 bytes), 16-byte
 // asynchronous copies into a shared-memory ring (124: bound by the shared-

@@ -1,9 +1,10 @@
 // Host runtime of the learned surrogate: parameters (FP32 master copies,
 // Adam moments, BF16 forward and flipped copies), activation buffers, the
 // forward and backward passes built from the BF16 tensor-core kernels of
-// lbm_conv_tc.cu (tcgen05: convolutions, 64 -> 64 weight gradients) or
-// lbm_conv.cu (mma.sync; the other weight gradients and the elementwise
-// kernels), and the rollout with LB fallback.
+// lbm_conv_tc.cu (tcgen05: convolutions and input gradients) and lbm_wgrad64.cu
+// (tcgen05: weight and bias gradients) or of lbm_conv.cu (conv_path 1: the same on
+// mma.sync; and the elementwise kernels of both), and the rollout with LB
+// fallback.
 #include <cuda_runtime.h>
 
 #include <algorithm>
