@@ -11,7 +11,7 @@ from gpu_common import oracle_case, slab_fields
 pytestmark = pytest.mark.gpu
 
 EX, EY = (0, 1, 0, -1, 0, 1, -1, -1, 1), (0, 0, 1, 0, -1, 1, 1, -1, -1)
-WALLS = dict(walls=1, accel_y=-1e-5, Tr_bottom=0.8, Tr_hot=0.95, hot_x0=3, hot_len=9)
+WALLS = dict(walls=1, accel_y=-1e-5, Tr_bottom=0.8, Tr_hot=0.95, hot_x0=3, hot_len=5)
 BITS = {"f16s": 11, "bf16s": 8}  # of the significand
 
 
@@ -48,3 +48,24 @@ def test_reflections_are_rounded_once(gpu_lib, tmp_path, nx, ny, opts, prec):
                 half = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(stored), 2.0**-14))) - BITS[prec])
                 err = np.abs(value - exact[i, y])
                 assert (err <= half + 1e-5 * np.abs(exact).max()).all(), (d, i, y, (err / half).max())
+
+
+STEPS = 7
+
+
+@pytest.mark.parametrize("prec", ["f16s", "bf16s"])
+@pytest.mark.parametrize("nx,ny", [(8, 8), (31, 9), (65, 11), (129, 8)])
+def test_walled_steps_match_oracle(gpu_lib, nx, ny, prec):
+    # stochastic rounding moves a value by less than one step of the format (2^-10 or
+    # 2^-7 of its size), once per step: after n steps by at most n times that of the
+    # largest population
+    from paper_2106_01557_gb300 import lbm
+    o = oracle_case(nx, ny, **WALLS)
+    lat = lbm.Lattice.create(nx, ny, precision=prec, **WALLS)
+    fields = slab_fields(o, seed=31, eps=0.01, uamp=0.005)
+    o.init_fields(*fields)
+    lat.set_fields(*fields)
+    o.step(STEPS)
+    lat.step(STEPS)
+    for got, want in zip(lat.get_populations(), (o.f, o.g)):
+        assert np.abs(got - want).max() < STEPS * 2.0 ** (1 - BITS[prec]) * np.abs(want).max()
