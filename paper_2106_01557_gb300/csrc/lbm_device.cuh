@@ -138,13 +138,19 @@ __device__ __forceinline__ void rest_as_complement(C m0, C l[9]) {
 }
 
 // l = M^-1 m = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4) m,
-// the weights folded into fused multiply-adds (28 operations)
+// the weights folded into fused multiply-adds (30 operations), but for m_1 and
+// m_2: their products are rounded once and shared by the populations of a column,
+// over which they cancel. Folded too (28 operations, 1% of a step that is bound by
+// its arithmetic) they left a bias in the sums m_0 and n_0 of every node: mass after
+// 100,000 boiling steps on 4096 x 1024 in FP32 -1.1e-4 instead of +1.7e-5, in FP16
+// -4.3e-4 instead of -7e-5, and over 120,000 of a slab in FP64 -5.2e-13 instead of
+// -1.5e-13.
 template <class C>
 __device__ __forceinline__ void populations9(const C m[9], C l[9]) {
-    const C a0 = ninth(m[0]);
-    const C axis = a0 - m[1] * C(1.0 / 36.0) - m[2] * C(1.0 / 18.0);
-    const C diag = a0 + m[1] * C(1.0 / 18.0) + m[2] * C(1.0 / 36.0);
-    l[0] = a0 - m[1] * C(1.0 / 9.0) + m[2] * C(1.0 / 9.0);
+    const C a0 = ninth(m[0]), a1 = m[1] * C(1.0 / 36.0), a2 = m[2] * C(1.0 / 36.0);
+    const C axis = a0 - a1 - C(2) * a2;
+    const C diag = a0 + C(2) * a1 + a2;
+    l[0] = a0 - C(4) * a1 + C(4) * a2;
     const C bx = m[3] * C(1.0 / 6.0), by = m[5] * C(1.0 / 6.0);
     const C px = bx - m[4] * C(1.0 / 6.0), py = by - m[6] * C(1.0 / 6.0);
     const C qx = bx + m[4] * C(1.0 / 12.0), qy = by + m[6] * C(1.0 / 12.0);
