@@ -485,7 +485,7 @@ __device__ __forceinline__ void put(S* __restrict__ out, const Geometry& G, int 
 // are transformed, once per DF; the strip along an open side calls this on
 // every row, which bounds the step of a small lattice (512 x 512 open on all
 // sides, FP32: 26 us with four back-transforms and a search over all ghosts
-// and directions, 12.5 so, against 10.9 periodic then; 11.2 and 9.3 now).
+// and directions, 12.5 so, against 10.9 periodic then; 11.4 and 9.4 now).
 // (f and g come as the nine values each so that the caller's arrays stay in
 // registers on the path that does not call this.)
 template <class C>

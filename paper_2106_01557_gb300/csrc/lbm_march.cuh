@@ -29,7 +29,7 @@
 // density pass and a block barrier per tile): FP32 115.0 -> 105.3 (a copy without
 // the collision took 104.6 then: what is left is mostly the memory mix), FP16 107.5
 // -> 85.9 (bound by the packed arithmetic of 12 warps per SM); with launches that
-// overlap (lbm_launch.cuh) and the later changes 103.4 (5.84 TB/s) and 79.5.
+// overlap (lbm_launch.cuh) and the later changes 103.4 (5.84 TB/s) and 80.4.
 // Tried for the rows: a ring of tensor-copied boxes per warp (124, whatever the
 // depth: about 10 cycles of the copy engine per line of 128 bytes), 16-byte
 // asynchronous copies into a shared-memory ring (124: bound by the shared-
@@ -327,7 +327,7 @@ __device__ __forceinline__ bool march_rows(const KC<C>& k, const K& kv, const Ge
             else dm = dc;  // beyond a wall: the adjacent node's density
         }
         // (later rows are not timed: with a timer read per row the step of a 4096 x
-        // 1024 lattice in FP16 went from 79.5 to 82.7 us, of a 128 x 128 one in FP32
+        // 1024 lattice in FP16 went from 79.5 to 82.7 us then, of a 128 x 128 one in FP32
         // from 3.93 to 4.03, and a load cannot be given up)
         C last;
         if constexpr (NPL == 2) last = dc.r.v.x;
